@@ -1,11 +1,14 @@
-"""ctypes binding of ``include/nuna.h``: same names, argument marshalling only.
+"""Binding of ``include/nuna.h``: same names, argument marshalling only.
 
 Rank buffers are passed as sequences of torch CUDA tensors (or raw device
 addresses); every step of every collective runs in the library's CUDA kernels.
+The collectives' arguments are marshalled by a small native module
+(``csrc/python/nuna_py.cpp``), everything else by ctypes.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Sequence
 
@@ -89,6 +92,7 @@ class NunaPlanInput(ctypes.Structure):
 
 
 _LIB_PATH = os.environ.get("NUNA_LIB") or os.path.join(os.path.dirname(os.path.abspath(__file__)), "libnuna.so")
+_NATIVE_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_nuna_py.so")
 _lib = None
 
 
@@ -179,25 +183,56 @@ def ptr_table(bufs: Sequence):
     return tab
 
 
+# The collectives the native module calls, in its order.
+_COLLECTIVES = ("nuna_allreduce", "nuna_allreduce_oneshot", "nuna_allreduce_twoshot", "nuna_reduce_scatter", "nuna_allgather",
+                "nuna_alltoall")
+_ALLREDUCE, _ONESHOT, _TWOSHOT, _REDUCE_SCATTER, _ALLGATHER, _ALLTOALL = range(6)
+
+
+def _load_native():
+    """Loads the marshalling module and points it at the library; the module's functions replace the loaders below."""
+    global _collective, _twoshot_static, _host, _stream_handle
+    L = lib()
+    if not os.path.exists(_NATIVE_PATH):
+        raise RuntimeError(f"{_NATIVE_PATH} is missing: run `python -m paper_2608_00867_b200.build`")
+    import torch  # noqa: F401  (the module links against torch's libraries, which importing torch loads)
+    spec = importlib.util.spec_from_file_location(__package__ + "._nuna_py", _NATIVE_PATH)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    at = lambda name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value
+    m.bind(tuple(at(n) for n in _COLLECTIVES), at("nuna_allreduce_twoshot_static"), at("nuna_allreduce_host"), NunaError)
+    _collective, _twoshot_static, _host, _stream_handle = m.collective, m.twoshot_static, m.host, m.stream_handle
+
+
+# (index, src, dst, count, dtype, flags, stream, check, nranks) -> status; likewise the others
+def _collective(*args):
+    _load_native()
+    return _collective(*args)
+
+
+def _twoshot_static(*args):
+    _load_native()
+    return _twoshot_static(*args)
+
+
+def _host(*args):
+    _load_native()
+    return _host(*args)
+
+
+def _stream_handle(stream):
+    _load_native()
+    return _stream_handle(stream)
+
+
 def _stream(stream) -> Optional[int]:
-    if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
-    if hasattr(stream, "cuda_stream"):
-        return stream.cuda_stream or None
-    return int(stream) or None
+    return _stream_handle(stream) or None
 
 
 def _finish(status: int, what: str, check: bool) -> int:
     if check and status != NUNA_OK:
         raise NunaError(status, what)
     return status
-
-
-def _collective(name, src, dst, count, dtype, flags, stream, check, nranks=None):
-    n = len(src) if nranks is None else nranks
-    st = getattr(lib(), name)(ptr_table(src), ptr_table(dst), n, count, dtype, flags, _stream(stream))
-    return _finish(st, name, check)
 
 
 def nuna_init(scratch_bytes: int = 0, check: bool = True) -> int:
@@ -209,27 +244,27 @@ def nuna_set_option(option: int, value: int, check: bool = True) -> int:
 
 
 def nuna_allreduce_oneshot(src, dst, count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective("nuna_allreduce_oneshot", src, dst, count, dtype, flags, stream, check, nranks)
+    return _collective(_ONESHOT, src, dst, count, dtype, flags, stream, check, nranks)
 
 
 def nuna_allreduce(src, dst, count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective("nuna_allreduce", src, dst, count, dtype, flags, stream, check, nranks)
+    return _collective(_ALLREDUCE, src, dst, count, dtype, flags, stream, check, nranks)
 
 
 def nuna_allreduce_twoshot(src, dst, count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective("nuna_allreduce_twoshot", src, dst, count, dtype, flags, stream, check, nranks)
+    return _collective(_TWOSHOT, src, dst, count, dtype, flags, stream, check, nranks)
 
 
 def nuna_reduce_scatter(src, dst, shard_count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective("nuna_reduce_scatter", src, dst, shard_count, dtype, flags, stream, check, nranks)
+    return _collective(_REDUCE_SCATTER, src, dst, shard_count, dtype, flags, stream, check, nranks)
 
 
 def nuna_allgather(src, dst, shard_count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective("nuna_allgather", src, dst, shard_count, dtype, flags, stream, check, nranks)
+    return _collective(_ALLGATHER, src, dst, shard_count, dtype, flags, stream, check, nranks)
 
 
 def nuna_alltoall(src, dst, block_count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective("nuna_alltoall", src, dst, block_count, dtype, flags, stream, check, nranks)
+    return _collective(_ALLTOALL, src, dst, block_count, dtype, flags, stream, check, nranks)
 
 
 NUNA_STATIC_MAX_COUNT = 2 * 1024 * 1024
@@ -238,20 +273,12 @@ NUNA_STATIC_MAX_COUNT = 2 * 1024 * 1024
 def nuna_allreduce_twoshot_static(src, dst, count, dtype=NUNA_BF16, stream=None, check=True) -> int:
     """The two-shot allreduce that never allocates: its scratch is a fixed array inside the library
     (at most NUNA_STATIC_MAX_COUNT elements per rank).  For callers that cannot call cudaMalloc."""
-    st = lib().nuna_allreduce_twoshot_static(ptr_table(src), ptr_table(dst), len(src), count, dtype, _stream(stream))
-    return _finish(st, "nuna_allreduce_twoshot_static", check)
+    return _twoshot_static(src, dst, count, dtype, stream, check)
 
 
 def nuna_allreduce_host(src, dst, count, dtype=NUNA_BF16, flags=0, two_shot=False, check=True) -> int:
     """``src`` / ``dst``: host buffers (numpy arrays, CPU tensors or addresses)."""
-    def haddr(x):
-        if hasattr(x, "ctypes"):
-            return x.ctypes.data
-        return _addr(x)
-    s = (ctypes.c_void_p * len(src))(*[haddr(x) for x in src])
-    d = (ctypes.c_void_p * len(dst))(*[haddr(x) for x in dst])
-    st = lib().nuna_allreduce_host(s, d, len(src), count, dtype, flags, 1 if two_shot else 0)
-    return _finish(st, "nuna_allreduce_host", check)
+    return _host(src, dst, count, dtype, flags, two_shot, check)
 
 
 def nuna_chain_create(src_sets, dst_sets, nnodes, count, dtype=NUNA_BF16, flags=0, two_shot=False, check=True):

@@ -1,14 +1,19 @@
-"""Builds ``libnuna.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds ``libnuna.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU) and, with the host compiler,
+``_nuna_py.so``, the native half of the Python binding."""
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnuna.so")
+NATIVE_SRC = os.path.join(CSRC, "python", "nuna_py.cpp")
+NATIVE = os.path.join(HERE, "_nuna_py.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -24,28 +29,49 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cpp")))
 
 
+def _older(target, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
+def _public_headers():
+    return glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) \
-        + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    return _older(LIB, sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + _public_headers())
+
+
+def _compile(cmd, target: str, verbose: bool) -> None:
+    tmp = target + f".tmp{os.getpid()}"
+    proc = subprocess.run(cmd + ["-o", tmp], capture_output=True, text=True)
+    if proc.returncode != 0:
+        sys.stderr.write(proc.stdout + proc.stderr)
+        raise RuntimeError(f"{cmd[0]} failed building {os.path.basename(target)}")
+    if verbose:
+        sys.stderr.write(proc.stderr)
+    os.replace(tmp, target)
+
+
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    """The marshalling module: reads addresses and the current stream out of torch's own objects."""
+    if not force and not _older(NATIVE, [NATIVE_SRC] + _public_headers()):
+        return NATIVE
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    inc = os.path.join(torch_dir, "include")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-Wall", "-shared", "-I" + sysconfig.get_paths()["include"]]
+    for d in (inc, os.path.join(inc, "torch", "csrc", "api", "include"), os.path.join(cuda, "include")):
+        cmd += ["-isystem", d]
+    cmd += [NATIVE_SRC, "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda"]
+    _compile(cmd, NATIVE, verbose)
+    return NATIVE
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_native(force, verbose)
     if not force and not is_stale():
         return LIB
-    nvcc = os.environ.get("NVCC", "nvcc")
-    tmp = LIB + f".tmp{os.getpid()}"
-    cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources()
-    proc = subprocess.run(cmd, capture_output=True, text=True)
-    if proc.returncode != 0:
-        sys.stderr.write(proc.stdout + proc.stderr)
-        raise RuntimeError("nvcc failed building libnuna.so")
-    if verbose:
-        sys.stderr.write(proc.stderr)
-    os.replace(tmp, LIB)
+    _compile([os.environ.get("NVCC", "nvcc")] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + sources(), LIB, verbose)
     return LIB
 
 
