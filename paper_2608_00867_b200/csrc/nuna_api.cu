@@ -195,15 +195,31 @@ static unsigned pick_grid(const Context* c, const Options& o, size_t nitems, int
     return (unsigned)std::max<size_t>(1, std::min(nitems, cap));
 }
 
-constexpr unsigned kLaunchPlain = 0u, kLaunchCooperative = 1u, kLaunchPdl = 2u;
+constexpr unsigned kLaunchPlain = 0u, kLaunchCooperative = 1u, kLaunchPdl = 2u, kLaunchOrdered = 4u;
 
-// Programmatic dependent launch pays off while a kernel is short enough for its launch latency to
-// matter.  For the one-shot it was measured to cost a few percent from about 16 MiB of sources (its
-// multi-wave grid competes with the successor's early blocks), so it is dropped there; the streaming
-// kernels (two-shot put, reduce-scatter, allgather) keep it at every size (4 MiB per rank: 12.6 -> 12.0 us).
+// kLaunchPdl: programmatic dependent launch.  kLaunchOrdered: the caller did not ask for one, but the kernel waits for
+// its predecessor before its first global access all the same (pdl_wait), so it may be launched either way with the same
+// result; launched into a stream directly it gets the programmatic attribute too.  A run of plain launches that the host
+// issues faster than the device drains costs a fixed 2.05 us step per kernel on B200: short kernels came out at 4.10 us
+// each whatever their work, longer ones rounded up to the next multiple of 2.05 us (a kernel of 3.8 us as a graph node took
+// 6.15, one of 16.0 took 18.4).  Behind a programmatic launch there is no such step, and the host call is 0.4 us cheaper.
+// While a stream is captured the caller's choice stands: the graph has the edges it asked for.
+// Programmatic launches pay off while a kernel is short enough for its launch latency to matter.  For the one-shot one
+// was measured to cost a few percent from about 16 MiB of sources (its multi-wave grid competes with the successor's
+// early blocks), so it is dropped there; the streaming kernels (two-shot put, reduce-scatter, allgather) keep it at
+// every size (4 MiB per rank: 12.6 -> 12.0 us).
 static unsigned launch_mode(unsigned flags, size_t total_src_bytes = 0)
 {
-    return ((flags & NUNA_LAUNCH_PDL) && total_src_bytes <= ((size_t)16 << 20)) ? kLaunchPdl : kLaunchPlain;
+    if (total_src_bytes > ((size_t)16 << 20)) return kLaunchPlain;
+    return (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchOrdered;
+}
+
+// The legacy default stream cannot be captured, and must not be asked about while another stream is.
+static bool capturing(cudaStream_t stream)
+{
+    if (stream == nullptr || stream == cudaStreamLegacy) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
 }
 
 static thread_local unsigned t_cluster_dim = 0;           // > 0: next launch() uses clusters of this many blocks
@@ -232,7 +248,7 @@ static int launch(void (*kernel)(Args...), unsigned grid, cudaStream_t stream, u
         attr[nattr].id = cudaLaunchAttributeCooperative;
         attr[nattr].val.cooperative = 1;
         ++nattr;
-    } else if (mode & kLaunchPdl) {
+    } else if ((mode & kLaunchPdl) || ((mode & kLaunchOrdered) && !capturing(stream))) {
         attr[nattr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[nattr].val.programmaticStreamSerializationAllowed = 1;
         ++nattr;
@@ -590,7 +606,7 @@ int launch_oneshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t 
         which = (flags & NUNA_PLACE_REGS) ? OneShotKernel::Regs : (flags & NUNA_PLACE_STAGED) ? OneShotKernel::Staged : OneShotKernel::Group;
     else if (place == NUNA_PLACE_AUTO) which = auto_kernel(c, o, nranks, bytes, flags);
     if (which == OneShotKernel::Regs) {
-        const unsigned m = (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchPlain;
+        const unsigned m = launch_mode(flags);
         // destinations per thread: all of them, so that a tile crosses the L2 -> SM fabric once (beyond 8 ranks the
         // sixteen-destination form: 9 ranks x 512 KiB 2.25 us against 2.71 in two passes of eight, 16 ranks x 1 MiB
         // 6.39 against 7.35); half of them for large cold messages, where two blocks per tile keep more DRAM loads
@@ -612,7 +628,7 @@ int launch_oneshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t 
     if (which == OneShotKernel::Staged) {
         return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
             constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
-            return launch_stage<N, DT>(c, o, p, count, flags, (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchPlain, stream);
+            return launch_stage<N, DT>(c, o, p, count, flags, launch_mode(flags), stream);
         });
     }
     if (which == OneShotKernel::Group) {
@@ -687,10 +703,11 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
     return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
         constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
         t_dyn_smem = (unsigned)N * tv * 16u;
+        const unsigned mode = pdl ? kLaunchPdl : kLaunchOrdered;
         if (bytes * (size_t)nranks >= ((size_t)64 << 20))           // bandwidth-bound: trade registers for resident blocks
-            return launch(k_twoshot_flags<N, DT, 6>, grid, stream, pdl ? kLaunchPdl : kLaunchPlain, p, scratch, tile_flags, count,
+            return launch(k_twoshot_flags<N, DT, 6>, grid, stream, mode, p, scratch, tile_flags, count,
                           tv, lead_max, bw, timeout_ns, debug_bits);
-        return launch(k_twoshot_flags<N, DT, 4>, grid, stream, pdl ? kLaunchPdl : kLaunchPlain, p, scratch, tile_flags, count, tv,
+        return launch(k_twoshot_flags<N, DT, 4>, grid, stream, mode, p, scratch, tile_flags, count, tv,
                       lead_max, bw, timeout_ns, debug_bits);
     });
 }
