@@ -195,31 +195,34 @@ static unsigned pick_grid(const Context* c, const Options& o, size_t nitems, int
     return (unsigned)std::max<size_t>(1, std::min(nitems, cap));
 }
 
-constexpr unsigned kLaunchPlain = 0u, kLaunchCooperative = 1u, kLaunchPdl = 2u, kLaunchOrdered = 4u;
+constexpr unsigned kLaunchPlain = 0u, kLaunchCooperative = 1u, kLaunchPdl = 2u;
 
-// kLaunchPdl: programmatic dependent launch.  kLaunchOrdered: the caller did not ask for one, but the kernel waits for
-// its predecessor before its first global access all the same (pdl_wait), so it may be launched either way with the same
-// result; launched into a stream directly it gets the programmatic attribute too.  A run of plain launches that the host
-// issues faster than the device drains costs a fixed 2.05 us step per kernel on B200: short kernels came out at 4.10 us
-// each whatever their work, longer ones rounded up to the next multiple of 2.05 us (a kernel of 3.8 us as a graph node took
-// 6.15, one of 16.0 took 18.4).  Behind a programmatic launch there is no such step, and the host call is 0.4 us cheaper.
-// While a stream is captured the caller's choice stands: the graph has the edges it asked for.
-// Programmatic launches pay off while a kernel is short enough for its launch latency to matter.  For the one-shot one
-// was measured to cost a few percent from about 16 MiB of sources (its multi-wave grid competes with the successor's
-// early blocks), so it is dropped there; the streaming kernels (two-shot put, reduce-scatter, allgather) keep it at
-// every size (4 MiB per rank: 12.6 -> 12.0 us).
+// Programmatic dependent launch pays off while a kernel is short enough for its launch latency to
+// matter.  For the one-shot it was measured to cost a few percent from about 16 MiB of sources (its
+// multi-wave grid competes with the successor's early blocks), so it is dropped there; the streaming
+// kernels (two-shot put, reduce-scatter, allgather) keep it at every size (4 MiB per rank: 12.6 -> 12.0 us).
 static unsigned launch_mode(unsigned flags, size_t total_src_bytes = 0)
 {
-    if (total_src_bytes > ((size_t)16 << 20)) return kLaunchPlain;
-    return (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchOrdered;
+    return ((flags & NUNA_LAUNCH_PDL) && total_src_bytes <= ((size_t)16 << 20)) ? kLaunchPdl : kLaunchPlain;
 }
 
-// The legacy default stream cannot be captured, and must not be asked about while another stream is.
-static bool capturing(cudaStream_t stream)
+// The flags a collective runs with.  Every collective kernel waits for its predecessor before its first global access
+// (pdl_wait), so it may be launched with or without the programmatic attribute with the same result, and a call that
+// goes into a stream directly gets it without asking.  A run of plain launches that the host issues faster than the
+// device drains costs a fixed 2.05 us step per kernel on B200: short kernels came out at 4.10 us each whatever their
+// work, longer ones rounded up to the next multiple of 2.05 us (a kernel of 3.8 us as a graph node took 6.15, one of
+// 16.0 took 18.4).  Behind a programmatic launch there is no such step, the host call is 0.4 us cheaper, and the
+// prefetch ahead of the wait pays as it does with the flag (8 x 4 MiB flag two-shot: 15.6 -> 14.2 us).  While a stream
+// is captured the caller's choice stands: the graph has the edges it asked for.  (The legacy default stream cannot be
+// captured, and must not be asked about while another stream is.)
+static unsigned effective_flags(unsigned flags, void* stream)
 {
-    if (stream == nullptr || stream == cudaStreamLegacy) return false;
+    if (flags & NUNA_LAUNCH_PDL) return flags;
+    const cudaStream_t s = (cudaStream_t)stream;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    if (s != nullptr && s != cudaStreamLegacy && (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone))
+        return flags;
+    return flags | NUNA_LAUNCH_PDL;
 }
 
 static thread_local unsigned t_cluster_dim = 0;           // > 0: next launch() uses clusters of this many blocks
@@ -248,7 +251,7 @@ static int launch(void (*kernel)(Args...), unsigned grid, cudaStream_t stream, u
         attr[nattr].id = cudaLaunchAttributeCooperative;
         attr[nattr].val.cooperative = 1;
         ++nattr;
-    } else if ((mode & kLaunchPdl) || ((mode & kLaunchOrdered) && !capturing(stream))) {
+    } else if (mode & kLaunchPdl) {
         attr[nattr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[nattr].val.programmaticStreamSerializationAllowed = 1;
         ++nattr;
@@ -703,7 +706,7 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
     return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
         constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
         t_dyn_smem = (unsigned)N * tv * 16u;
-        const unsigned mode = pdl ? kLaunchPdl : kLaunchOrdered;
+        const unsigned mode = pdl ? kLaunchPdl : kLaunchPlain;
         if (bytes * (size_t)nranks >= ((size_t)64 << 20))           // bandwidth-bound: trade registers for resident blocks
             return launch(k_twoshot_flags<N, DT, 6>, grid, stream, mode, p, scratch, tile_flags, count,
                           tv, lead_max, bw, timeout_ns, debug_bits);
@@ -765,10 +768,11 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
     const size_t epv = elems_per_vec(dtype);
     const unsigned mode = launch_mode(flags);
     if (shard % epv) {
-        const unsigned grid = pick_grid(c, o, ceil_div(shard * nranks, kThreads), 8);
+        const size_t tiles = std::max<size_t>(1, ceil_div(shard / epv, (size_t)kRaggedTile));
         return dispatch(nranks, 1, dtype, [&](auto n_, auto u_, auto d_) -> int {
             NUNA_NUD(n_, u_, d_);
-            return launch(k_reduce_scatter_scalar<N, DT>, grid, stream, mode, p, shard);
+            auto k = k_reduce_scatter_ragged<N, DT>;
+            return launch(k, pick_grid(c, o, (tiles + 1) * N, NUNA_OCC(k), 0), stream, mode, p, shard, tiles);
         });
     }
     const size_t shard_vec = shard / epv;
@@ -781,28 +785,30 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
     });
 }
 
-// Allgather and alltoall copy bits: they work on 16-byte vectors when a shard is a whole number of
-// them, otherwise on 16-bit units (every element type is a multiple of that).
+// Allgather and alltoall copy bits: they work on 16-byte vectors, shifted to the destination's alignment when a shard is
+// no whole number of them; what is left at the ends goes in 16-bit units (every element type is a multiple of that).
 int launch_allgather(Context* c, const RankPtrs& p, int nranks, size_t shard_bytes, unsigned flags, cudaStream_t stream)
 {
     const Options o = snapshot(c);
     const unsigned mode = launch_mode(flags);
-    if (shard_bytes % 16) {
-        const size_t shard16 = shard_bytes / 2;
-        const unsigned grid = pick_grid(c, o, ceil_div(shard16 * nranks, kThreads), 8);
-        return launch(k_allgather_scalar, grid, stream, mode, p, nranks, shard16);
-    }
     const size_t shard_vec = shard_bytes / 16;
+    // small tiles: about four blocks per SM, 16 ... 256 vectors each
+    const size_t per = ceil_div(ceil_div(shard_vec * (size_t)nranks, (size_t)c->num_sms * 4), (size_t)8) * 8;
+    const unsigned small_tv = (unsigned)std::min<size_t>(kThreads, std::max<size_t>(16, per));
+    const bool prefetch = prefetch_pays(o, flags, nranks, shard_vec * 16);
+    if (shard_bytes % 16) {
+        const unsigned tv = std::min(kRaggedGather, small_tv);
+        const size_t tiles = std::max<size_t>(1, ceil_div(shard_vec + 7, (size_t)tv));          // the first may be short by 7 vectors
+        return launch(k_allgather_ragged, pick_grid(c, o, tiles * nranks, 0, 0), stream, mode, p, nranks, shard_bytes, tiles, tv,
+                      prefetch ? 1 : 0);
+    }
     const size_t out_total = shard_bytes * (size_t)nranks * (size_t)nranks;
     if (o.ag_bulk_vecs == 0 && out_total <= ((size_t)128 << 20)) {
-        // register form with small tiles: about four blocks per SM, tiles of 16 ... 256 vectors
-        const size_t per = ceil_div(ceil_div(shard_vec * (size_t)nranks, (size_t)c->num_sms * 4), (size_t)8) * 8;
-        const unsigned tv = (unsigned)std::min<size_t>(kThreads, std::max<size_t>(16, per));
-        const size_t tiles = ceil_div(shard_vec, (size_t)tv);
+        // register form with small tiles
+        const size_t tiles = ceil_div(shard_vec + (shard_vec % 8 ? 7 : 0), (size_t)small_tv);   // the first tile of a shard may be short
         const unsigned grid = (unsigned)(tiles * nranks);
         if (o.blocks <= 0 || (size_t)o.blocks >= grid)             // one tile per block: a capped grid takes the looping form below
-            return launch(k_allgather_small, grid, stream, mode, p, nranks, shard_vec, tiles, tv,
-                          prefetch_pays(o, flags, nranks, shard_vec * 16) ? 1 : 0);
+            return launch(k_allgather_small, grid, stream, mode, p, nranks, shard_vec, small_tv, prefetch ? 1 : 0);
     }
     if (o.ag_bulk_vecs != 1) {
         // Default: the bulk-copy form, one block per (rank, tile); the copy engine moves the tile in once and
@@ -815,7 +821,7 @@ int launch_allgather(Context* c, const RankPtrs& p, int nranks, size_t shard_byt
         if (tiles * (size_t)nranks <= ((size_t)1 << 24)) {
             t_dyn_smem = tv * 16u;
             return launch(k_allgather_bulk, (unsigned)(tiles * nranks), stream, mode, p, nranks, shard_vec, tiles, tv, &c->bw->status,
-                          o.timeout_ns, prefetch_pays(o, flags, nranks, shard_vec * 16) ? 1 : 0);
+                          o.timeout_ns, prefetch ? 1 : 0);
         }
     }
     // One block per (rank, tile) storing to all N destinations.  Splitting a tile's destinations over
@@ -834,9 +840,11 @@ int launch_alltoall(Context* c, const RankPtrs& p, int nranks, size_t block_byte
     const Options o = snapshot(c);
     const unsigned mode = launch_mode(flags);
     if (block_bytes % 16) {
-        const size_t block16 = block_bytes / 2;
-        const unsigned grid = pick_grid(c, o, ceil_div(block16 * nranks * nranks, kThreads), 8);
-        return launch(k_alltoall_scalar, grid, stream, mode, p, nranks, block16);
+        // four vectors per thread from 16 MiB of sources (8 x 8 x 1 MB blocks 23.6 against 22.9 us, 8 x 8 x 18 KB 1.6 against 1.9)
+        const bool wide = block_bytes * (size_t)nranks * (size_t)nranks >= ((size_t)16 << 20);
+        const size_t tiles = std::max<size_t>(1, ceil_div(block_bytes / 16 + 7, (size_t)kRaggedRow * (wide ? 4 : 2)));
+        return launch(wide ? k_alltoall_ragged<4> : k_alltoall_ragged<2>, pick_grid(c, o, tiles * nranks * nranks, 0, 0), stream, mode, p,
+                      nranks, block_bytes, tiles);
     }
     const size_t block_vec = block_bytes / 16;
     if (o.ag_bulk_vecs != 1) {
@@ -961,7 +969,7 @@ int nuna_allreduce_oneshot(const void* const* src, void* const* dst, int nranks,
     if (flags & NUNA_TWOSHOT_PUT) return NUNA_ERR_INVALID_ARG;
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
-    return launch_oneshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, flags, (cudaStream_t)stream);
+    return launch_oneshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, effective_flags(flags, stream), (cudaStream_t)stream);
 }
 
 int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks, size_t count, int dtype,
@@ -982,7 +990,7 @@ int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,
             if ((st = ensure_scratch(c, need)) != NUNA_OK) return st;
         }
     }
-    return launch_twoshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, flags, (cudaStream_t)stream);
+    return launch_twoshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, effective_flags(flags, stream), (cudaStream_t)stream);
 }
 
 int nuna_allreduce(const void* const* src, void* const* dst, int nranks, size_t count, int dtype, unsigned flags,
@@ -993,6 +1001,7 @@ int nuna_allreduce(const void* const* src, void* const* dst, int nranks, size_t 
     // 128 KiB at 8 and 64 KiB at 16.  Beyond it the put form of the two-shot is the fastest kernel at every
     // size; the flag-synchronised form is used instead when the caller asks for it (NUNA_TWOSHOT_SYNC),
     // from the size where it beats the one-shot (measured per rank count, kSyncFactor x the put crossover).
+    flags = effective_flags(flags, stream);
     const size_t bytes = count * elem_size(dtype);
     size_t limit = nranks <= 2 ? ((size_t)1 << 20) : nranks <= 4 ? ((size_t)512 << 10)
                  : nranks <= 8 ? ((size_t)128 << 10) : ((size_t)64 << 10);
@@ -1030,7 +1039,7 @@ int nuna_reduce_scatter(const void* const* src, void* const* dst, int nranks, si
     if (flags & NUNA_TWOSHOT_PUT) return NUNA_ERR_INVALID_ARG;
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
-    return launch_reduce_scatter(c, make_ptrs(src, dst, nranks), nranks, dtype, shard_count, flags, (cudaStream_t)stream);
+    return launch_reduce_scatter(c, make_ptrs(src, dst, nranks), nranks, dtype, shard_count, effective_flags(flags, stream), (cudaStream_t)stream);
 }
 
 int nuna_allgather(const void* const* src, void* const* dst, int nranks, size_t shard_count, int dtype,
@@ -1045,7 +1054,7 @@ int nuna_allgather(const void* const* src, void* const* dst, int nranks, size_t 
     if (flags & NUNA_TWOSHOT_PUT) return NUNA_ERR_INVALID_ARG;
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
-    return launch_allgather(c, make_ptrs(src, dst, nranks), nranks, shard_count * elem_size(dtype), flags, (cudaStream_t)stream);
+    return launch_allgather(c, make_ptrs(src, dst, nranks), nranks, shard_count * elem_size(dtype), effective_flags(flags, stream), (cudaStream_t)stream);
 }
 
 int nuna_alltoall(const void* const* src, void* const* dst, int nranks, size_t block_count, int dtype,
@@ -1060,7 +1069,7 @@ int nuna_alltoall(const void* const* src, void* const* dst, int nranks, size_t b
     if (flags & NUNA_TWOSHOT_PUT) return NUNA_ERR_INVALID_ARG;
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
-    return launch_alltoall(c, make_ptrs(src, dst, nranks), nranks, block_count * elem_size(dtype), flags, (cudaStream_t)stream);
+    return launch_alltoall(c, make_ptrs(src, dst, nranks), nranks, block_count * elem_size(dtype), effective_flags(flags, stream), (cudaStream_t)stream);
 }
 
 int nuna_allreduce_host(const void* const* src, void* const* dst, int nranks, size_t count, int dtype,
@@ -1437,5 +1446,6 @@ extern "C" int nuna_allreduce_twoshot_static(const void* const* src, void* const
     if ((st = static_setup(&s)) != NUNA_OK) return st;
     // tiles of 4 KiB per source (the fixed flag array has one word per 4 KiB of the shard), fewer vectors for many ranks
     return launch_twoshot_flags(s->num_sms, 0, make_ptrs(src, dst, nranks), nranks, dtype, count, kStaticTileVec, kStaticTileVec,
-                                s->shard, s->flags, s->barrier, 1000000000ull, false, 0u, (cudaStream_t)stream);
+                                s->shard, s->flags, s->barrier, 1000000000ull, (effective_flags(0u, stream) & NUNA_LAUNCH_PDL) != 0u, 0u,
+                                (cudaStream_t)stream);
 }

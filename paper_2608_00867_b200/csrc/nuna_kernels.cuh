@@ -921,17 +921,74 @@ k_reduce_scatter(const RankPtrs p, const size_t shard_vec, const size_t tiles_pe
     pdl_trigger();
 }
 
-// Any shard length: one element per thread (slow path, used when S % 8 != 0).
-template <int N, int DT>
-__global__ void __launch_bounds__(kThreads)
-k_reduce_scatter_scalar(const RankPtrs p, const size_t shard)
+// Any shard length.  Shard r starts `sh` bytes into a 16-byte vector of every source (the same sh in all of them), so the
+// sources are still read and folded as aligned vectors; the result stream is then shifted to the destination's alignment,
+// which costs one exchange between neighbouring threads per folded vector instead of one per source.  A tile is
+// kRaggedTile result vectors (whole 128-byte lines of the destination) made from one source vector more; lane 31 of a warp takes its neighbour from the next
+// warp's lane 0 through shared memory.  What no whole source vector covers (fewer than three vectors at the end of a
+// shard) goes element by element, as an item of its own so that it adds no second round trip to a tile's.  Bound by the
+// reads, like the aligned kernel.  8 ranks x 67 229 bf16 per shard 2.73 -> 2.3 us, 4 x 7 137 545 85 -> 42 us (1.03 of the
+// copy peak) against one element per thread.
+constexpr int kRaggedTile = kThreads - 8;
+
+// 16 bytes starting `sh` (0 ... 15, a multiple of 2) bytes into the 32 bytes {a, b}.
+__device__ __forceinline__ uint4 align_bytes(uint4 a, uint4 b, unsigned sh)
 {
+    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z;
+    if (sh & 8u) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = b.w; }
+    if (sh & 4u) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
+    const unsigned bits = (sh & 3u) * 8u;
+    return make_uint4(__funnelshift_r(w0, w1, bits), __funnelshift_r(w1, w2, bits), __funnelshift_r(w2, w3, bits),
+                      __funnelshift_r(w3, w4, bits));
+}
+
+__device__ __forceinline__ uint4 shfl_down_v4(uint4 v)
+{
+    return make_uint4(__shfl_down_sync(0xFFFFFFFFu, v.x, 1), __shfl_down_sync(0xFFFFFFFFu, v.y, 1),
+                      __shfl_down_sync(0xFFFFFFFFu, v.z, 1), __shfl_down_sync(0xFFFFFFFFu, v.w, 1));
+}
+
+template <int N, int DT>
+__global__ void __launch_bounds__(kThreads, min_blocks(N))
+k_reduce_scatter_ragged(const RankPtrs p, const size_t shard, const size_t tiles_per_shard)
+{
+    constexpr size_t kE = Elem<DT>::kElems;
+    __shared__ uint4 edge[kThreads / 32];
     pdl_wait();
-    const size_t total = shard * N;
-    for (size_t e = (size_t)blockIdx.x * kThreads + threadIdx.x; e < total; e += (size_t)gridDim.x * kThreads) {
-        const int r = (int)(e / shard);
-        store_elem<DT>(p.dst[r], e - (size_t)r * shard, fold_scalar<N, DT>(p, e));
+    const size_t whole = shard * N / kE;                            // whole vectors of a source
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x / 32u;
+    for (unsigned item = blockIdx.x; item < (unsigned)(tiles_per_shard + 1) * N; item += gridDim.x) {
+        const int r = (int)(item % N);
+        const size_t tile = item / N;
+        const size_t e0 = (size_t)r * shard, q0 = e0 / kE;
+        const unsigned sh = (unsigned)(e0 % kE) * Elem<DT>::kBytes;
+        const size_t more = sh ? 1 : 0;                             // source vectors beyond the result vectors
+        const size_t have = whole > q0 + more ? whole - q0 - more : 0;
+        const size_t nd = shard / kE < have ? shard / kE : have;    // result vectors made of whole source vectors
+        if (tile == tiles_per_shard) {
+            const size_t i = nd * kE + threadIdx.x;                 // at most 3 * kE - 1 elements
+            if (i < shard) store_elem<DT>(p.dst[r], i, fold_scalar<N, DT>(p, e0 + i));
+            continue;
+        }
+        const size_t j = tile * kRaggedTile + threadIdx.x;
+        uint4 o = make_uint4(0u, 0u, 0u, 0u);
+        if (nd != 0 && j < nd + more) {
+            uint4 v[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) v[k] = ld_src(p.src[k] + q0 + j);
+            o = fold_vectors<N, DT>(v);
+        }
+        if (sh) {                                                   // the same for the whole block
+            uint4 next = shfl_down_v4(o);
+            if (lane == 0) edge[warp] = o;
+            __syncthreads();
+            if (lane == 31u && warp + 1 < kThreads / 32) next = edge[warp + 1];
+            o = align_bytes(o, next, sh);
+        }
+        if (threadIdx.x < kRaggedTile && j < nd) st_stream(p.dst[r] + j, o);
+        if (sh) __syncthreads();                                    // nobody overwrites an edge that is still to be read
     }
+    pdl_trigger();
 }
 
 // ---- allgather: work item = (rank r, tile of shard r, group of destinations); local load, remote store ----
@@ -983,16 +1040,18 @@ k_allgather(const RankPtrs p, const int nranks, const size_t shard_vec, const si
 // the bulk-copy form below up to 128 MiB of output (16 x 8 KiB 1.28 against 1.68 us, 16 x 64 KiB 3.46 against 3.81,
 // 8 x 64 KiB 1.60 against 1.92, 16 x 512 KiB 22.9 against 24.1; 8 x 8 MiB 96.5 against 93.9).
 __global__ void __launch_bounds__(kThreads)
-k_allgather_small(const RankPtrs p, const int nranks, const size_t shard_vec, const size_t tiles_per_shard, const unsigned tv,
-                  const int prefetch)
+k_allgather_small(const RankPtrs p, const int nranks, const size_t shard_vec, const unsigned tv, const int prefetch)
 {
     const int r = (int)(blockIdx.x % (unsigned)nranks);
-    const size_t tile = blockIdx.x / (unsigned)nranks;
-    const size_t i0 = tile * tv;
-    if (prefetch && threadIdx.x == 0 && i0 < shard_vec)
-        prefetch_l2_bulk(p.src[r] + i0, (unsigned)(shard_vec - i0 < (size_t)tv ? shard_vec - i0 : (size_t)tv) * 16u);
+    // tiles end on 128-byte lines of the destinations: the first one is short by what the shard starts into a line (shards of
+    // 65 552 bytes 3.66 -> 3.51 us; it changes nothing for the bulk copies of k_alltoall_bulk)
+    const size_t tile = blockIdx.x / (unsigned)nranks, skip = (size_t)r * shard_vec & 7u;
+    if (prefetch && threadIdx.x == 0) {
+        const size_t i0 = tile ? tile * tv - skip : 0, i1 = tile * tv + tv - skip;
+        if (i0 < shard_vec) prefetch_l2_bulk(p.src[r] + i0, (unsigned)((i1 < shard_vec ? i1 : shard_vec) - i0) * 16u);
+    }
     pdl_wait();
-    const size_t i = i0 + threadIdx.x;
+    const size_t i = tile * tv + threadIdx.x - skip;                // wraps below zero in the first tile: not < shard_vec
     if (threadIdx.x < tv && i < shard_vec) {
         const uint4 v = ld_src(p.src[r] + i);
         for (int d = 0; d < nranks; ++d) st_stream(p.dst[d] + (size_t)r * shard_vec + i, v);
@@ -1045,16 +1104,58 @@ k_allgather_bulk(const RankPtrs p, const int nranks, const size_t shard_vec, con
     pdl_trigger();
 }
 
+// Any shard length (in bytes, a multiple of 2): shard r lands `sh` bytes into a 16-byte vector of every destination.  A
+// thread makes one aligned destination vector out of two neighbouring source vectors (its own and the lane's before it)
+// and stores it N times; the bytes ahead of the first and behind the last such vector (at most 22 units of 16 bits) are
+// the last warp's, side by side with the vectors, so a tile is at most kRaggedGather vectors.  Bound by the N stores per
+// load, as in k_allgather_small, whose tile sizes it uses otherwise.
+constexpr unsigned kRaggedGather = kThreads - 32;
+
 __global__ void __launch_bounds__(kThreads)
-k_allgather_scalar(const RankPtrs p, const int nranks, const size_t shard)
+k_allgather_ragged(const RankPtrs p, const int nranks, const size_t shard_bytes, const size_t tiles_per_shard, const unsigned tv,
+                   const int prefetch)
 {
-    pdl_wait();
-    const size_t total = shard * nranks;
-    for (size_t e = (size_t)blockIdx.x * kThreads + threadIdx.x; e < total; e += (size_t)gridDim.x * kThreads) {
-        const int r = (int)(e / shard);
-        const uint16_t v = ld_src16(reinterpret_cast<const uint16_t*>(p.src[r]) + (e - (size_t)r * shard));
-        for (int d = 0; d < nranks; ++d) reinterpret_cast<uint16_t*>(p.dst[d])[e] = v;
+    const size_t nw = shard_bytes / 16;                             // whole source vectors
+    if (prefetch && threadIdx.x == 0) {
+        const size_t i0 = (size_t)(blockIdx.x / (unsigned)nranks) * tv;
+        if (i0 < nw) prefetch_l2_bulk(p.src[blockIdx.x % (unsigned)nranks] + i0, (unsigned)(nw - i0 < (size_t)tv ? nw - i0 : (size_t)tv) * 16u);
     }
+    pdl_wait();
+    for (unsigned item = blockIdx.x; item < (unsigned)tiles_per_shard * (unsigned)nranks; item += gridDim.x) {
+        const unsigned r = item % (unsigned)nranks;
+        const size_t tile = item / (unsigned)nranks;
+        const size_t off = (size_t)r * shard_bytes;
+        const unsigned sh = (unsigned)(off & 15u);
+        // destination vector off / 16 + t; a warp's stores start on a 128-byte line (half-written sectors cost 16 x 64 KiB
+        // shards, one element ragged, 0.5 us), so the first tile is short by what the shard starts into a line
+        const size_t t0 = sh ? 1 : 0, t = tile * tv + threadIdx.x - (off / 16 & 7u);       // wraps below zero: not < nw
+        const bool mine = threadIdx.x < tv && t < nw;
+        const bool edge = sh && (threadIdx.x & 31u) == 0 && mine && t != 0;
+        uint4 cur = make_uint4(0u, 0u, 0u, 0u), before = cur, out;
+        if (mine) cur = ld_src(p.src[r] + t);
+        if (edge) before = ld_src(p.src[r] + t - 1);                // in flight together with the warp's own vectors
+        out = cur;
+        if (sh) {                                                   // the same for the whole block
+            uint4 prev = make_uint4(__shfl_up_sync(0xFFFFFFFFu, cur.x, 1), __shfl_up_sync(0xFFFFFFFFu, cur.y, 1),
+                                    __shfl_up_sync(0xFFFFFFFFu, cur.z, 1), __shfl_up_sync(0xFFFFFFFFu, cur.w, 1));
+            if (edge) prev = before;
+            out = align_bytes(prev, cur, 16u - sh);
+        }
+        if (mine && t >= t0)
+            for (int d = 0; d < nranks; ++d) st_stream(p.dst[d] + off / 16 + t, out);
+        if (threadIdx.x >= kRaggedGather) {
+            const size_t head = nw > t0 ? 16 * t0 - (t0 ? sh : 0) : 0;                     // source bytes [0, head) and [body, end) are left
+            const size_t body = nw > t0 ? 16 * nw - sh : 0;
+            const size_t first = (tile == 0 ? head : 0) / 2, last = (tile == tiles_per_shard - 1 ? shard_bytes - body : 0) / 2;
+            const size_t k = threadIdx.x - kRaggedGather;
+            if (k < first + last) {
+                const size_t at = k < first ? k : body / 2 + (k - first);
+                const uint16_t h = ld_src16(reinterpret_cast<const uint16_t*>(p.src[r]) + at);
+                for (int d = 0; d < nranks; ++d) reinterpret_cast<uint16_t*>(p.dst[d])[off / 2 + at] = h;
+            }
+        }
+    }
+    pdl_trigger();
 }
 
 // ---- alltoall: work item = (sender r, receiver d, tile of the block r sends to d) -------------------------
@@ -1118,18 +1219,65 @@ k_alltoall_bulk(const RankPtrs p, const int nranks, const size_t block_vec, cons
     pdl_trigger();
 }
 
-// Any block length (used when S % 8 != 0): one element per thread.
+// Any block length (in bytes, a multiple of 2).  Sender and receiver see the block at unrelated 16-byte phases: a thread
+// makes an aligned destination vector out of two neighbouring aligned source vectors, the second one its right-hand
+// lane's; the ends of a block (at most 22 units of 16 bits) are the last warp's, as in k_allgather_ragged.  Each of the
+// other threads makes U vectors so that enough loads are in flight (with one store per load nothing else hides their
+// latency).  8 ranks x 32 769 bf16 per block 8.1 -> 2.5 us, 4 x 5 332 391 300 -> 55 us against one element per thread.
+constexpr unsigned kRaggedRow = kThreads - 32;
+
+template <int U>
 __global__ void __launch_bounds__(kThreads)
-k_alltoall_scalar(const RankPtrs p, const int nranks, const size_t block)
+k_alltoall_ragged(const RankPtrs p, const int nranks, const size_t block_bytes, const size_t tiles_per_block)
 {
     pdl_wait();
-    const size_t per_rank = block * nranks, total = per_rank * nranks;
-    for (size_t e = (size_t)blockIdx.x * kThreads + threadIdx.x; e < total; e += (size_t)gridDim.x * kThreads) {
-        const int d = (int)(e / per_rank);
-        const size_t within = e - (size_t)d * per_rank;
-        const int r = (int)(within / block);
-        const size_t i = within - (size_t)r * block;
-        reinterpret_cast<uint16_t*>(p.dst[d])[within] = ld_src16(reinterpret_cast<const uint16_t*>(p.src[r]) + (size_t)d * block + i);
+    const unsigned pairs = (unsigned)(nranks * nranks);
+    const size_t whole = block_bytes * nranks / 16;                 // whole vectors of a source
+    for (unsigned item = blockIdx.x; item < (unsigned)tiles_per_block * pairs; item += gridDim.x) {
+        const unsigned pair = item % pairs;                         // pairs fastest: neighbours hit different buffers
+        const size_t tile = item / pairs;
+        const unsigned r = pair / (unsigned)nranks, d = pair % (unsigned)nranks;
+        const size_t a = (size_t)d * block_bytes, b = (size_t)r * block_bytes;            // byte offsets in source and destination
+        const unsigned sb = (unsigned)(b & 15u), sh = (unsigned)((a - sb) & 15u);
+        const size_t t0 = sb ? 1 : 0, more = sh ? 1 : 0;            // first destination vector that belongs to the block alone
+        const size_t q0 = (a + 16 * t0 - sb) / 16;                  // its first source vector
+        size_t n = (block_bytes + sb) / 16 > t0 ? (block_bytes + sb) / 16 - t0 : 0;       // such destination vectors ...
+        if (n > (whole > q0 + more ? whole - q0 - more : 0)) n = whole > q0 + more ? whole - q0 - more : 0;   // ... made of whole source vectors
+        if (threadIdx.x >= kRaggedRow) {
+            const size_t head = n ? 16 * t0 - sb * t0 : 0, body = n ? head + 16 * n : 0;  // block bytes [0, head) and [body, end) are left
+            const size_t first = (tile == 0 ? head : 0) / 2, last = (tile == tiles_per_block - 1 ? block_bytes - body : 0) / 2;
+            const size_t k = threadIdx.x - kRaggedRow;
+            if (k < first + last) {
+                const size_t at = k < first ? k : body / 2 + (k - first);
+                reinterpret_cast<uint16_t*>(p.dst[d])[b / 2 + at] = ld_src16(reinterpret_cast<const uint16_t*>(p.src[r]) + a / 2 + at);
+            }
+            continue;
+        }
+        uint4* out = p.dst[d] + b / 16 + t0;
+        const uint4* in = p.src[r] + q0;
+        // a warp's stores start on a 128-byte line, as in k_allgather_ragged; i wraps below zero in the first tile
+        const size_t base = tile * (kRaggedRow * U) + threadIdx.x - ((b / 16 + t0) & 7u);
+        uint4 v[U], behind[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const size_t i = base + (size_t)u * kRaggedRow;
+            v[u] = behind[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (n != 0 && i < n + more) v[u] = ld_src(in + i);
+            if (sh && (threadIdx.x & 31u) == 31u && i < n) behind[u] = ld_src(in + i + 1);   // in flight together with the rest
+        }
+        if (sh) {                                                   // the same for the whole block
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                uint4 next = shfl_down_v4(v[u]);
+                if ((threadIdx.x & 31u) == 31u) next = behind[u];
+                v[u] = align_bytes(v[u], next, sh);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const size_t i = base + (size_t)u * kRaggedRow;
+            if (i < n) st_stream(out + i, v[u]);
+        }
     }
     pdl_trigger();
 }
