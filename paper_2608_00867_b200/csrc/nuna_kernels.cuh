@@ -307,7 +307,7 @@ __device__ __forceinline__ void oneshot_item(const RankPtrs& p, size_t nvec, siz
 
 template <int N, int U, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N * U))
-k_oneshot_rr(const RankPtrs p, const size_t count, const size_t ntiles)
+k_oneshot_rr(const RankPtrs p, const size_t count, const size_t ntiles, const ParamPad<16>)
 {
     pdl_wait();
     const size_t nvec = count / Elem<DT>::kElems;
@@ -541,7 +541,7 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
 
 template <int N, int C, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
-k_oneshot_regs(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int mode)
+k_oneshot_regs(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int mode, const ParamPad<8>)
 {
     oneshot_regs_body<N, C, DT, false>(p, count, ntiles, tv, mode, nullptr, 0u, 0u);
 }
@@ -909,7 +909,7 @@ __device__ __forceinline__ void reduce_tile(const RankPtrs& p, uint4* out, size_
 // against 6.40.)
 template <int N, int U, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N * U))
-k_reduce_scatter(const RankPtrs p, const size_t shard_vec, const size_t tiles_per_shard)
+k_reduce_scatter(const RankPtrs p, const size_t shard_vec, const size_t tiles_per_shard, const ParamPad<16>)
 {
     pdl_wait();
     const size_t nitems = tiles_per_shard * N;
@@ -950,7 +950,7 @@ __device__ __forceinline__ uint4 shfl_down_v4(uint4 v)
 
 template <int N, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
-k_reduce_scatter_ragged(const RankPtrs p, const size_t shard, const size_t tiles_per_shard)
+k_reduce_scatter_ragged(const RankPtrs p, const size_t shard, const size_t tiles_per_shard, const ParamPad<16>)
 {
     constexpr size_t kE = Elem<DT>::kElems;
     __shared__ uint4 edge[kThreads / 32];
@@ -1040,7 +1040,8 @@ k_allgather(const RankPtrs p, const int nranks, const size_t shard_vec, const si
 // the bulk-copy form below up to 128 MiB of output (16 x 8 KiB 1.28 against 1.68 us, 16 x 64 KiB 3.46 against 3.81,
 // 8 x 64 KiB 1.60 against 1.92, 16 x 512 KiB 22.9 against 24.1; 8 x 8 MiB 96.5 against 93.9).
 __global__ void __launch_bounds__(kThreads)
-k_allgather_small(const RankPtrs p, const int nranks, const size_t shard_vec, const unsigned tv, const int prefetch)
+k_allgather_small(const RankPtrs p, const int nranks, const size_t shard_vec, const unsigned tv, const int prefetch,
+                  const ParamPad<8>)
 {
     const int r = (int)(blockIdx.x % (unsigned)nranks);
     // tiles end on 128-byte lines of the destinations: the first one is short by what the shard starts into a line (shards of
@@ -1077,7 +1078,7 @@ __device__ __forceinline__ void bulk_store_drain()       // this thread's bulk s
 // tv = vectors per tile; shared memory = tv * 16 bytes.
 __global__ void __launch_bounds__(kThreads)
 k_allgather_bulk(const RankPtrs p, const int nranks, const size_t shard_vec, const size_t tiles_per_shard, const unsigned tv,
-                 unsigned* status, const unsigned long long timeout_ns, const int prefetch)
+                 unsigned* status, const unsigned long long timeout_ns, const int prefetch, const ParamPad<44>)
 {
     extern __shared__ __align__(128) unsigned char stage_raw[];
     __shared__ __align__(8) uint64_t bar;
@@ -1194,7 +1195,7 @@ k_alltoall(const RankPtrs p, const int nranks, const size_t block_vec, const siz
 // touching a register.  tv = vectors per tile; shared memory = tv * 16 bytes; one block per (pair, tile).
 __global__ void __launch_bounds__(kThreads)
 k_alltoall_bulk(const RankPtrs p, const int nranks, const size_t block_vec, const size_t tiles_per_block, const unsigned tv,
-                unsigned* status, const unsigned long long timeout_ns, const int prefetch)
+                unsigned* status, const unsigned long long timeout_ns, const int prefetch, const ParamPad<44>)
 {
     extern __shared__ __align__(128) unsigned char stage_raw[];
     __shared__ __align__(8) uint64_t bar;
@@ -1228,7 +1229,7 @@ constexpr unsigned kRaggedRow = kThreads - 32;
 
 template <int U>
 __global__ void __launch_bounds__(kThreads)
-k_alltoall_ragged(const RankPtrs p, const int nranks, const size_t block_bytes, const size_t tiles_per_block)
+k_alltoall_ragged(const RankPtrs p, const int nranks, const size_t block_bytes, const size_t tiles_per_block, const ParamPad<8>)
 {
     pdl_wait();
     const unsigned pairs = (unsigned)(nranks * nranks);
@@ -1409,7 +1410,7 @@ __device__ __forceinline__ void half_sync(int id) { asm volatile("bar.sync %0, 1
 template <int N, int DT, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
 k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const size_t count, const unsigned tv,
-                const unsigned lead_max, BarrierWords* bw, const unsigned long long timeout_ns, const unsigned int debug)
+                const unsigned lead_max, BarrierWords* bw, const unsigned long long timeout_ns, const unsigned int debug, const ParamPad<44>)
 {
     constexpr unsigned kHalf = kThreads / 2;
     const unsigned wait_bias = debug & 1u;
@@ -1516,7 +1517,7 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
 // slower up to 4 MiB per rank -- 512 KiB: 3.2 vs 2.85 us -- and within 1.5 % beyond, so it was not kept.)
 template <int N, int U, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N * U))
-k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const int prefetch)
+k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const int prefetch, const ParamPad<12>)
 {
     const size_t nvec = count / Elem<DT>::kElems;
     if (prefetch && blockIdx.x < ntiles && threadIdx.x < N) {        // thread r: source r's slice of the first tile

@@ -14,6 +14,15 @@ struct RankPtrs {
     uint4* dst[kMaxRanks];
 };
 
+// Unused trailing kernel argument.  The driver's launch call costs the host 0.35 us more unless the kernel's parameters
+// come to 20 ... 32 bytes beyond a multiple of 64 (measured in steps of 4 bytes from 16 to 450 bytes, two machines,
+// 1.65 against 2.0 us with a programmatic launch; plain launches want exactly 32).  The kernels that small eager calls
+// take are padded to 288 or 352 bytes; launch_padded() checks it.
+template <int kBytes>
+struct ParamPad {
+    unsigned char unused[kBytes];
+};
+
 // Kernel argument of the single-kernel chain: the buffer sets its nodes rotate over, by value.
 constexpr int kMaxChainSets = 8;
 struct ChainSets {
