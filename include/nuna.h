@@ -91,9 +91,9 @@ typedef enum { NUNA_BF16 = 0, NUNA_F16 = 1, NUNA_F32 = 2 } nuna_dtype_t;   /* el
  * stream capture behave as if the flag were given; in a captured graph the edge is an ordinary one and the
  * kernel is chosen for it unless the flag is given.  The round-robin one-shot ignores it above 16 MiB of sources, where it was measured
  * not to pay.  Unless
- * NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot (below 8 MiB per rank), of either
- * two-shot form (up to 128 MiB of sources; 8 MiB beyond 8 ranks) and of the bulk-copy allgather and
- * alltoall also asks L2, before that wait, to fetch its first tile of the sources (a prefetch returns
+ * NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot and of the put form (up to 64 MiB of
+ * sources; beyond 8 MiB the first wave only), of the flag-synchronised two-shot and of the allgather and
+ * alltoall (up to 128 MiB of sources; 8 MiB beyond 8 ranks) also asks L2, before that wait, to fetch its first tile of the sources (a prefetch returns
  * nothing to the kernel; L2 is the point of coherence, so what the predecessor still writes is what the
  * loads after the wait see).                                                                            */
 #define NUNA_LAUNCH_PDL       64u
@@ -313,13 +313,15 @@ int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,
                            size_t count, int dtype, unsigned flags, void* stream);
 
 /* Allreduce with the algorithm chosen by message size -- the counterpart of the paper's per-collective
- * choice between routing schemes by a size threshold (Section 4.1.2): one-shot while the message is small
- * enough for its single step to win (measured: up to 1 MiB per rank at 2 ranks, 512 KiB at 4, 128 KiB at
- * 8, 64 KiB at 16; under NUNA_PLACE_AUTO, whose one-shot kernel shares each tile's loads between the
- * destinations, 8 MiB of sources in total with NUNA_LAUNCH_PDL, without it 2 MiB (512 KiB beyond 8 ranks);
- * and again from 8 MiB per rank at 8 ranks or fewer, cold), beyond that the put form of the two-shot.
- * With NUNA_TWOSHOT_SYNC the large-message choice is the flag-synchronised two-shot instead, from eight
- * times those sizes (below, the one-shot is faster than it).  Same bits whichever is chosen.            */
+ * choice between routing schemes by a size threshold (Section 4.1.2), at measured crossovers.  Under
+ * NUNA_PLACE_AUTO, whose one-shot kernel shares each tile's loads between the destinations: one-shot at every
+ * size (up to 16 MiB of sources in total beyond 8 ranks).  Otherwise the put form of the two-shot, except that
+ * the round-robin one-shot takes the smallest messages: with NUNA_LAUNCH_PDL up to 16 KiB per rank (256 KiB with
+ * NUNA_HINT_RESIDENT) at 4 ranks or fewer, without it up to 1 MiB at 2 ranks, 512 KiB at 4, 64 KiB at 8, 8 KiB
+ * at 16.  With NUNA_TWOSHOT_SYNC the large-message choice is the flag-synchronised two-shot instead, from 8 MiB
+ * per rank at 2 ranks, 4 MiB at 4, 1 MiB at 8, 512 KiB at 16 (or, under NUNA_PLACE_AUTO, 64 MiB of sources in
+ * total with NUNA_LAUNCH_PDL, 16 MiB without it; 4 MiB beyond 8 ranks, where that is more).  Same bits whichever
+ * is chosen.                                                                                              */
 int nuna_allreduce(const void* const* src, void* const* dst, int nranks,
                    size_t count, int dtype, unsigned flags, void* stream);
 

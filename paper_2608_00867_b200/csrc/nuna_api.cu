@@ -240,6 +240,7 @@ static unsigned effective_flags(unsigned flags, void* stream)
 }
 
 static thread_local unsigned t_cluster_dim = 0;           // > 0: next launch() uses clusters of this many blocks
+static thread_local unsigned t_block = 0;                 // > 0: next launch() uses blocks of this many threads
 static thread_local unsigned t_dyn_smem = 0;              // next launch() requests this much dynamic shared memory
 
 template <typename... Args, typename... Act>
@@ -247,7 +248,8 @@ static int launch(void (*kernel)(Args...), unsigned grid, cudaStream_t stream, u
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(t_block > 0 ? t_block : (unsigned)kThreads, 1, 1);
+    t_block = 0;
     cfg.dynamicSmemBytes = t_dyn_smem;
     t_dyn_smem = 0;
     cfg.stream = stream;
@@ -565,44 +567,75 @@ static int launch_group(Context* c, const Options& o, const RankPtrs& p, size_t 
     return launch(k, grid, stream, mode, p, count, ntiles);
 }
 
-// Co-located group sharing the tile through registers: one (tile, C destinations) item per block.
-// Tile size (vectors per source), measured at 8 ranks, 8 KiB ... 64 MiB per rank, cold and L2-resident:
-// one block per SM with tiles of 8 ... 56 vectors while the message is that small (64 blocks of 8 vectors at
-// 8 KiB: 1.08 us per L2-resident graph node against 1.38 us with eight full blocks); then four blocks per SM
-// with tiles of 56 ... 256 vectors (512 KiB cold behind a dependent launch: 586 blocks of 56 vectors, 2.1 us
-// against 2.8 us with 256 full tiles); full tiles beyond.  Tiles never exceed a block's width: contiguous
-// chunks of several rows per block were slower from 8 MiB per rank (23.0 against 21.7 us).
-// `resident` = blocks of the kernel an SM holds: the blocks must fit in one wave (16 ranks, 3 blocks per SM, 256 KiB
-// per rank: 3.46 us with 586 blocks of 56 vectors, 2.42 us with 294 of 112).
-static unsigned regs_tile_vecs(const Context* c, const Options& o, size_t nvec, int ksplit, int resident)
+// How the kernels that hold a tile in registers and store it to several destinations (k_oneshot_regs, k_twoshot_put)
+// are launched: vectors per source per tile, threads per block, and how many blocks prefetch ahead of the wait.
+struct TileShape {
+    unsigned tv, threads, prefetch_blocks;
+};
+
+// One tile per block.  Measured at 2, 4, 8 and 16 ranks, 16 KiB ... 64 MiB per rank, tiles of 16 ... 256 vectors in blocks
+// of 32 ... 256 threads, as dependent graph nodes (us at 8 ranks; u = vectors per source and SM; `ksplit` blocks share a
+// tile, each with a part of the destinations):
+// * u <= 56: one block per SM, tiles of 8 ... 56 vectors (8 KiB: 1.08 resident against 1.38 with eight full blocks).
+// * up to 8 MiB of sources: four blocks per SM, as many as stay resident, tiles of 56 ... 256 vectors (512 KiB cold: 2.1
+//   against 2.8 with full tiles; 16 ranks x 256 KiB, three blocks per SM: 3.46 with 586 blocks, 2.42 with 294).
+// * 8 to 16 MiB of sources, cold: eight blocks per SM, i.e. two waves, tiles from 112 vectors: the second wave's loads run
+//   beside the first one's stores (2 MiB 6.16 -> 5.4, 1.5 MiB 4.79 -> 4.2; 4 ranks x 4 MiB 5.87 -> 5.4).
+// * 16 to 64 MiB, cold: tiles of 192 vectors (256 up to 4 ranks) in blocks of just so many threads, and only the first wave
+//   prefetches: later blocks would ask L2 for what they load at once (4 MiB 11.4 -> 11.0, 6 MiB 16.9 -> 16.1, 8 MiB
+//   21.5 -> 21.1; 4 ranks x 8 MiB 11.5 -> 10.9).
+// * beyond, cold: no prefetch, half the destinations per block; half-full blocks from 5 to 8 ranks (64 MiB 159.3 -> 157.6).
+// * L2-resident sources: narrower blocks, cheaper to start: 128 threads up to u = 32 (16 KiB 1.05 -> 1.02), beyond 4 ranks
+//   one block per SM of just as many threads as the tile up to u = 128 (128 KiB 1.22 -> 1.13, 256 KiB 1.37 -> 1.32), blocks
+//   of 128 vectors and threads from u = 448 (2 MiB 4.2 -> 3.5, 4 ranks x 2 MiB 3.2 -> 2.2); otherwise the full-width blocks
+//   above are ahead.  (Cold, narrow blocks are slower up to 8 MiB of sources: more of them start
+//   on an SM while the predecessor still drains, unevenly -- 512 KiB 2.07 with 256 threads, 2.6 with 64.)
+// `resident` = full-width blocks of the kernel an SM holds.
+static TileShape tile_shape(const Context* c, const Options& o, int nranks, size_t nvec, int ksplit, int resident, unsigned flags,
+                            bool may_prefetch)
 {
-    if (o.regs_vecs > 0) return (unsigned)std::min(kThreads, std::max(8, o.regs_vecs / 8 * 8));
-    const size_t units = nvec * (size_t)ksplit;
+    const size_t sms = (size_t)c->num_sms, units = nvec * (size_t)ksplit, total = nvec * 16 * (size_t)nranks;
     const size_t per_sm = (size_t)std::max(1, std::min(4, resident));
-    if (o.blocks > 0 && (size_t)o.blocks < (size_t)c->num_sms * per_sm) {          // a capped grid: as few tiles as blocks, then full tiles
-        const size_t capped = ceil_div(ceil_div(units, (size_t)o.blocks), (size_t)8) * 8;
-        return (unsigned)std::min<size_t>(kThreads, std::max<size_t>(8, capped));
+    const bool hot = (flags & NUNA_HINT_RESIDENT) != 0u;
+    const auto tile_for = [&](size_t blocks) { return ceil_div(ceil_div(units, blocks), (size_t)8) * 8; };
+    const auto clamp = [](size_t v, size_t lo) { return (unsigned)std::min<size_t>(kThreads, std::max(lo, v)); };
+    const unsigned everyone = may_prefetch && !hot && o.prefetch != 1 ? ~0u : 0u, first_wave = everyone ? (unsigned)(sms * 4) : 0u;
+    if (o.regs_vecs > 0) return {(unsigned)std::min(kThreads, std::max(8, o.regs_vecs / 8 * 8)), (unsigned)kThreads, everyone};
+    if (o.blocks > 0 && (size_t)o.blocks < sms * per_sm)             // a capped grid: as few tiles as blocks, then full tiles
+        return {clamp(tile_for((size_t)o.blocks), 8), (unsigned)kThreads, everyone};
+    if (hot && units <= sms * 32) return {clamp(tile_for(sms), 16), 128u, 0u};
+    if (hot && nranks > 4 && units <= sms * 128) {
+        const unsigned tv = clamp(tile_for(sms), 64);
+        return {tv, (tv + 31u) / 32u * 32u, 0u};
     }
-    const size_t one = ceil_div(ceil_div(units, (size_t)c->num_sms), (size_t)8) * 8;
-    if (one <= 56) return (unsigned)std::max<size_t>(8, one);
-    const size_t many = ceil_div(ceil_div(units, (size_t)c->num_sms * per_sm), (size_t)8) * 8;
-    return (unsigned)std::min<size_t>(kThreads, std::max<size_t>(56, many));
+    if (hot && units > sms * 448) return {128u, 128u, 0u};
+    if (units <= sms * 56) return {clamp(tile_for(sms), 8), (unsigned)kThreads, everyone};
+    if (hot || total < ((size_t)8 << 20)) return {clamp(tile_for(sms * per_sm), 56), (unsigned)kThreads, everyone};
+    if (total <= ((size_t)16 << 20))
+        return {clamp(tile_for(sms * 2 * per_sm), 112), (unsigned)kThreads, total <= ((size_t)8 << 20) ? everyone : first_wave};
+    if (total <= ((size_t)64 << 20)) {
+        const unsigned tv = nranks <= 4 || nranks > 8 ? 256u : 192u;
+        return {tv, tv, first_wave};
+    }
+    return {nranks <= 4 || nranks > 8 ? 256u : 128u, (unsigned)kThreads, 0u};
 }
 
 template <int N, int C, int DT>
-static int launch_regs(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned flags, unsigned mode, bool may_prefetch,
-                       cudaStream_t stream)
+static int launch_regs(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned flags, unsigned mode, cudaStream_t stream)
 {
-    auto k = k_oneshot_regs<N, C, DT>;
     constexpr int kSplit = (N + C - 1) / C;
+    auto k = k_oneshot_regs<N, C, DT, false>;
+    // L2-resident sources from 8 ranks, where the fewer instructions show (8 ranks x 16 KiB 1.04 -> 1.00 us per node, x 64 KiB
+    // 1.08 -> 1.07; below, the general form measured 2 % faster)
+    if constexpr (kSplit == 1 && N >= 8)
+        if (flags & NUNA_HINT_RESIDENT) k = k_oneshot_regs<N, C, DT, true>;
     const size_t nvec = count / Elem<DT>::kElems;
-    const unsigned tv = regs_tile_vecs(c, o, nvec, kSplit, NUNA_OCC(k));
-    const size_t ntiles = ceil_div(nvec, (size_t)tv);
+    const TileShape t = tile_shape(c, o, N, nvec, kSplit, NUNA_OCC(k), flags, mode == kLaunchPdl);
+    const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
     const size_t nitems = std::max<size_t>(ntiles * kSplit, (count % Elem<DT>::kElems) ? (size_t)N : 0);
     const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), NUNA_OCC(k), 0);
-    // cold sources behind a dependent launch: fetch into L2 while the predecessor drains
-    const bool prefetch = may_prefetch && mode == kLaunchPdl && !(flags & NUNA_HINT_RESIDENT) && o.prefetch != 1;
-    return launch_padded(k, grid, stream, mode, p, count, ntiles, tv, ((flags & NUNA_HINT_RESIDENT) ? 0 : 1) | (prefetch ? 2 : 0));
+    t_block = t.threads;
+    return launch_padded(k, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
 }
 
 // Staged group kernel: one tile per block.  Tile size (vectors per source): large enough that a tile's
@@ -645,20 +678,18 @@ int launch_oneshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t 
         const unsigned m = launch_mode(flags);
         // destinations per thread: all of them, so that a tile crosses the L2 -> SM fabric once (beyond 8 ranks the
         // sixteen-destination form: 9 ranks x 512 KiB 2.25 us against 2.71 in two passes of eight, 16 ranks x 1 MiB
-        // 6.39 against 7.35); half of them for large cold messages, where two blocks per tile keep more DRAM loads
-        // in flight (8 ranks x 16 MiB cold: 41.8 us with four, 42.0 with eight)
+        // 6.39 against 7.35); half of them for cold messages beyond 64 MiB of sources, where two blocks per tile keep more
+        // DRAM loads in flight (8 ranks x 16 MiB: 41.0 us with four, 41.4 with eight; x 64 MiB 157.6 against 160.2)
         const int all = nranks > 8 ? 16 : std::min(8, pow2_at_least(nranks));
-        const bool large_cold = !(flags & NUNA_HINT_RESIDENT) && bytes >= ((size_t)8 << 20);
+        const bool large_cold = !(flags & NUNA_HINT_RESIDENT) && bytes * (size_t)nranks > ((size_t)64 << 20);
         int coloc = o.coloc > 0 ? o.coloc : (large_cold ? std::min(8, std::max(2, pow2_at_least(nranks) / 2)) : all);
         while (coloc > 2 && coloc / 2 >= nranks) coloc >>= 1;
         return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
             constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
-            // from 8 MiB per rank the prefetch only adds requests to a saturated memory system
-            // (8 ranks, four destinations per thread: 16 MiB 45.5 us with, 41.2 without; 64 MiB 175 against 158)
-            if constexpr (N > 8) { if (coloc >= 16) return launch_regs<N, 16, DT>(c, o, p, count, flags, m, !large_cold, stream); }
-            if (coloc >= 8) return launch_regs<N, 8, DT>(c, o, p, count, flags, m, !large_cold, stream);
-            if (coloc >= 4) return launch_regs<N, 4, DT>(c, o, p, count, flags, m, !large_cold, stream);
-            return launch_regs<N, 2, DT>(c, o, p, count, flags, m, !large_cold, stream);
+            if constexpr (N > 8) { if (coloc >= 16) return launch_regs<N, 16, DT>(c, o, p, count, flags, m, stream); }
+            if (coloc >= 8) return launch_regs<N, 8, DT>(c, o, p, count, flags, m, stream);
+            if (coloc >= 4) return launch_regs<N, 4, DT>(c, o, p, count, flags, m, stream);
+            return launch_regs<N, 2, DT>(c, o, p, count, flags, m, stream);
         });
     }
     if (which == OneShotKernel::Staged) {
@@ -768,12 +799,14 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
     return dispatch(nranks, pick_unroll(o, nranks), dtype, [&](auto n_, auto u_, auto d_) -> int {
         NUNA_NUD(n_, u_, d_);
         auto k = k_twoshot_put<N, U, DT>;
-        const size_t ntiles = ceil_div(nvec, (size_t)kThreads * U);
+        // host-memory sources (max_blocks > 0) are read through the link, not through L2: no prefetch, full tiles
+        TileShape t = max_blocks > 0 ? TileShape{(unsigned)kThreads, (unsigned)kThreads, 0u}
+                                     : tile_shape(c, o, nranks, nvec, 1, NUNA_OCC(k), flags, mode == kLaunchPdl);
+        const size_t ntiles = ceil_div(nvec, (size_t)t.tv * U);
         unsigned grid = pick_grid(c, o, std::max<size_t>(ntiles, 1), NUNA_OCC(k), 0);
         if (max_blocks > 0 && o.blocks <= 0) grid = std::min(grid, max_blocks);
-        // device-memory sources behind a dependent launch: fetch the first tile into L2 while the predecessor drains
-        const bool prefetch = max_blocks == 0 && prefetch_pays(o, flags, nranks, count * elem_size(dtype));
-        return launch_padded(k, grid, stream, mode, p, count, ntiles, prefetch ? 1 : 0);
+        t_block = t.threads;
+        return launch_padded(k, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
     });
 }
 
@@ -1029,34 +1062,34 @@ int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,
 int nuna_allreduce(const void* const* src, void* const* dst, int nranks, size_t count, int dtype, unsigned flags,
                    void* stream)
 {
-    // Crossover measured on B200, cold and L2-resident: the one-shot's N-fold re-reads cost more the
-    // more ranks there are, so its single step wins up to 1 MiB per rank at 2 ranks, 512 KiB at 4,
-    // 128 KiB at 8 and 64 KiB at 16.  Beyond it the put form of the two-shot is the fastest kernel at every
-    // size; the flag-synchronised form is used instead when the caller asks for it (NUNA_TWOSHOT_SYNC),
-    // from the size where it beats the one-shot (measured per rank count, kSyncFactor x the put crossover).
+    // Measured on B200 at 2, 3, 4, 6, 8 and 16 ranks, 8 KiB ... 64 MiB per rank, cold and L2-resident (us per graph node).
+    // Without NUNA_PLACE_AUTO the one-shot is the round-robin kernel, whose re-reads cost more the more ranks there are.
+    // Behind a dependent launch the put form is ahead of it (8 ranks x 8 KiB 1.14 against 1.29, x 1 MiB 3.14 against 4.92)
+    // but for the smallest messages of few ranks (2 x 8 KiB 0.92 against 0.86; L2-resident 2 x 256 KiB 1.04 against 1.01);
+    // launched plainly, where nothing is prefetched, the one-shot's many blocks pay up to 1 MiB per rank at 2 ranks (2.24
+    // against 2.16), 512 KiB at 4, 64 KiB at 8 and 8 KiB at 16.
+    // With NUNA_PLACE_AUTO the one-shot is the register-sharing kernel, equal to the put form within 2 % at every size and
+    // ahead of it beyond 64 MiB of sources, where two blocks share a tile (8 x 64 MiB 157 against 160); beyond 8 ranks and
+    // 16 MiB the put form is ahead (16 x 2 MiB 11.55 against 11.95).
     flags = effective_flags(flags, stream);
     const size_t bytes = count * elem_size(dtype);
-    size_t limit = nranks <= 2 ? ((size_t)1 << 20) : nranks <= 4 ? ((size_t)512 << 10)
-                 : nranks <= 8 ? ((size_t)128 << 10) : ((size_t)64 << 10);
-    // with NUNA_PLACE_AUTO the one-shot side is the register-sharing kernel, which stays ahead of the put form up
-    // to 8 MiB of sources in total behind a dependent launch (8 ranks, cold: 128 KiB 1.51 vs 1.92 us, 1 MiB 3.33 vs
-    // 3.74, 2 MiB 6.44 vs 6.16; 4 ranks: 2 MiB 3.34 vs 3.52, 4 MiB 5.79 vs 5.73) and up to 2 MiB launched plainly
-    // (8 ranks: 256 KiB 2.65 vs 2.70, 512 KiB 3.29 vs 3.17; beyond 8 ranks, where it needs two passes over the
-    // sources, a quarter of that); 16 ranks behind a dependent launch: 256 KiB 2.33 vs 3.21, 512 KiB 3.52 vs 4.25,
-    // 1 MiB 7.3 vs 6.6
-    // From 8 MiB per rank at 8 ranks or fewer it is ahead again, with two blocks per tile (8 ranks: 8 MiB 21.3 vs 21.6 us,
-    // 16 MiB 41.2 vs 42.1, 64 MiB 157.7 vs 160.8).
-    bool oneshot_large = false;
-    if ((flags & NUNA_PLACE_MASK) == NUNA_PLACE_AUTO) {
-        const size_t total = (flags & NUNA_LAUNCH_PDL) ? (size_t)8 << 20 : (size_t)2 << 20;
-        limit = std::max(limit, ((nranks <= 8 || (flags & NUNA_LAUNCH_PDL)) ? total : total / 4) / (size_t)nranks);
-        oneshot_large = nranks <= 8 && bytes >= ((size_t)8 << 20) && !(flags & NUNA_HINT_RESIDENT);
-    }
-    constexpr size_t kSyncFactor = 8;
+    const bool autop = (flags & NUNA_PLACE_MASK) == NUNA_PLACE_AUTO, pdl = (flags & NUNA_LAUNCH_PDL) != 0u;
     const bool sync_form = (flags & NUNA_TWOSHOT_SYNC) && !(flags & NUNA_TWOSHOT_PUT);
     const unsigned base = flags & ~(NUNA_TWOSHOT_SYNC | NUNA_TWOSHOT_PUT | (sync_form ? 0u : NUNA_TWOSHOT_SYS_SCOPE));
-    if (nranks <= 1 || bytes <= (sync_form ? limit * kSyncFactor : limit) || (oneshot_large && !sync_form))
-        return nuna_allreduce_oneshot(src, dst, nranks, count, dtype, base, stream);
+    size_t limit;                                              // the largest message, in bytes per rank, for the one-shot
+    if (sync_form) {
+        // asked for explicitly; the one-shot takes what is too small for two dependent phases
+        limit = nranks <= 2 ? ((size_t)1 << 20) : nranks <= 4 ? ((size_t)512 << 10) : nranks <= 8 ? ((size_t)128 << 10) : ((size_t)64 << 10);
+        if (autop) limit = std::max(limit, (pdl ? (size_t)8 << 20 : nranks <= 8 ? (size_t)2 << 20 : (size_t)512 << 10) / (size_t)std::max(1, nranks));
+        limit *= 8;
+    } else if (autop) {
+        limit = nranks <= 8 ? ~(size_t)0 : ((size_t)16 << 20) / (size_t)nranks;
+    } else if (pdl) {
+        limit = nranks > 4 ? 0 : (flags & NUNA_HINT_RESIDENT) ? ((size_t)256 << 10) : ((size_t)16 << 10);
+    } else {
+        limit = nranks <= 2 ? ((size_t)1 << 20) : nranks <= 4 ? ((size_t)512 << 10) : nranks <= 8 ? ((size_t)64 << 10) : ((size_t)8 << 10);
+    }
+    if (nranks <= 1 || bytes <= limit) return nuna_allreduce_oneshot(src, dst, nranks, count, dtype, base, stream);
     return nuna_allreduce_twoshot(src, dst, nranks, count, dtype, sync_form ? base : (base | NUNA_TWOSHOT_PUT), stream);
 }
 
@@ -1353,16 +1386,15 @@ int nuna_debug_oneshot_regs_traced(const void* const* src, void* const* dst, siz
     const Options o = snapshot(c);
     auto k = k_oneshot_regs_timed<N, 8, kBf16>;
     const size_t nvec = count / 8;
-    const unsigned tv = regs_tile_vecs(c, o, nvec, 1, NUNA_OCC(k));
-    const size_t ntiles = ceil_div(nvec, (size_t)tv);
+    const unsigned mode = (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchPlain;
+    const TileShape t = tile_shape(c, o, N, nvec, 1, NUNA_OCC(k), flags, mode == kLaunchPdl);
+    const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
     const size_t nitems = std::max<size_t>(ntiles, (count % 8) ? (size_t)N : 0);
     const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), NUNA_OCC(k), 0);
-    const unsigned mode = (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchPlain;
-    const bool large_cold = !(flags & NUNA_HINT_RESIDENT) && count * 2 >= ((size_t)8 << 20);
-    const bool prefetch = !large_cold && mode == kLaunchPdl && !(flags & NUNA_HINT_RESIDENT) && o.prefetch != 1;
     if (grid_blocks) *grid_blocks = grid;
-    return launch(k, grid, (cudaStream_t)stream, mode, make_ptrs(src, dst, N), count, ntiles, tv,
-                  ((flags & NUNA_HINT_RESIDENT) ? 0 : 1) | (prefetch ? 2 : 0), trace, slot, (unsigned)NUNA_DEBUG_TRACE_BLOCKS);
+    t_block = t.threads;
+    return launch(k, grid, (cudaStream_t)stream, mode, make_ptrs(src, dst, N), count, ntiles, t.tv,
+                  (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks, trace, slot, (unsigned)NUNA_DEBUG_TRACE_BLOCKS);
 }
 
 /* Test hook: a flag-synchronised two-shot whose consumers wait for a flag value that nobody publishes

@@ -477,23 +477,24 @@ __device__ __forceinline__ uint4 fold_vectors_own(const uint4 (&v)[N])
 // grid allows.  The host sizes the tile by the message: a small message is cut into many small tiles
 // (every SM gets a few blocks of a few warps each; measured faster than few full blocks at every size
 // below 4 MiB per rank), a large one uses full tiles.
-// mode bit 0: streaming stores (destinations are not re-read soon); bit 1: every block asks L2 for its
-// first tile's source slices before it waits for the predecessor kernel (dependent launches with cold
-// sources only: without a predecessor there is nothing to overlap with).
+// The block has 32 ... kThreads threads, at least tv.  stream_stores: destinations are not re-read soon.  The first
+// prefetch_blocks blocks ask L2 for their first tile's source slices before they wait for the predecessor kernel
+// (dependent launches with cold sources only: without a predecessor there is nothing to overlap with).
+// kHot: L2-resident sources, i.e. stream_stores = prefetch_blocks = 0 known at compile time.
 // kTimed (a measurement aid): thread 0 of every block also records, in nanoseconds of the global timer, when the
 // block started, when its wait for the predecessor returned and when it had issued its last store, plus the SM
 // it ran on: trace[(slot * trace_blocks + blockIdx.x) * 4 + {0, 1, 2, 3}] for blockIdx.x < trace_blocks.
-template <int N, int C, int DT, bool kTimed>
+template <int N, int C, int DT, bool kTimed, bool kHot>
 __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_t count, const size_t ntiles, const unsigned tv,
-                                                  const int mode, unsigned long long* trace, const unsigned slot,
-                                                  const unsigned trace_blocks)
+                                                  const int stream_stores, const unsigned prefetch_blocks,
+                                                  unsigned long long* trace, const unsigned slot, const unsigned trace_blocks)
 {
     constexpr int kSplit = (N + C - 1) / C;
     const size_t nvec = count / Elem<DT>::kElems;
     const size_t nitems = ntiles * kSplit;
     unsigned long long t_in = 0, t_wait = 0;
     if (kTimed && threadIdx.x == 0) t_in = globaltimer_ns();
-    if ((mode & 2) && blockIdx.x < nitems && threadIdx.x < N) {
+    if (!kHot && blockIdx.x < prefetch_blocks && blockIdx.x < nitems && threadIdx.x < N) {
         const size_t i0 = ((size_t)blockIdx.x / kSplit) * tv;        // thread r fetches source r's slice
         const uint4* a = p.src[0];
 #pragma unroll
@@ -502,7 +503,6 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
     }
     pdl_wait();
     if (kTimed && threadIdx.x == 0) t_wait = globaltimer_ns();
-    const int stream_stores = mode & 1;
     for (size_t item = blockIdx.x; item < nitems; item += gridDim.x) {
         const size_t i = (item / kSplit) * tv + threadIdx.x;
         const int d0 = (int)(item % kSplit) * C;
@@ -515,7 +515,7 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
                 const int d = d0 + c;
                 if (d < N) {
                     const uint4 o = fold_vectors_own<N, DT>(v);
-                    if (stream_stores) st_stream(p.dst[d] + i, o); else st_dst(p.dst[d] + i, o);
+                    if (!kHot && stream_stores) st_stream(p.dst[d] + i, o); else st_dst(p.dst[d] + i, o);
                 }
             }
         }
@@ -539,19 +539,20 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
     }
 }
 
-template <int N, int C, int DT>
+template <int N, int C, int DT, bool kHot>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
-k_oneshot_regs(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int mode, const ParamPad<8>)
+k_oneshot_regs(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int stream_stores,
+               const unsigned prefetch_blocks, const ParamPad<4>)
 {
-    oneshot_regs_body<N, C, DT, false>(p, count, ntiles, tv, mode, nullptr, 0u, 0u);
+    oneshot_regs_body<N, C, DT, false, kHot>(p, count, ntiles, tv, stream_stores, prefetch_blocks, nullptr, 0u, 0u);
 }
 
 template <int N, int C, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
-k_oneshot_regs_timed(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int mode,
-                     unsigned long long* trace, const unsigned slot, const unsigned trace_blocks)
+k_oneshot_regs_timed(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int stream_stores,
+                     const unsigned prefetch_blocks, unsigned long long* trace, const unsigned slot, const unsigned trace_blocks)
 {
-    oneshot_regs_body<N, C, DT, true>(p, count, ntiles, tv, mode, trace, slot, trace_blocks);
+    oneshot_regs_body<N, C, DT, true, false>(p, count, ntiles, tv, stream_stores, prefetch_blocks, trace, slot, trace_blocks);
 }
 
 // ---- one-shot allreduce, co-located group staged through shared memory ---------------------------------
@@ -1515,37 +1516,45 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
 // Two-shot without the intermediate: the block that reduces a tile stores it into all N destinations.
 // (A form that moves the tile through shared memory with bulk copies in both directions was measured too:
 // slower up to 4 MiB per rank -- 512 KiB: 3.2 vs 2.85 us -- and within 1.5 % beyond, so it was not kept.)
+// A tile is U rows of tv vectors; block, tile and prefetch as in k_oneshot_regs.
 template <int N, int U, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N * U))
-k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const int prefetch, const ParamPad<12>)
+k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int stream_stores,
+              const unsigned prefetch_blocks, const ParamPad<4>)
 {
     const size_t nvec = count / Elem<DT>::kElems;
-    if (prefetch && blockIdx.x < ntiles && threadIdx.x < N) {        // thread r: source r's slice of the first tile
-        const size_t i0 = (size_t)blockIdx.x * (size_t)(kThreads * U);
+    if (blockIdx.x < prefetch_blocks && blockIdx.x < ntiles && threadIdx.x < N) {        // thread r: source r's slice of the first tile
+        const size_t i0 = (size_t)blockIdx.x * (tv * U);
         const uint4* a = p.src[0];
 #pragma unroll
         for (int r = 1; r < N; ++r) if ((int)threadIdx.x == r) a = p.src[r];
-        if (i0 < nvec) prefetch_l2_bulk(a + i0, (unsigned)(nvec - i0 < (size_t)(kThreads * U) ? nvec - i0 : (size_t)(kThreads * U)) * 16u);
+        if (i0 < nvec) prefetch_l2_bulk(a + i0, (unsigned)(nvec - i0 < (size_t)(tv * U) ? nvec - i0 : (size_t)(tv * U)) * 16u);
     }
     pdl_wait();
     for (size_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const size_t base = tile * (size_t)(kThreads * U) + threadIdx.x;
+        const size_t base = tile * (tv * U) + threadIdx.x;
+        const size_t end = threadIdx.x < tv ? nvec : 0;
         uint4 v[U][N];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const size_t i = base + (size_t)u * kThreads;
-            if (i < nvec) {
+            const size_t i = base + (size_t)u * tv;
+            if (i < end) {
 #pragma unroll
                 for (int r = 0; r < N; ++r) v[u][r] = ld_src(p.src[r] + i);
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const size_t i = base + (size_t)u * kThreads;
-            if (i < nvec) {
+            const size_t i = base + (size_t)u * tv;
+            if (i < end) {
                 const uint4 o = fold_vectors<N, DT>(v[u]);
+                if (stream_stores) {
 #pragma unroll
-                for (int d = 0; d < N; ++d) st_stream(p.dst[d] + i, o);
+                    for (int d = 0; d < N; ++d) st_stream(p.dst[d] + i, o);
+                } else {
+#pragma unroll
+                    for (int d = 0; d < N; ++d) st_dst(p.dst[d] + i, o);
+                }
             }
         }
     }
