@@ -1156,8 +1156,9 @@ int nuna_allreduce_host(const void* const* src, void* const* dst, int nranks, si
     // and writes crossing the host link in both directions at once, no staging copies.  (Bringing the sources
     // in by copy engine in 1-16 pipelined chunks while the kernel stores straight into the host destinations
     // was measured slower at every size -- 8 x 512 KiB: 214-690 us against 174 us -- because each of the
-    // 8 x chunks asynchronous copies costs about 4 us of host time to enqueue.)
-    if (two_shot && (flags & NUNA_TWOSHOT_PUT)) {
+    // 8 x chunks asynchronous copies costs about 4 us of host time to enqueue.)  The one-shot without a placement of its
+    // own gives the same bits, so it goes the same way (8 x 12 KB: 77 us with staging copies, 17 in place).
+    if (two_shot ? (flags & NUNA_TWOSHOT_PUT) != 0u : (flags & NUNA_PLACE_MASK) != NUNA_PLACE_AWARE) {
         const void* msrc[NUNA_MAX_RANKS];
         void* mdst[NUNA_MAX_RANKS];
         bool mapped = true;
@@ -1174,10 +1175,11 @@ int nuna_allreduce_host(const void* const* src, void* const* dst, int nranks, si
             mdst[r] = ad.devicePointer;
         }
         if (mapped) {
-            // Few blocks: reads of host memory issued by many SMs at once get less out of the link than the same
-            // reads from a few (8 x 512 KiB: 134 us with 24 blocks, 166 us with one block per tile; 8 x 4 MiB: 859
-            // against 1084 us; swept over 2-48 blocks and both unroll factors).
-            st = launch_twoshot_put(c, make_ptrs(msrc, mdst, nranks), nranks, dtype, count, flags & ~NUNA_LAUNCH_PDL, c->stream, 24u);
+            // Few blocks: reads of host memory issued by many SMs at once get less out of the link than the same reads
+            // from a few, and twelve suffice to fill it (8 x 512 KiB: 166 us with one block per tile, 124.9 with 24 blocks,
+            // 122.8 with 12, 123.0 with 8; 8 x 64 KiB 31.6 with 24, 30.4 with 12; 2 x 2 MB 117.5 with 12, 130 with 8).
+            // What is left: either direction of the link alone takes 89 us of device time for 4 MiB.
+            st = launch_twoshot_put(c, make_ptrs(msrc, mdst, nranks), nranks, dtype, count, flags & ~NUNA_LAUNCH_PDL, c->stream, 12u);
             if (st != NUNA_OK) return st;
             return cudaStreamSynchronize(c->stream) == cudaSuccess ? NUNA_OK : NUNA_ERR_CUDA;
         }
