@@ -183,50 +183,34 @@ def ptr_table(bufs: Sequence):
     return tab
 
 
-# The collectives the native module calls, in its order.
+# The collectives the native module is pointed at, in its order.
 _COLLECTIVES = ("nuna_allreduce", "nuna_allreduce_oneshot", "nuna_allreduce_twoshot", "nuna_reduce_scatter", "nuna_allgather",
                 "nuna_alltoall")
-_ALLREDUCE, _ONESHOT, _TWOSHOT, _REDUCE_SCATTER, _ALLGATHER, _ALLTOALL = range(6)
+_native = None
 
 
 def _load_native():
-    """Loads the marshalling module and points it at the library; the module's functions replace the loaders below."""
-    global _collective, _twoshot_static, _host, _stream_handle
-    L = lib()
-    if not os.path.exists(_NATIVE_PATH):
-        raise RuntimeError(f"{_NATIVE_PATH} is missing: run `python -m paper_2608_00867_b200.build`")
-    import torch  # noqa: F401  (the module links against torch's libraries, which importing torch loads)
-    spec = importlib.util.spec_from_file_location(__package__ + "._nuna_py", _NATIVE_PATH)
-    m = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(m)
-    at = lambda name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value
-    m.bind(tuple(at(n) for n in _COLLECTIVES), at("nuna_allreduce_twoshot_static"), at("nuna_allreduce_host"), NunaError)
-    _collective, _twoshot_static, _host, _stream_handle = m.collective, m.twoshot_static, m.host, m.stream_handle
-
-
-# (index, src, dst, count, dtype, flags, stream, check, nranks) -> status; likewise the others
-def _collective(*args):
-    _load_native()
-    return _collective(*args)
-
-
-def _twoshot_static(*args):
-    _load_native()
-    return _twoshot_static(*args)
-
-
-def _host(*args):
-    _load_native()
-    return _host(*args)
-
-
-def _stream_handle(stream):
-    _load_native()
-    return _stream_handle(stream)
+    """Loads the marshalling module, points it at the library, and puts its functions, which have the same names and
+    signatures, in the place of this module's: a call then enters native code directly."""
+    global _native
+    if _native is None:
+        L = lib()
+        if not os.path.exists(_NATIVE_PATH):
+            raise RuntimeError(f"{_NATIVE_PATH} is missing: run `python -m paper_2608_00867_b200.build`")
+        import torch  # noqa: F401  (the module links against torch's libraries, which importing torch loads)
+        spec = importlib.util.spec_from_file_location(__package__ + "._nuna_py", _NATIVE_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        at = lambda name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value
+        m.bind(tuple(at(n) for n in _COLLECTIVES), at("nuna_allreduce_twoshot_static"), at("nuna_allreduce_host"), NunaError)
+        for name in _COLLECTIVES + ("nuna_allreduce_twoshot_static", "nuna_allreduce_host"):
+            globals()[name] = getattr(m, name)
+        _native = m
+    return _native
 
 
 def _stream(stream) -> Optional[int]:
-    return _stream_handle(stream) or None
+    return _load_native().stream_handle(stream) or None
 
 
 def _finish(status: int, what: str, check: bool) -> int:
@@ -244,27 +228,27 @@ def nuna_set_option(option: int, value: int, check: bool = True) -> int:
 
 
 def nuna_allreduce_oneshot(src, dst, count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective(_ONESHOT, src, dst, count, dtype, flags, stream, check, nranks)
+    return _load_native().nuna_allreduce_oneshot(src, dst, count, dtype, flags, stream, check, nranks)
 
 
 def nuna_allreduce(src, dst, count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective(_ALLREDUCE, src, dst, count, dtype, flags, stream, check, nranks)
+    return _load_native().nuna_allreduce(src, dst, count, dtype, flags, stream, check, nranks)
 
 
 def nuna_allreduce_twoshot(src, dst, count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective(_TWOSHOT, src, dst, count, dtype, flags, stream, check, nranks)
+    return _load_native().nuna_allreduce_twoshot(src, dst, count, dtype, flags, stream, check, nranks)
 
 
 def nuna_reduce_scatter(src, dst, shard_count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective(_REDUCE_SCATTER, src, dst, shard_count, dtype, flags, stream, check, nranks)
+    return _load_native().nuna_reduce_scatter(src, dst, shard_count, dtype, flags, stream, check, nranks)
 
 
 def nuna_allgather(src, dst, shard_count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective(_ALLGATHER, src, dst, shard_count, dtype, flags, stream, check, nranks)
+    return _load_native().nuna_allgather(src, dst, shard_count, dtype, flags, stream, check, nranks)
 
 
 def nuna_alltoall(src, dst, block_count, dtype=NUNA_BF16, flags=0, stream=None, check=True, nranks=None) -> int:
-    return _collective(_ALLTOALL, src, dst, block_count, dtype, flags, stream, check, nranks)
+    return _load_native().nuna_alltoall(src, dst, block_count, dtype, flags, stream, check, nranks)
 
 
 NUNA_STATIC_MAX_COUNT = 2 * 1024 * 1024
@@ -273,12 +257,12 @@ NUNA_STATIC_MAX_COUNT = 2 * 1024 * 1024
 def nuna_allreduce_twoshot_static(src, dst, count, dtype=NUNA_BF16, stream=None, check=True) -> int:
     """The two-shot allreduce that never allocates: its scratch is a fixed array inside the library
     (at most NUNA_STATIC_MAX_COUNT elements per rank).  For callers that cannot call cudaMalloc."""
-    return _twoshot_static(src, dst, count, dtype, stream, check)
+    return _load_native().nuna_allreduce_twoshot_static(src, dst, count, dtype, stream, check)
 
 
 def nuna_allreduce_host(src, dst, count, dtype=NUNA_BF16, flags=0, two_shot=False, check=True) -> int:
     """``src`` / ``dst``: host buffers (numpy arrays, CPU tensors or addresses)."""
-    return _host(src, dst, count, dtype, flags, two_shot, check)
+    return _load_native().nuna_allreduce_host(src, dst, count, dtype, flags, two_shot, check)
 
 
 def nuna_chain_create(src_sets, dst_sets, nnodes, count, dtype=NUNA_BF16, flags=0, two_shot=False, check=True):

@@ -18,7 +18,7 @@ namespace nuna {
 
 std::atomic<unsigned long long> g_launches{0};
 static std::mutex g_ctx_mutex;
-static Context* g_ctx[kMaxDevices] = {};
+static std::atomic<Context*> g_ctx[kMaxDevices];              // written under g_ctx_mutex
 
 static int static_status_read_and_clear(unsigned* out);     // the allocation-free entry point's status word (end of file)
 constexpr unsigned kMinFlagTileVec = 16;                    // smallest two-shot tile (vectors): 256 bytes of shard per flag
@@ -51,8 +51,9 @@ int get_context(Context** out)
 {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return NUNA_ERR_CUDA;
+    if ((*out = g_ctx[dev].load(std::memory_order_acquire)) != nullptr) return NUNA_OK;
     std::lock_guard<std::mutex> lock(g_ctx_mutex);
-    if (!g_ctx[dev]) {
+    if (!g_ctx[dev].load(std::memory_order_relaxed)) {
         Context* c = new Context();
         c->device = dev;
         cudaDeviceProp prop;
@@ -73,9 +74,9 @@ int get_context(Context** out)
         c->opt.ag_bulk_vecs = env_int("NUNA_AG_BULK_VECS", 0);
         c->opt.regs_vecs = env_int("NUNA_REGS_VECS", 0);
         c->opt.prefetch = env_int("NUNA_PREFETCH", 0);
-        g_ctx[dev] = c;
+        g_ctx[dev].store(c, std::memory_order_release);
     }
-    *out = g_ctx[dev];
+    *out = g_ctx[dev].load(std::memory_order_relaxed);
     return NUNA_OK;
 }
 
@@ -183,10 +184,8 @@ static int pick_unroll(const Options& o, int nranks)
 // Resident blocks per SM of a kernel, looked up once per device (the cache is one slot per device and
 // kernel instantiation; racing first calls compute the same value).
 template <typename K>
-static int occupancy(K kernel, std::atomic<int>* cache /* [kMaxDevices] */)
+static int occupancy(K kernel, int dev, std::atomic<int>* cache /* [kMaxDevices] */)
 {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
     int n = cache[dev].load(std::memory_order_relaxed);
     if (n == 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, 0) != cudaSuccess || n < 1) n = 1;
@@ -194,7 +193,7 @@ static int occupancy(K kernel, std::atomic<int>* cache /* [kMaxDevices] */)
     }
     return n;
 }
-#define NUNA_OCC(kernel) ([&]() { static std::atomic<int> cache_[kMaxDevices]; return occupancy(kernel, cache_); }())
+#define NUNA_OCC(kernel) ([&]() { static std::atomic<int> cache_[kMaxDevices]; return occupancy(kernel, c->device, cache_); }())
 
 // Grid size: `waves` x (SMs x resident blocks per SM), never more than the work items.  Streaming
 // kernels (two-shot put, reduce-scatter, allgather) run one item per block (waves = 0: no cap): leaving

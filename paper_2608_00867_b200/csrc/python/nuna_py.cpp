@@ -24,11 +24,23 @@ typedef int (*CollectiveFn)(const void* const*, void* const*, int, size_t, int, 
 typedef int (*StaticFn)(const void* const*, void* const*, int, size_t, int, void*);
 typedef int (*HostFn)(const void* const*, void* const*, int, size_t, int, unsigned, int);
 
-// Indices of `collective` (the order of _COLLECTIVES in binding.py).
+// The six collectives of one signature (the order of _COLLECTIVES in binding.py).
 constexpr int kCollectives = 6;
 CollectiveFn g_collective[kCollectives] = {};
 const char* const kNames[kCollectives] = {"nuna_allreduce", "nuna_allreduce_oneshot", "nuna_allreduce_twoshot",
                                           "nuna_reduce_scatter", "nuna_allgather", "nuna_alltoall"};
+// Argument names of the module's functions, interned, and how many of them a call has to give.
+struct Signature {
+    const char* text[8];
+    int n, required;
+    PyObject* name[8];
+};
+Signature g_count = {{"src", "dst", "count", "dtype", "flags", "stream", "check", "nranks"}, 8, 3, {}};
+Signature g_shard = {{"src", "dst", "shard_count", "dtype", "flags", "stream", "check", "nranks"}, 8, 3, {}};
+Signature g_block = {{"src", "dst", "block_count", "dtype", "flags", "stream", "check", "nranks"}, 8, 3, {}};
+Signature g_fixed = {{"src", "dst", "count", "dtype", "stream", "check"}, 6, 3, {}};
+Signature g_hosts = {{"src", "dst", "count", "dtype", "flags", "two_shot", "check"}, 7, 3, {}};
+const Signature* const kSignature[kCollectives] = {&g_count, &g_count, &g_count, &g_shard, &g_shard, &g_block};
 StaticFn g_static = nullptr;
 HostFn g_host = nullptr;
 PyObject* g_error = nullptr;               // binding.NunaError
@@ -165,71 +177,98 @@ PyObject* finish(int status, const char* what, PyObject* check)
     return PyLong_FromLong(status);
 }
 
-bool arity(Py_ssize_t got, Py_ssize_t want)
+// Sorts a call's arguments, positional and by name, into out[0 ... sig.n), null where none was given.
+bool arguments(const char* what, const Signature& sig, PyObject* const* args, Py_ssize_t npos, PyObject* kwnames, PyObject** out)
 {
-    if (got == want) return true;
-    PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, got);
-    return false;
+    if (npos > sig.n) {
+        PyErr_Format(PyExc_TypeError, "%s() takes at most %d arguments (%zd given)", what, sig.n, npos);
+        return false;
+    }
+    for (int i = 0; i < sig.n; ++i) out[i] = i < npos ? args[i] : nullptr;
+    for (Py_ssize_t k = 0, nkw = kwnames ? PyTuple_GET_SIZE(kwnames) : 0; k < nkw; ++k) {
+        PyObject* key = PyTuple_GET_ITEM(kwnames, k);
+        int at = 0;
+        while (at < sig.n && key != sig.name[at]) ++at;             // names in a call's source are interned
+        if (at == sig.n)
+            for (at = 0; at < sig.n && PyUnicode_Compare(key, sig.name[at]) != 0;) ++at;
+        if (at == sig.n || out[at]) {
+            PyErr_Format(PyExc_TypeError, at == sig.n ? "%s() got an unexpected keyword argument '%U'"
+                                                      : "%s() got multiple values for argument '%U'", what, key);
+            return false;
+        }
+        out[at] = args[npos + k];
+    }
+    for (int i = 0; i < sig.required; ++i)
+        if (!out[i]) {
+            PyErr_Format(PyExc_TypeError, "%s() missing required argument: '%s'", what, sig.text[i]);
+            return false;
+        }
+    return true;
 }
 
-// collective(index, src, dst, count, dtype, flags, stream, check, nranks)
-PyObject* collective(PyObject*, PyObject* const* a, Py_ssize_t nargs)
+bool to_u64_or(PyObject* x, unsigned long long fallback, unsigned long long* out)
 {
-    if (!arity(nargs, 9)) return nullptr;
-    const long op = PyLong_AsLong(a[0]);
-    if (op < 0 || op >= kCollectives || !g_collective[op]) {
-        if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, "bind() has not been called");
-        return nullptr;
-    }
+    if (x) return to_u64(x, out);
+    *out = fallback;
+    return true;
+}
+
+template <int kOp>
+PyObject* collective(PyObject*, PyObject* const* args, Py_ssize_t npos, PyObject* kwnames)
+{
+    PyObject* a[8];
+    if (!arguments(kNames[kOp], *kSignature[kOp], args, npos, kwnames, a)) return nullptr;
     Table src, dst;
     unsigned long long count, dtype, flags, nranks;
     void* stream;
-    if (!src.fill(a[1], false) || !dst.fill(a[2], false) || !to_u64(a[3], &count) || !to_u64(a[4], &dtype) || !to_u64(a[5], &flags) ||
-        !to_stream(a[6], &stream))
+    if (!src.fill(a[0], false) || !dst.fill(a[1], false) || !to_u64(a[2], &count) || !to_u64_or(a[3], NUNA_BF16, &dtype) ||
+        !to_u64_or(a[4], 0, &flags) || !to_stream(a[5] ? a[5] : Py_None, &stream))
         return nullptr;
     nranks = (unsigned long long)src.n;
-    if (a[8] != Py_None && !to_u64(a[8], &nranks)) return nullptr;
+    if (a[7] && a[7] != Py_None && !to_u64(a[7], &nranks)) return nullptr;
     int st;
     Py_BEGIN_ALLOW_THREADS
-    st = g_collective[op](src.p, dst.p, (int)nranks, (size_t)count, (int)dtype, (unsigned)flags, stream);
+    st = g_collective[kOp](src.p, dst.p, (int)nranks, (size_t)count, (int)dtype, (unsigned)flags, stream);
     Py_END_ALLOW_THREADS
-    return finish(st, kNames[op], a[7]);
+    return finish(st, kNames[kOp], a[6] ? a[6] : Py_True);
 }
 
-// twoshot_static(src, dst, count, dtype, stream, check)
-PyObject* twoshot_static(PyObject*, PyObject* const* a, Py_ssize_t nargs)
+PyObject* twoshot_static(PyObject*, PyObject* const* args, Py_ssize_t npos, PyObject* kwnames)
 {
-    if (!arity(nargs, 6)) return nullptr;
+    PyObject* a[8];
+    if (!arguments("nuna_allreduce_twoshot_static", g_fixed, args, npos, kwnames, a)) return nullptr;
     Table src, dst;
     unsigned long long count, dtype;
     void* stream;
-    if (!src.fill(a[0], false) || !dst.fill(a[1], false) || !to_u64(a[2], &count) || !to_u64(a[3], &dtype) || !to_stream(a[4], &stream))
+    if (!src.fill(a[0], false) || !dst.fill(a[1], false) || !to_u64(a[2], &count) || !to_u64_or(a[3], NUNA_BF16, &dtype) ||
+        !to_stream(a[4] ? a[4] : Py_None, &stream))
         return nullptr;
     int st;
     Py_BEGIN_ALLOW_THREADS
     st = g_static(src.p, dst.p, (int)src.n, (size_t)count, (int)dtype, stream);
     Py_END_ALLOW_THREADS
-    return finish(st, "nuna_allreduce_twoshot_static", a[5]);
+    return finish(st, "nuna_allreduce_twoshot_static", a[5] ? a[5] : Py_True);
 }
 
-// host(src, dst, count, dtype, flags, two_shot, check)
-PyObject* host(PyObject*, PyObject* const* a, Py_ssize_t nargs)
+PyObject* host(PyObject*, PyObject* const* args, Py_ssize_t npos, PyObject* kwnames)
 {
-    if (!arity(nargs, 7)) return nullptr;
+    PyObject* a[8];
+    if (!arguments("nuna_allreduce_host", g_hosts, args, npos, kwnames, a)) return nullptr;
     Table src, dst;
     unsigned long long count, dtype, flags;
-    if (!src.fill(a[0], true) || !dst.fill(a[1], true) || !to_u64(a[2], &count) || !to_u64(a[3], &dtype) || !to_u64(a[4], &flags))
+    if (!src.fill(a[0], true) || !dst.fill(a[1], true) || !to_u64(a[2], &count) || !to_u64_or(a[3], NUNA_BF16, &dtype) ||
+        !to_u64_or(a[4], 0, &flags))
         return nullptr;
-    const int two = PyObject_IsTrue(a[5]);
+    const int two = a[5] ? PyObject_IsTrue(a[5]) : 0;
     if (two < 0) return nullptr;
     int st;
     Py_BEGIN_ALLOW_THREADS
     st = g_host(src.p, dst.p, (int)src.n, (size_t)count, (int)dtype, (unsigned)flags, two);
     Py_END_ALLOW_THREADS
-    return finish(st, "nuna_allreduce_host", a[6]);
+    return finish(st, "nuna_allreduce_host", a[6] ? a[6] : Py_True);
 }
 
-// current_stream(stream) -> handle as an integer, the way `stream` arguments are read
+// stream_handle(stream) -> handle as an integer, the way `stream` arguments are read
 PyObject* stream_handle(PyObject*, PyObject* x)
 {
     void* s;
@@ -259,10 +298,20 @@ PyObject* bind(PyObject*, PyObject* args)
     Py_RETURN_NONE;
 }
 
+#define NUNA_KW(fn) (PyCFunction)(void (*)(void))(fn), METH_FASTCALL | METH_KEYWORDS
+#define NUNA_REST ", dtype=0, flags=0, stream=None, check=True, nranks=None)\n--\n\n"
+
 PyMethodDef methods[] = {
-    {"collective", (PyCFunction)(void (*)(void))collective, METH_FASTCALL, nullptr},
-    {"twoshot_static", (PyCFunction)(void (*)(void))twoshot_static, METH_FASTCALL, nullptr},
-    {"host", (PyCFunction)(void (*)(void))host, METH_FASTCALL, nullptr},
+    {"nuna_allreduce", NUNA_KW(collective<0>), "nuna_allreduce(src, dst, count" NUNA_REST},
+    {"nuna_allreduce_oneshot", NUNA_KW(collective<1>), "nuna_allreduce_oneshot(src, dst, count" NUNA_REST},
+    {"nuna_allreduce_twoshot", NUNA_KW(collective<2>), "nuna_allreduce_twoshot(src, dst, count" NUNA_REST},
+    {"nuna_reduce_scatter", NUNA_KW(collective<3>), "nuna_reduce_scatter(src, dst, shard_count" NUNA_REST},
+    {"nuna_allgather", NUNA_KW(collective<4>), "nuna_allgather(src, dst, shard_count" NUNA_REST},
+    {"nuna_alltoall", NUNA_KW(collective<5>), "nuna_alltoall(src, dst, block_count" NUNA_REST},
+    {"nuna_allreduce_twoshot_static", NUNA_KW(twoshot_static),
+     "nuna_allreduce_twoshot_static(src, dst, count, dtype=0, stream=None, check=True)\n--\n\n"},
+    {"nuna_allreduce_host", NUNA_KW(host),
+     "nuna_allreduce_host(src, dst, count, dtype=0, flags=0, two_shot=False, check=True)\n--\n\n"},
     {"stream_handle", (PyCFunction)stream_handle, METH_O, nullptr},
     {"bind", (PyCFunction)bind, METH_VARARGS, nullptr},
     {nullptr, nullptr, 0, nullptr}};
@@ -278,5 +327,7 @@ PyMODINIT_FUNC PyInit__nuna_py()
     g_s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
     g_s_ctypes = PyUnicode_InternFromString("ctypes");
     g_s_data = PyUnicode_InternFromString("data");
+    for (Signature* sig : {&g_count, &g_shard, &g_block, &g_fixed, &g_hosts})
+        for (int i = 0; i < sig->n; ++i) sig->name[i] = PyUnicode_InternFromString(sig->text[i]);
     return PyModule_Create(&module_def);
 }

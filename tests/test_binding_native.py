@@ -68,3 +68,22 @@ def test_numbers_streams_and_errors():
     for bad in ((src, None, 8), (src, [None, None], 8), (src, dst, 1.5), (src, dst, "8")):
         with pytest.raises(TypeError):
             nb.nuna_allreduce(*bad, stream=0)
+
+
+def test_arguments_by_name_and_position():
+    """The native functions take their place on the first call and keep the names, the order and the defaults."""
+    import inspect
+    src, dst = [A, A + 4096], [A + 8192, A + 12288]
+    for name, count in (("nuna_allreduce", "count"), ("nuna_reduce_scatter", "shard_count"), ("nuna_allgather", "shard_count"),
+                        ("nuna_alltoall", "block_count")):
+        call = getattr(nb, name)
+        call(src, dst, 0, stream=0)
+        native = getattr(nb, name)
+        assert list(inspect.signature(native).parameters) == ["src", "dst", count, "dtype", "flags", "stream", "check", "nranks"]
+        for f in (call, native):
+            assert f(src, dst, 8, 9, 0, 0, False, 2) == nb.NUNA_ERR_UNSUPPORTED_DTYPE
+            assert f(check=False, dst=dst, stream=0, src=src, dtype=9, **{count: 8}) == nb.NUNA_ERR_UNSUPPORTED_DTYPE
+            assert f(src, dst, 8, nb.NUNA_BF16, 3, stream=0, check=False) == nb.NUNA_ERR_INVALID_ARG
+            for args, kw in (((src, dst), {}), ((src, dst, 0), {"dst": dst}), ((src, dst, 0), {"nosuch": 1}), ((src,) * 9, {})):
+                with pytest.raises(TypeError):
+                    f(*args, **kw)
