@@ -747,14 +747,19 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
         // Tile bytes across all N sources, from a sweep at 8 ranks (16 ... 256 vectors per tile at every size):
         // small tiles while the message is small (more blocks, less latency per tile), 32 KiB once there are
         // plenty.  At 8 MiB of sources 16 KiB tiles make 1024 blocks for 592 resident ones and the second
-        // wave's consumers wait (10.3 us against 7.6 us with 12 KiB tiles), hence the step back there.
+        // wave's consumers wait (10.3 us against 7.6 us with 12 KiB tiles), hence the step back there.  From 10 ranks
+        // fewer blocks are resident, and larger tiles are ahead from 4 to 14 MiB (16 ranks x 320 KiB 6.3 us with 24 KiB
+        // tiles, 8.3 with 12; x 512 KiB 6.9 against 8.7; 12 x 400 KiB 6.1 against 7.9; 9 x 700 KiB 7.1 against 6.6).
         // Between 16 and 64 MiB of sources 24 KiB tiles with a lead of five blocks per SM are ahead (3 MiB per rank 11.6
         // against 12.3 us, 4 MiB 14.2 against 15.1, 6 MiB 19.1 against 21.3, 7 MiB 21.6 against 24.2; at 8 MiB 27.2
-        // against 24.8, hence the upper limit).
+        // against 24.8, hence the upper limit; a lead of four is 2 % faster at 4 MiB and 10 ... 30 % slower elsewhere).
         const size_t src_bytes = bytes * (size_t)nranks;
         mid_sized = nranks <= 8 && src_bytes > ((size_t)16 << 20) && src_bytes < ((size_t)64 << 20);   // 16 ranks: no gain
+        const bool many = nranks >= 10;
         const unsigned tile_src = src_bytes <= ((size_t)512 << 10) ? 4096u : src_bytes <= ((size_t)1 << 20) ? 8192u
-                                : src_bytes <= ((size_t)8 << 20) ? 12288u
+                                : src_bytes <= ((size_t)4 << 20) ? 12288u
+                                : src_bytes <= ((size_t)8 << 20) ? (many ? 24576u : 12288u)
+                                : src_bytes <= ((size_t)14 << 20) ? (many ? 32768u : 16384u)
                                 : src_bytes <= ((size_t)16 << 20) ? 16384u : mid_sized ? 24576u : 32768u;
         tv = tile_src / 16u / (unsigned)nranks;
     }
