@@ -89,13 +89,12 @@ typedef enum { NUNA_BF16 = 0, NUNA_F16 = 1, NUNA_F32 = 2 } nuna_dtype_t;   /* el
  * while its predecessor in the stream drains; it waits for that grid's completion and memory visibility before
  * its first global access, so results are those of an ordinary stream-ordered launch.  Collectives called outside
  * stream capture behave as if the flag were given; in a captured graph the edge is an ordinary one and the
- * kernel is chosen for it unless the flag is given.  The round-robin one-shot ignores it above 16 MiB of sources, where it was measured
- * not to pay.  Unless
- * NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot and of the put form (up to 64 MiB of
- * sources; beyond 8 MiB the first wave only), of the flag-synchronised two-shot and of the allgather and
- * alltoall (up to 128 MiB of sources; 8 MiB beyond 8 ranks) also asks L2, before that wait, to fetch its first tile of the sources (a prefetch returns
- * nothing to the kernel; L2 is the point of coherence, so what the predecessor still writes is what the
- * loads after the wait see).                                                                            */
+ * kernel is chosen for it unless the flag is given.  The round-robin one-shot ignores it above 16 MiB of sources,
+ * where it was measured not to pay.  Unless NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot
+ * and of the put form (up to 64 MiB of sources; beyond 8 MiB the first wave only), of the flag-synchronised
+ * two-shot and of the allgather and alltoall (up to 128 MiB of sources; 8 MiB beyond 8 ranks) also asks L2,
+ * before that wait, to fetch its first tile of the sources (a prefetch returns nothing to the kernel; L2 is the
+ * point of coherence, so what the predecessor still writes is what the loads after the wait see).          */
 #define NUNA_LAUNCH_PDL       64u
 /* `flags`, bit 7, with NUNA_PLACE_AWARE on nuna_allreduce_oneshot: dispatch the co-located groups through
  * per-SM work lists.  The lists are planned by Algorithm 1 from the topology the last
@@ -281,7 +280,8 @@ int nuna_init(size_t scratch_bytes);
  *                           into shared memory, one bulk store per destination; tile size by message size);
  *                           >= 8: the bulk-copy form with tiles of that many 16-byte vectors; 1: the register form
  *                           with full tiles (16-byte loads and stores by every thread)
- *  NUNA_OPT_REGS_VECS       16-byte vectors per source per tile of the NUNA_PLACE_REGS kernel (8 ... 256; 0 = by size)
+ *  NUNA_OPT_REGS_VECS       16-byte vectors per source per tile of the NUNA_PLACE_REGS kernel and of the put form
+ *                           (8 ... 256; 0 = by size)
  *  NUNA_OPT_PREFETCH        1: kernels launched with NUNA_LAUNCH_PDL do not ask L2 for their first tile ahead of the
  *                           wait for their predecessor (0 = they do, unless NUNA_HINT_RESIDENT is given); a
  *                           measurement aid, the prefetch changes no result

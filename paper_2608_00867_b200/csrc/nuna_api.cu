@@ -576,10 +576,11 @@ struct TileShape {
 // of 32 ... 256 threads, as dependent graph nodes (us at 8 ranks; u = vectors per source and SM; `ksplit` blocks share a
 // tile, each with a part of the destinations):
 // * u <= 56: one block per SM, tiles of 8 ... 56 vectors (8 KiB: 1.08 resident against 1.38 with eight full blocks).
-// * up to 8 MiB of sources: four blocks per SM, as many as stay resident, tiles of 56 ... 256 vectors (512 KiB cold: 2.1
+// * up to 6 MiB of sources: four blocks per SM, as many as stay resident, tiles of 56 ... 256 vectors (512 KiB cold: 2.1
 //   against 2.8 with full tiles; 16 ranks x 256 KiB, three blocks per SM: 3.46 with 586 blocks, 2.42 with 294).
-// * 8 to 16 MiB of sources, cold: eight blocks per SM, i.e. two waves, tiles from 112 vectors: the second wave's loads run
-//   beside the first one's stores (2 MiB 6.16 -> 5.4, 1.5 MiB 4.79 -> 4.2; 4 ranks x 4 MiB 5.87 -> 5.4).
+// * 6 to 16 MiB of sources, cold: eight blocks per SM, i.e. two waves, tiles from 112 vectors: the second wave's loads run
+//   beside the first one's stores (2 MiB 6.16 -> 5.4, 1.5 MiB 4.79 -> 4.2; 4 ranks x 4 MiB 5.87 -> 5.4; 4 ranks x 2 MB,
+//   three sets in turn: 3.6 with one full wave of 216 vectors, 2.6 with 112).
 // * 16 to 64 MiB, cold: tiles of 192 vectors (256 up to 4 ranks) in blocks of just so many threads, and only the first wave
 //   prefetches: later blocks would ask L2 for what they load at once (4 MiB 11.4 -> 11.0, 6 MiB 16.9 -> 16.1, 8 MiB
 //   21.5 -> 21.1; 4 ranks x 8 MiB 11.5 -> 10.9).
@@ -609,9 +610,10 @@ static TileShape tile_shape(const Context* c, const Options& o, int nranks, size
     }
     if (hot && units > sms * 448) return {128u, 128u, 0u};
     if (units <= sms * 56) return {clamp(tile_for(sms), 8), (unsigned)kThreads, everyone};
-    if (hot || total < ((size_t)8 << 20)) return {clamp(tile_for(sms * per_sm), 56), (unsigned)kThreads, everyone};
+    const unsigned four = clamp(tile_for(sms * per_sm), 56);
+    if (hot || total < ((size_t)6 << 20)) return {four, (unsigned)kThreads, everyone};
     if (total <= ((size_t)16 << 20))
-        return {clamp(tile_for(sms * 2 * per_sm), 112), (unsigned)kThreads, total <= ((size_t)8 << 20) ? everyone : first_wave};
+        return {std::min(four, clamp(tile_for(sms * 2 * per_sm), 112)), (unsigned)kThreads, total <= ((size_t)8 << 20) ? everyone : first_wave};
     if (total <= ((size_t)64 << 20)) {
         const unsigned tv = nranks <= 4 || nranks > 8 ? 256u : 192u;
         return {tv, tv, first_wave};

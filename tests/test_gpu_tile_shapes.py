@@ -1,5 +1,5 @@
 """The register-sharing one-shot, the put form and the size-selected allreduce on both sides of every line of the rule
-that chooses their tiles and blocks: vectors per SM (32, 56, 128, 448) and bytes of sources in total (8, 16, 64 MiB),
+that chooses their tiles and blocks: vectors per SM (32, 56, 128, 448) and bytes of sources in total (6, 8, 16, 64 MiB),
 one vector below, at and above it, with a ragged end.  Bit for bit against a rank-ordered binary32 fold in torch."""
 import pytest
 import torch
@@ -17,7 +17,7 @@ CALLS = {"regs": (nb.nuna_allreduce_oneshot, nb.NUNA_PLACE_AWARE | nb.NUNA_PLACE
 
 def vectors(n):
     per_sm = [SMS * u for u in (1, 16, 32, 56, 64, 128, 448)]
-    total = [(m << 20) // 16 // n for m in (8, 16, 64)]
+    total = [(m << 20) // 16 // n for m in (6, 8, 16, 64)]
     return sorted({v + d for v in per_sm + total for d in (-1, 0, 1)})
 
 
