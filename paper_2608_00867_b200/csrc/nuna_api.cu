@@ -1284,7 +1284,8 @@ int nuna_shutdown(void)
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return NUNA_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g_ctx_mutex);
-    Context* c = g_ctx[dev];
+    // out of the table first: a call that comes while this one waits for the device finds none, and waits for the lock
+    Context* c = g_ctx[dev].exchange(nullptr, std::memory_order_acq_rel);
     if (!c) return NUNA_OK;
     cudaDeviceSynchronize();
     if (c->bw) cudaFree(c->bw);
@@ -1295,7 +1296,6 @@ int nuna_shutdown(void)
     for (auto& kv : c->sm_plans) cudaFree(kv.second.base);
     for (unsigned* d : c->retired_plans) cudaFree(d);
     delete c;
-    g_ctx[dev] = nullptr;
     return NUNA_OK;
 }
 
