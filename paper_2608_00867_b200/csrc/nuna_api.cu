@@ -1002,6 +1002,33 @@ int launch_chain_persistent(Context* c, const ChainSets& sets, int nsets, int nn
 
 using namespace nuna;
 
+// The allreduce forms behind their argument checks; `flags` are the ones to run with.
+static int run_oneshot(const void* const* src, void* const* dst, int nranks, size_t count, int dtype, unsigned flags, void* stream)
+{
+    Context* c = nullptr;
+    const int st = get_context(&c);
+    if (st != NUNA_OK) return st;
+    return launch_oneshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, flags, (cudaStream_t)stream);
+}
+
+static int run_twoshot(const void* const* src, void* const* dst, int nranks, size_t count, int dtype, unsigned flags, void* stream)
+{
+    Context* c = nullptr;
+    int st = get_context(&c);
+    if (st != NUNA_OK) return st;
+    if (!(flags & NUNA_TWOSHOT_PUT)) {
+        std::lock_guard<std::mutex> lock(c->mutex);
+        const size_t need = (count * elem_size(dtype) + 15) & ~(size_t)15;
+        if (need > c->scratch_bytes || !c->scratch) {
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing((cudaStream_t)stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone)
+                return NUNA_ERR_CAPTURING;             // growing the scratch allocates: call nuna_init first
+            if ((st = ensure_scratch(c, need)) != NUNA_OK) return st;
+        }
+    }
+    return launch_twoshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, flags, (cudaStream_t)stream);
+}
+
 extern "C" {
 
 int nuna_init(size_t scratch_bytes)
@@ -1044,9 +1071,7 @@ int nuna_allreduce_oneshot(const void* const* src, void* const* dst, int nranks,
     int st = check_args(src, dst, nranks, count, count, dtype, flags & ~NUNA_TWOSHOT_PUT, true);
     if (st != NUNA_OK || count == 0) return st;
     if (flags & NUNA_TWOSHOT_PUT) return NUNA_ERR_INVALID_ARG;
-    Context* c = nullptr;
-    if ((st = get_context(&c)) != NUNA_OK) return st;
-    return launch_oneshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, effective_flags(flags, stream), (cudaStream_t)stream);
+    return run_oneshot(src, dst, nranks, count, dtype, effective_flags(flags, stream), stream);
 }
 
 int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks, size_t count, int dtype,
@@ -1055,24 +1080,15 @@ int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,
     if (has_chain_bits(flags)) return NUNA_ERR_INVALID_ARG;
     int st = check_args(src, dst, nranks, count, count, dtype, flags, true);
     if (st != NUNA_OK || count == 0) return st;
-    Context* c = nullptr;
-    if ((st = get_context(&c)) != NUNA_OK) return st;
-    if (!(flags & NUNA_TWOSHOT_PUT)) {
-        std::lock_guard<std::mutex> lock(c->mutex);
-        const size_t need = (count * elem_size(dtype) + 15) & ~(size_t)15;
-        if (need > c->scratch_bytes || !c->scratch) {
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing((cudaStream_t)stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone)
-                return NUNA_ERR_CAPTURING;             // growing the scratch allocates: call nuna_init first
-            if ((st = ensure_scratch(c, need)) != NUNA_OK) return st;
-        }
-    }
-    return launch_twoshot(c, make_ptrs(src, dst, nranks), nranks, dtype, count, effective_flags(flags, stream), (cudaStream_t)stream);
+    return run_twoshot(src, dst, nranks, count, dtype, effective_flags(flags, stream), stream);
 }
 
 int nuna_allreduce(const void* const* src, void* const* dst, int nranks, size_t count, int dtype, unsigned flags,
                    void* stream)
 {
+    if (has_chain_bits(flags)) return NUNA_ERR_INVALID_ARG;
+    const int st = check_args(src, dst, nranks, count, count, dtype, flags, true);
+    if (st != NUNA_OK || count == 0) return st;
     // Measured on B200 at 2, 3, 4, 6, 8 and 16 ranks, 8 KiB ... 64 MiB per rank, cold and L2-resident (us per graph node).
     // Without NUNA_PLACE_AUTO the one-shot is the round-robin kernel, whose re-reads cost more the more ranks there are.
     // Behind a dependent launch the put form is ahead of it (8 ranks x 8 KiB 1.14 against 1.29, x 1 MiB 3.14 against 4.92)
@@ -1100,8 +1116,8 @@ int nuna_allreduce(const void* const* src, void* const* dst, int nranks, size_t 
     } else {
         limit = nranks <= 2 ? ((size_t)1 << 20) : nranks <= 4 ? ((size_t)512 << 10) : nranks <= 8 ? ((size_t)64 << 10) : ((size_t)8 << 10);
     }
-    if (nranks <= 1 || bytes <= limit) return nuna_allreduce_oneshot(src, dst, nranks, count, dtype, base, stream);
-    return nuna_allreduce_twoshot(src, dst, nranks, count, dtype, sync_form ? base : (base | NUNA_TWOSHOT_PUT), stream);
+    if (nranks <= 1 || bytes <= limit) return run_oneshot(src, dst, nranks, count, dtype, base, stream);
+    return run_twoshot(src, dst, nranks, count, dtype, sync_form ? base : (base | NUNA_TWOSHOT_PUT), stream);
 }
 
 int nuna_reduce_scatter(const void* const* src, void* const* dst, int nranks, size_t shard_count, int dtype,

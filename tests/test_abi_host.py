@@ -80,6 +80,36 @@ def test_validation_happens_before_any_cuda_call():
     assert rs(ok_src, [A + 2048, A + 12288], 1024) == nb.NUNA_ERR_ALIAS        # src[0] spans 2*1024 elements
 
 
+NO_CUDA_CALL = """
+import ctypes, sys
+L = ctypes.CDLL(sys.argv[1])
+A, STALE = 1 << 20, 0x7F0000001000                # fake aligned addresses; a stream handle that is none any more
+good = (ctypes.c_void_p * 4)(A, A + 4096), (ctypes.c_void_p * 4)(A + 8192, A + 12288)
+odd = (ctypes.c_void_p * 2)(A + 2, A + 4096)
+for name in ("nuna_allreduce", "nuna_allreduce_oneshot", "nuna_allreduce_twoshot", "nuna_reduce_scatter", "nuna_allgather", "nuna_alltoall"):
+    f = getattr(L, name)
+    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_int, ctypes.c_uint, ctypes.c_void_p]
+    for flags in (0, 2, 1024):
+        assert f(*good, 2, 0, 0, flags, STALE) == 0, name
+        assert f(*good, 2, 8, 9, flags, STALE) == 2, name
+        assert f(odd, good[1], 2, 8, 0, flags, STALE) == 3, name
+        assert f(good[0], good[0], 2, 8, 0, flags, STALE) == 4, name
+        assert f(*good, 17, 8, 0, flags, STALE) == 8, name
+"""
+
+
+def test_refused_and_empty_calls_never_reach_the_driver(tmp_path):
+    """With a stand-in for the driver's library that reports being loaded, which the first CUDA runtime call does."""
+    import subprocess
+    import sys
+    (tmp_path / "f.c").write_text('#include <stdio.h>\n__attribute__((constructor)) static void up(void) { puts("driver loaded"); fflush(stdout); }')
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(tmp_path / "libcuda.so.1"), str(tmp_path / "f.c")], check=True)
+    run = subprocess.run([sys.executable, "-c", NO_CUDA_CALL, nb._LIB_PATH], capture_output=True, text=True,
+                         env={**os.environ, "LD_LIBRARY_PATH": str(tmp_path)})
+    assert run.returncode == 0, run.stderr
+    assert "driver loaded" not in run.stdout
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(nb, "_lib", None)
     monkeypatch.setattr(nb, "_LIB_PATH", "/nonexistent/libnuna.so")
