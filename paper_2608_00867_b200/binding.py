@@ -12,6 +12,8 @@ import importlib.util
 import os
 from typing import Optional, Sequence
 
+from . import build
+
 NUNA_OK = 0
 NUNA_ERR_INVALID_ARG = 1
 NUNA_ERR_UNSUPPORTED_DTYPE = 2
@@ -92,7 +94,6 @@ class NunaPlanInput(ctypes.Structure):
 
 
 _LIB_PATH = os.environ.get("NUNA_LIB") or os.path.join(os.path.dirname(os.path.abspath(__file__)), "libnuna.so")
-_NATIVE_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_nuna_py.so")
 _lib = None
 
 
@@ -195,10 +196,11 @@ def _load_native():
     global _native
     if _native is None:
         L = lib()
-        if not os.path.exists(_NATIVE_PATH):
-            raise RuntimeError(f"{_NATIVE_PATH} is missing: run `python -m paper_2608_00867_b200.build`")
+        path = build.native_path()
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: run `python -m paper_2608_00867_b200.build`")
         import torch  # noqa: F401  (the module links against torch's libraries, which importing torch loads)
-        spec = importlib.util.spec_from_file_location(__package__ + "._nuna_py", _NATIVE_PATH)
+        spec = importlib.util.spec_from_file_location(__package__ + "._nuna_py", path)
         m = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(m)
         at = lambda name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value

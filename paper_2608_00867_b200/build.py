@@ -1,10 +1,11 @@
 """Builds ``libnuna.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU) and, with the host compiler,
-``_nuna_py.so``, the native half of the Python binding."""
+``_nuna_py``, the native half of the Python binding."""
 from __future__ import annotations
 
 import glob
 import importlib.util
 import os
+import re
 import subprocess
 import sys
 import sysconfig
@@ -13,7 +14,20 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnuna.so")
 NATIVE_SRC = os.path.join(CSRC, "python", "nuna_py.cpp")
-NATIVE = os.path.join(HERE, "_nuna_py.so")
+
+
+def _torch_version() -> str:
+    """The installed torch's version, without importing it."""
+    path = os.path.join(os.path.dirname(importlib.util.find_spec("torch").origin), "version.py")
+    with open(path) as f:
+        return re.search(r"^__version__ = ['\"](.+)['\"]", f.read(), re.M).group(1)
+
+
+def native_path() -> str:
+    """Where the marshalling module for this Python and this torch is.  It is compiled against the insides of both, so a
+    module built for others has another name and is neither taken for up to date nor loaded."""
+    return os.path.join(HERE, f"_nuna_py.torch-{_torch_version()}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -54,8 +68,9 @@ def _compile(cmd, target: str, verbose: bool) -> None:
 
 def build_native(force: bool = False, verbose: bool = False) -> str:
     """The marshalling module: reads addresses and the current stream out of torch's own objects."""
-    if not force and not _older(NATIVE, [NATIVE_SRC] + _public_headers()):
-        return NATIVE
+    target = native_path()
+    if not force and not _older(target, [NATIVE_SRC] + _public_headers()):
+        return target
     torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
     inc = os.path.join(torch_dir, "include")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
@@ -63,8 +78,8 @@ def build_native(force: bool = False, verbose: bool = False) -> str:
     for d in (inc, os.path.join(inc, "torch", "csrc", "api", "include"), os.path.join(cuda, "include")):
         cmd += ["-isystem", d]
     cmd += [NATIVE_SRC, "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda"]
-    _compile(cmd, NATIVE, verbose)
-    return NATIVE
+    _compile(cmd, target, verbose)
+    return target
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -1,5 +1,7 @@
 """Argument marshalling of the native half of the binding: every form a rank buffer, a stream or a number may take.
 No GPU: the library's own argument checks tell what arrived (they run before any CUDA call)."""
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -87,3 +89,13 @@ def test_arguments_by_name_and_position():
             for args, kw in (((src, dst), {}), ((src, dst, 0), {"dst": dst}), ((src, dst, 0), {"nosuch": 1}), ((src,) * 9, {})):
                 with pytest.raises(TypeError):
                     f(*args, **kw)
+
+
+def test_a_module_built_for_another_torch_or_python_is_not_loaded(monkeypatch):
+    import sysconfig
+    assert torch.__version__ in os.path.basename(nbuild.native_path())
+    assert nbuild.native_path().endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    monkeypatch.setattr(nbuild, "_torch_version", lambda: "0.0.1")
+    monkeypatch.setattr(nb, "_native", None)
+    with pytest.raises(RuntimeError, match="torch-0.0.1.*is missing"):
+        nb._load_native()
