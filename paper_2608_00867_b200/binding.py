@@ -192,7 +192,8 @@ _native = None
 
 def _load_native():
     """Loads the marshalling module, points it at the library, and puts its functions, which have the same names and
-    signatures, in the place of this module's: a call then enters native code directly."""
+    signatures, in the place of this module's: a call then enters native code directly.  A function that the caller has
+    put in the place of one of them meanwhile stays."""
     global _native
     if _native is None:
         L = lib()
@@ -205,8 +206,9 @@ def _load_native():
         spec.loader.exec_module(m)
         at = lambda name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value
         m.bind(tuple(at(n) for n in _COLLECTIVES), at("nuna_allreduce_twoshot_static"), at("nuna_allreduce_host"), NunaError)
-        for name in _COLLECTIVES + ("nuna_allreduce_twoshot_static", "nuna_allreduce_host"):
-            globals()[name] = getattr(m, name)
+        for name, stand_in in _STAND_INS.items():
+            if globals()[name] is stand_in:
+                globals()[name] = getattr(m, name)
         _native = m
     return _native
 
@@ -265,6 +267,10 @@ def nuna_allreduce_twoshot_static(src, dst, count, dtype=NUNA_BF16, stream=None,
 def nuna_allreduce_host(src, dst, count, dtype=NUNA_BF16, flags=0, two_shot=False, check=True) -> int:
     """``src`` / ``dst``: host buffers (numpy arrays, CPU tensors or addresses)."""
     return _load_native().nuna_allreduce_host(src, dst, count, dtype, flags, two_shot, check)
+
+
+# This module's own functions that _load_native replaces.
+_STAND_INS = {name: globals()[name] for name in _COLLECTIVES + ("nuna_allreduce_twoshot_static", "nuna_allreduce_host")}
 
 
 def nuna_chain_create(src_sets, dst_sets, nnodes, count, dtype=NUNA_BF16, flags=0, two_shot=False, check=True):

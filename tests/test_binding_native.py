@@ -1,6 +1,8 @@
 """Argument marshalling of the native half of the binding: every form a rank buffer, a stream or a number may take.
 No GPU: the library's own argument checks tell what arrived (they run before any CUDA call)."""
 import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -99,3 +101,22 @@ def test_a_module_built_for_another_torch_or_python_is_not_loaded(monkeypatch):
     monkeypatch.setattr(nb, "_native", None)
     with pytest.raises(RuntimeError, match="torch-0.0.1.*is missing"):
         nb._load_native()
+
+
+def test_loading_the_native_module_keeps_what_the_caller_has_put_in_place():
+    code = """
+from paper_2608_00867_b200 import binding as nb
+own = nb.nuna_allreduce
+calls = []
+def traced(*a, **k):
+    calls.append(k["stream"])
+    return own(*a, **k)
+nb.nuna_allreduce = traced
+other = nb.nuna_alltoall
+src, dst = [1 << 20, (1 << 20) + 4096], [(1 << 20) + 8192, (1 << 20) + 12288]
+assert nb.nuna_alltoall(src, dst, 0, stream=0) == 0                  # loads the native module
+assert nb.nuna_alltoall is not other and nb.nuna_allreduce is traced
+assert nb.nuna_allreduce(src, dst, 0, stream=0) == 0 and calls == [0]
+"""
+    run = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(nb.__file__)), capture_output=True, text=True)
+    assert run.returncode == 0, run.stderr
