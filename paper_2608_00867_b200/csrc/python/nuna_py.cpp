@@ -15,6 +15,7 @@
 #include <cstdint>
 #include <exception>
 #include <memory>
+#include <new>
 
 #include "../../../include/nuna.h"
 
@@ -101,19 +102,27 @@ bool address_of(PyObject* x, bool host, void** out)
 
 // The addresses of a sequence of rank buffers.  The table has at least NUNA_MAX_RANKS entries, null beyond the
 // sequence, so that an explicit `nranks` larger than the sequence reads nulls (an argument error), not the stack.
+// It keeps the sequence until the call is made: an iterator's buffers may have no other owner.
 struct Table {
     void* fixed[NUNA_MAX_RANKS] = {};
     std::unique_ptr<void*[]> heap;
     void** p = fixed;
     Py_ssize_t n = 0;
+    PyObject* seq = nullptr;
+
+    ~Table() { Py_XDECREF(seq); }
 
     bool fill(PyObject* bufs, bool host)
     {
-        PyObject* seq = PySequence_Fast(bufs, "rank buffers must be a sequence");
+        seq = PySequence_Fast(bufs, "rank buffers must be a sequence");
         if (!seq) return false;
         n = PySequence_Fast_GET_SIZE(seq);
         if (n > NUNA_MAX_RANKS) {
-            heap.reset(new void*[(size_t)n]());
+            heap.reset(new (std::nothrow) void*[(size_t)n]());
+            if (!heap) {
+                PyErr_NoMemory();
+                return false;
+            }
             p = heap.get();
         }
         bool ok = true;
@@ -124,7 +133,6 @@ struct Table {
             ok = address_of(x, host, &p[i]);
             Py_DECREF(x);
         }
-        Py_DECREF(seq);
         return ok;
     }
 };

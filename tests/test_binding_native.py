@@ -3,6 +3,7 @@ No GPU: the library's own argument checks tell what arrived (they run before any
 import os
 import subprocess
 import sys
+import weakref
 
 import numpy as np
 import pytest
@@ -40,6 +41,24 @@ def test_table_forms(n, wrap):
     dst[-1] = Buf(2 * A + 64 * (n - 1) + 2)
     if n <= 16:                              # the last entry arrived: it is the misaligned one
         assert nb.nuna_allreduce(wrap(src), wrap(dst), 8, stream=0, check=False) == nb.NUNA_ERR_ALIGNMENT
+
+
+def test_buffers_of_an_iterator_live_until_the_call_is_made():
+    alive = []
+
+    class Watched(Buf):
+        def __init__(self, addr):
+            super().__init__(addr)
+            alive.append(weakref.ref(self))
+
+    class Last(Buf):                         # the last address that is read before the call
+        def data_ptr(self):
+            self.seen = [w() is not None for w in alive]
+            return self.addr
+
+    last = Last(2 * A + 64)
+    status = nb.nuna_allreduce((Watched(A + 64 * i) for i in range(2)), [2 * A, last], 8, dtype=9, stream=0, check=False)
+    assert status == nb.NUNA_ERR_UNSUPPORTED_DTYPE and last.seen == [True, True]
 
 
 @pytest.mark.parametrize("kind", [torch.Tensor, torch.nn.Parameter, Sub])
