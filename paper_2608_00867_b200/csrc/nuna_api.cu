@@ -3,6 +3,8 @@
 #include "nuna_debug.h"
 #include "nuna_kernels.cuh"
 
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
@@ -1002,6 +1004,38 @@ int launch_chain_persistent(Context* c, const ChainSets& sets, int nsets, int nn
 
 using namespace nuna;
 
+// The device address of `bytes` bytes of page-locked host memory, or null unless all of them are page-locked and the
+// device sees them in one piece.  The first byte does not speak for the rest: a program may have registered a part of
+// its buffer, or registered it in parts, so the ranges are followed to the end (one step for any single allocation).
+static void* mapped_host(const void* host, size_t bytes)
+{
+    typedef CUresult (*Attributes)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Attributes attributes = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) == cudaSuccess &&
+                        found == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<Attributes>(fn) : nullptr;
+    }();
+    if (!attributes) return nullptr;
+    uintptr_t first = 0;
+    for (size_t done = 0; done < bytes;) {
+        // one driver call for all of them: 16 buffers cost 1 us more with a call per attribute
+        unsigned type = 0, managed = 0;
+        CUdeviceptr at = 0, start = 0;
+        size_t size = 0;
+        CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                      CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+        void* to[] = {&type, &managed, &at, &start, &size};
+        if (attributes(5, what, to, (CUdeviceptr)(uintptr_t)host + done) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed || !at ||
+            (done && at != first + done) || start > at || start + size <= at)
+            return nullptr;
+        if (!done) first = at;
+        done += start + size - at;
+    }
+    return reinterpret_cast<void*>(first);
+}
+
 // The allreduce forms behind their argument checks; `flags` are the ones to run with.
 static int run_oneshot(const void* const* src, void* const* dst, int nranks, size_t count, int dtype, unsigned flags, void* stream)
 {
@@ -1190,16 +1224,9 @@ int nuna_allreduce_host(const void* const* src, void* const* dst, int nranks, si
         void* mdst[NUNA_MAX_RANKS];
         bool mapped = true;
         for (int r = 0; r < nranks && mapped; ++r) {
-            cudaPointerAttributes as, ad;
-            if (cudaPointerGetAttributes(&as, src[r]) != cudaSuccess || cudaPointerGetAttributes(&ad, dst[r]) != cudaSuccess) {
-                cudaGetLastError();
-                mapped = false;
-                break;
-            }
-            mapped = as.type == cudaMemoryTypeHost && ad.type == cudaMemoryTypeHost && as.devicePointer && ad.devicePointer &&
-                     (((uintptr_t)as.devicePointer | (uintptr_t)ad.devicePointer) & 15u) == 0;
-            msrc[r] = as.devicePointer;
-            mdst[r] = ad.devicePointer;
+            msrc[r] = mapped_host(src[r], bytes);
+            mdst[r] = mapped_host(dst[r], bytes);
+            mapped = msrc[r] && mdst[r] && (((uintptr_t)msrc[r] | (uintptr_t)mdst[r]) & 15u) == 0;
         }
         if (mapped) {
             // Few blocks: reads of host memory issued by many SMs at once get less out of the link than the same reads
@@ -1314,6 +1341,9 @@ int nuna_shutdown(void)
     delete c;
     return NUNA_OK;
 }
+
+// See nuna_debug.h.
+int nuna_debug_host_mapped(const void* host, size_t bytes) { return host && bytes && mapped_host(host, bytes) ? 1 : 0; }
 
 /* Test hook: the per-SM work lists planned for a one-shot of `ntiles` tiles under `topo` (NULL = no probe),
  * by the general planner (generic != 0) or the closed form.  off: [num_sms + 1], tiles: [ntiles].          */

@@ -54,6 +54,9 @@ int nuna_debug_oneshot_regs_traced(const void* const* src, void* const* dst, siz
  * for its own predecessor instead of after.                                                              */
 int nuna_debug_launch_floor(unsigned blocks, unsigned flags, int trigger_first, void* stream);
 
+/* 1 if a kernel may work on these bytes of host memory in place (nuna_allreduce_host): all of them are page-locked. */
+int nuna_debug_host_mapped(const void* host, size_t bytes);
+
 /* The probe's host-side clustering / verdict on a caller-supplied (num_sms x nlines) latency matrix.   */
 int nuna_debug_analyse_topology(const float* lat, const float* lat_rep, int num_sms, int nlines, nuna_topology_t* out);
 
