@@ -183,19 +183,20 @@ static int pick_unroll(const Options& o, int nranks)
     return u;
 }
 
-// Resident blocks per SM of a kernel, looked up once per device (the cache is one slot per device and
-// kernel instantiation; racing first calls compute the same value).
-template <typename K>
-static int occupancy(K kernel, int dev, std::atomic<int>* cache /* [kMaxDevices] */)
+// Resident blocks per SM of a kernel, looked up once per device (racing first calls compute the same value).  The kernel is
+// a template argument, so that the slot it is kept in belongs to that one instantiation: instantiations of one template
+// share their pointer's type but not their registers.
+template <auto kKernel>
+static int resident_blocks(const Context* c)
 {
-    int n = cache[dev].load(std::memory_order_relaxed);
+    static std::atomic<int> cache[kMaxDevices];
+    int n = cache[c->device].load(std::memory_order_relaxed);
     if (n == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, 0) != cudaSuccess || n < 1) n = 1;
-        cache[dev].store(n, std::memory_order_relaxed);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kKernel, kThreads, 0) != cudaSuccess || n < 1) n = 1;
+        cache[c->device].store(n, std::memory_order_relaxed);
     }
     return n;
 }
-#define NUNA_OCC(kernel) ([&]() { static std::atomic<int> cache_[kMaxDevices]; return occupancy(kernel, c->device, cache_); }())
 
 // Grid size: `waves` x (SMs x resident blocks per SM), never more than the work items.  Streaming
 // kernels (two-shot put, reduce-scatter, allgather) run one item per block (waves = 0: no cap): leaving
@@ -532,14 +533,14 @@ int prepare_oneshot(Context* c, int nranks, int dtype, size_t count, unsigned fl
 template <int N, int C, int DT>
 static int launch_sm_lists(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned mode, cudaStream_t stream)
 {
-    auto k = k_oneshot_sm<N, C, DT, false>;
+    constexpr auto k = k_oneshot_sm<N, C, DT, false>;
     SmPlan pl;
     const int st = get_sm_plan(c, N, count / Elem<DT>::kElems, C, o.domains, stream, &pl);
     if (st != NUNA_OK) return st;
     SmLists sl;
     sl.off = pl.off; sl.tiles = pl.tiles; sl.cursor = pl.cursor; sl.present = pl.present; sl.ctl = pl.ctl;
     sl.nonempty = pl.nonempty; sl.num_sms = c->num_sms;
-    const size_t cap = (size_t)c->num_sms * (size_t)NUNA_OCC(k);
+    const size_t cap = (size_t)c->num_sms * (size_t)resident_blocks<k>(c);
     const unsigned grid = (unsigned)std::min(cap, std::max<size_t>((size_t)c->num_sms, (size_t)pl.total));
     const unsigned blocks_per_sm = (unsigned)std::max<size_t>(1, grid / (size_t)c->num_sms);
     return launch(k, grid, stream, mode, p, count, sl, blocks_per_sm, (unsigned*)nullptr);
@@ -560,11 +561,11 @@ static int launch_cluster(const Options& o, const RankPtrs& p, size_t count, uns
 template <int N, int C, int DT>
 static int launch_group(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned mode, cudaStream_t stream)
 {
-    auto k = k_oneshot_group<N, C, DT>;
+    constexpr auto k = k_oneshot_group<N, C, DT>;
     const size_t nvec = count / Elem<DT>::kElems;
     const size_t ntiles = ceil_div(nvec, (size_t)(kThreads / C));
     const size_t nitems = std::max<size_t>(ntiles * ((N + C - 1) / C), (count % Elem<DT>::kElems) ? (size_t)N : 0);
-    const unsigned grid = pick_grid(c, o, nitems, NUNA_OCC(k));
+    const unsigned grid = pick_grid(c, o, nitems, resident_blocks<k>(c));
     return launch(k, grid, stream, mode, p, count, ntiles);
 }
 
@@ -623,22 +624,27 @@ static TileShape tile_shape(const Context* c, const Options& o, int nranks, size
     return {nranks <= 4 || nranks > 8 ? 256u : 128u, (unsigned)kThreads, 0u};
 }
 
+template <auto kKernel, int N, int C, int DT>
+static int launch_regs_as(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned flags, unsigned mode, cudaStream_t stream)
+{
+    constexpr int kSplit = (N + C - 1) / C;
+    const size_t nvec = count / Elem<DT>::kElems;
+    const TileShape t = tile_shape(c, o, N, nvec, kSplit, resident_blocks<kKernel>(c), flags, mode == kLaunchPdl);
+    const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
+    const size_t nitems = std::max<size_t>(ntiles * kSplit, (count % Elem<DT>::kElems) ? (size_t)N : 0);
+    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), 0, 0);
+    t_block = t.threads;
+    return launch_padded(kKernel, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
+}
+
 template <int N, int C, int DT>
 static int launch_regs(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned flags, unsigned mode, cudaStream_t stream)
 {
-    constexpr int kSplit = (N + C - 1) / C;
-    auto k = k_oneshot_regs<N, C, DT, false>;
     // L2-resident sources from 8 ranks, where the fewer instructions show (8 ranks x 16 KiB 1.04 -> 1.00 us per node, x 64 KiB
     // 1.08 -> 1.07; below, the general form measured 2 % faster)
-    if constexpr (kSplit == 1 && N >= 8)
-        if (flags & NUNA_HINT_RESIDENT) k = k_oneshot_regs<N, C, DT, true>;
-    const size_t nvec = count / Elem<DT>::kElems;
-    const TileShape t = tile_shape(c, o, N, nvec, kSplit, NUNA_OCC(k), flags, mode == kLaunchPdl);
-    const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
-    const size_t nitems = std::max<size_t>(ntiles * kSplit, (count % Elem<DT>::kElems) ? (size_t)N : 0);
-    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), NUNA_OCC(k), 0);
-    t_block = t.threads;
-    return launch_padded(k, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
+    if constexpr (N <= C && N >= 8)
+        if (flags & NUNA_HINT_RESIDENT) return launch_regs_as<k_oneshot_regs<N, C, DT, true>, N, C, DT>(c, o, p, count, flags, mode, stream);
+    return launch_regs_as<k_oneshot_regs<N, C, DT, false>, N, C, DT>(c, o, p, count, flags, mode, stream);
 }
 
 // Staged group kernel: one tile per block.  Tile size (vectors per source): large enough that a tile's
@@ -728,11 +734,11 @@ int launch_oneshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t 
     }
     return dispatch(nranks, pick_unroll(o, nranks), dtype, [&](auto n_, auto u_, auto d_) -> int {
         NUNA_NUD(n_, u_, d_);
-        auto k = k_oneshot_rr<N, U, DT>;
+        constexpr auto k = k_oneshot_rr<N, U, DT>;
         const size_t ntiles = ceil_div(nvec, (size_t)kThreads * U);
         const size_t nitems = std::max<size_t>(ntiles * N, (count % epv) ? (size_t)N : 0);
         // one resident wave while the message is small enough for latency to matter, four beyond
-        const unsigned grid = pick_grid(c, o, nitems, NUNA_OCC(k), bytes >= ((size_t)8 << 20) ? 4 : 1);
+        const unsigned grid = pick_grid(c, o, nitems, resident_blocks<k>(c), bytes >= ((size_t)8 << 20) ? 4 : 1);
         return launch_padded(k, grid, stream, mode, p, count, ntiles);
     });
 }
@@ -806,12 +812,12 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
     const size_t nvec = count / elems_per_vec(dtype);
     return dispatch(nranks, pick_unroll(o, nranks), dtype, [&](auto n_, auto u_, auto d_) -> int {
         NUNA_NUD(n_, u_, d_);
-        auto k = k_twoshot_put<N, U, DT>;
+        constexpr auto k = k_twoshot_put<N, U, DT>;
         // host-memory sources (max_blocks > 0) are read through the link, not through L2: no prefetch, full tiles
         TileShape t = max_blocks > 0 ? TileShape{(unsigned)kThreads, (unsigned)kThreads, 0u}
-                                     : tile_shape(c, o, nranks, nvec, 1, NUNA_OCC(k), flags, mode == kLaunchPdl);
+                                     : tile_shape(c, o, nranks, nvec, 1, resident_blocks<k>(c), flags, mode == kLaunchPdl);
         const size_t ntiles = ceil_div(nvec, (size_t)t.tv * U);
-        unsigned grid = pick_grid(c, o, std::max<size_t>(ntiles, 1), NUNA_OCC(k), 0);
+        unsigned grid = pick_grid(c, o, std::max<size_t>(ntiles, 1), resident_blocks<k>(c), 0);
         if (max_blocks > 0 && o.blocks <= 0) grid = std::min(grid, max_blocks);
         t_block = t.threads;
         return launch_padded(k, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
@@ -845,16 +851,16 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
         const size_t tiles = std::max<size_t>(1, ceil_div(shard / epv, (size_t)kRaggedTile));
         return dispatch(nranks, 1, dtype, [&](auto n_, auto u_, auto d_) -> int {
             NUNA_NUD(n_, u_, d_);
-            auto k = k_reduce_scatter_ragged<N, DT>;
-            return launch_padded(k, pick_grid(c, o, (tiles + 1) * N, NUNA_OCC(k), 0), stream, mode, p, shard, tiles);
+            constexpr auto k = k_reduce_scatter_ragged<N, DT>;
+            return launch_padded(k, pick_grid(c, o, (tiles + 1) * N, resident_blocks<k>(c), 0), stream, mode, p, shard, tiles);
         });
     }
     const size_t shard_vec = shard / epv;
     return dispatch(nranks, pick_unroll(o, nranks), dtype, [&](auto n_, auto u_, auto d_) -> int {
         NUNA_NUD(n_, u_, d_);
-        auto k = k_reduce_scatter<N, U, DT>;
+        constexpr auto k = k_reduce_scatter<N, U, DT>;
         const size_t tiles = ceil_div(shard_vec, (size_t)kThreads * U);
-        const unsigned grid = pick_grid(c, o, tiles * N, NUNA_OCC(k), 0);
+        const unsigned grid = pick_grid(c, o, tiles * N, resident_blocks<k>(c), 0);
         return launch_padded(k, grid, stream, mode, p, shard_vec, tiles);
     });
 }
@@ -908,9 +914,9 @@ int launch_allgather(Context* c, const RankPtrs& p, int nranks, size_t shard_byt
     // 5.4 us with 8): the stores, not the block count, are the limit.
     constexpr int U = 2;
     const int dsplit = 1;
-    auto k = k_allgather<U>;
+    constexpr auto k = k_allgather<U>;
     const size_t tiles = ceil_div(shard_vec, (size_t)kThreads * U);
-    const unsigned grid = pick_grid(c, o, tiles * nranks * dsplit, NUNA_OCC(k), 0);
+    const unsigned grid = pick_grid(c, o, tiles * nranks * dsplit, resident_blocks<k>(c), 0);
     return launch(k, grid, stream, mode, p, nranks, shard_vec, tiles, dsplit);
 }
 
@@ -939,9 +945,9 @@ int launch_alltoall(Context* c, const RankPtrs& p, int nranks, size_t block_byte
         }
     }
     constexpr int U = 2;
-    auto k = k_alltoall<U>;
+    constexpr auto k = k_alltoall<U>;
     const size_t tiles = ceil_div(block_vec, (size_t)kThreads * U);
-    const unsigned grid = pick_grid(c, o, tiles * nranks * nranks, NUNA_OCC(k), 0);
+    const unsigned grid = pick_grid(c, o, tiles * nranks * nranks, resident_blocks<k>(c), 0);
     return launch(k, grid, stream, mode, p, nranks, block_vec, tiles);
 }
 
@@ -1402,22 +1408,22 @@ int nuna_debug_access_latency(const void* const* src, void* const* dst, size_t c
     if (cudaMalloc(&d_hist, kLatBins * sizeof(unsigned)) != cudaSuccess) return NUNA_ERR_CUDA;
     cudaMemset(d_hist, 0, kLatBins * sizeof(unsigned));
     if (placement == 0) {
-        auto k = k_latency_rr<N, kBf16>;
+        constexpr auto k = k_latency_rr<N, kBf16>;
         const size_t ntiles = ceil_div(nvec, (size_t)kThreads);
-        st = launch(k, pick_grid(c, o, ntiles * N, NUNA_OCC(k)), (cudaStream_t)0, kLaunchPlain, p, count, ntiles, d_hist);
+        st = launch(k, pick_grid(c, o, ntiles * N, resident_blocks<k>(c)), (cudaStream_t)0, kLaunchPlain, p, count, ntiles, d_hist);
     } else if (placement == 1) {
-        auto k = k_latency_group<N, 8, kBf16>;
+        constexpr auto k = k_latency_group<N, 8, kBf16>;
         const size_t ntiles = ceil_div(nvec, (size_t)(kThreads / 8));
-        st = launch(k, pick_grid(c, o, ntiles, NUNA_OCC(k)), (cudaStream_t)0, kLaunchPlain, p, count, ntiles, d_hist);
+        st = launch(k, pick_grid(c, o, ntiles, resident_blocks<k>(c)), (cudaStream_t)0, kLaunchPlain, p, count, ntiles, d_hist);
     } else {
-        auto k = k_oneshot_sm<N, 8, kBf16, true>;
+        constexpr auto k = k_oneshot_sm<N, 8, kBf16, true>;
         SmPlan pl;
         st = get_sm_plan(c, N, nvec, 8, o.domains, (cudaStream_t)0, &pl);
         if (st == NUNA_OK) {
             SmLists sl;
             sl.off = pl.off; sl.tiles = pl.tiles; sl.cursor = pl.cursor; sl.present = pl.present; sl.ctl = pl.ctl;
             sl.nonempty = pl.nonempty; sl.num_sms = c->num_sms;
-            const size_t cap = (size_t)c->num_sms * (size_t)NUNA_OCC(k);
+            const size_t cap = (size_t)c->num_sms * (size_t)resident_blocks<k>(c);
             const unsigned grid = (unsigned)std::min(cap, std::max<size_t>((size_t)c->num_sms, (size_t)pl.total));
             st = launch(k, grid, (cudaStream_t)0, kLaunchPlain, p, count, sl,
                         (unsigned)std::max<size_t>(1, grid / (size_t)c->num_sms), d_hist);
@@ -1443,13 +1449,13 @@ int nuna_debug_oneshot_regs_traced(const void* const* src, void* const* dst, siz
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
     const Options o = snapshot(c);
-    auto k = k_oneshot_regs_timed<N, 8, kBf16>;
+    constexpr auto k = k_oneshot_regs_timed<N, 8, kBf16>;
     const size_t nvec = count / 8;
     const unsigned mode = (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchPlain;
-    const TileShape t = tile_shape(c, o, N, nvec, 1, NUNA_OCC(k), flags, mode == kLaunchPdl);
+    const TileShape t = tile_shape(c, o, N, nvec, 1, resident_blocks<k>(c), flags, mode == kLaunchPdl);
     const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
     const size_t nitems = std::max<size_t>(ntiles, (count % 8) ? (size_t)N : 0);
-    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), NUNA_OCC(k), 0);
+    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), resident_blocks<k>(c), 0);
     if (grid_blocks) *grid_blocks = grid;
     t_block = t.threads;
     return launch(k, grid, (cudaStream_t)stream, mode, make_ptrs(src, dst, N), count, ntiles, t.tv,
