@@ -624,27 +624,37 @@ static TileShape tile_shape(const Context* c, const Options& o, int nranks, size
     return {nranks <= 4 || nranks > 8 ? 256u : 128u, (unsigned)kThreads, 0u};
 }
 
-template <auto kKernel, int N, int C, int DT>
-static int launch_regs_as(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned flags, unsigned mode, cudaStream_t stream)
+// Whether a kernel runs its form without the tile loop, which wants a block per item (us per node, looping | once):
+// * cold, up to 4 ranks, at every size (2 x 64 KiB 0.999 | 0.947, 4 x 512 KiB 1.845 | 1.787, 3 x 4 MiB 4.39 | 4.32); beyond, the
+//   loop is ahead (8 x 64 KiB 1.358 | 1.398, 16 x 256 KiB 2.38 | 3.61: every block pays for the longer text of more ranks).
+// * L2-resident, where the text is shorter, with one block per SM or fewer (u <= 128) at every rank count, and up to 8 ranks with
+//   blocks as wide as their tiles (u > 448) again; between the two the loop is 1 ... 2 % ahead (8 x 384 KiB 1.505 | 1.55).
+static bool runs_once(const Context* c, int nranks, size_t units, unsigned flags)
 {
-    constexpr int kSplit = (N + C - 1) / C;
-    const size_t nvec = count / Elem<DT>::kElems;
-    const TileShape t = tile_shape(c, o, N, nvec, kSplit, resident_blocks<kKernel>(c), flags, mode == kLaunchPdl);
-    const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
-    const size_t nitems = std::max<size_t>(ntiles * kSplit, (count % Elem<DT>::kElems) ? (size_t)N : 0);
-    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), 0, 0);
-    t_block = t.threads;
-    return launch_padded(kKernel, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
+    const size_t sms = (size_t)c->num_sms;
+    if (!(flags & NUNA_HINT_RESIDENT)) return nranks <= 4;
+    return units <= sms * 128 || (units > sms * 448 && nranks <= 8);
 }
 
 template <int N, int C, int DT>
 static int launch_regs(Context* c, const Options& o, const RankPtrs& p, size_t count, unsigned flags, unsigned mode, cudaStream_t stream)
 {
-    // L2-resident sources from 8 ranks, where the fewer instructions show (8 ranks x 16 KiB 1.04 -> 1.00 us per node, x 64 KiB
-    // 1.08 -> 1.07; below, the general form measured 2 % faster)
-    if constexpr (N <= C && N >= 8)
-        if (flags & NUNA_HINT_RESIDENT) return launch_regs_as<k_oneshot_regs<N, C, DT, true>, N, C, DT>(c, o, p, count, flags, mode, stream);
-    return launch_regs_as<k_oneshot_regs<N, C, DT, false>, N, C, DT>(c, o, p, count, flags, mode, stream);
+    constexpr int kSplit = (N + C - 1) / C;
+    constexpr auto looping = k_oneshot_regs<N, C, DT, false, false>;
+    const bool hot = (flags & NUNA_HINT_RESIDENT) != 0u;
+    const size_t nvec = count / Elem<DT>::kElems;
+    const TileShape t = tile_shape(c, o, N, nvec, kSplit, resident_blocks<looping>(c), flags, mode == kLaunchPdl);
+    const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
+    const size_t nitems = std::max<size_t>(ntiles * kSplit, (count % Elem<DT>::kElems) ? (size_t)N : 0);
+    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), 0, 0);
+    const bool once = grid >= nitems && runs_once(c, N, nvec * kSplit, flags);
+    const auto go = [&](auto kernel) { return launch_padded(kernel, grid, stream, mode, p, count, ntiles, t.tv, hot ? 0 : 1, t.prefetch_blocks); };
+    t_block = t.threads;
+    if constexpr (kSplit == 1) { if (hot && once) return go(k_oneshot_regs<N, C, DT, true, true>); }
+    // 8 ranks x 512 KiB 1.745 -> 1.705 us; below 8 ranks it is up to 2 % slower than the general form
+    if constexpr (kSplit == 1 && N >= 8) { if (hot) return go(k_oneshot_regs<N, C, DT, false, true>); }
+    if constexpr (N <= 4) { if (!hot && once) return go(k_oneshot_regs<N, C, DT, true, false>); }
+    return go(looping);
 }
 
 // Staged group kernel: one tile per block.  Tile size (vectors per source): large enough that a tile's
@@ -812,15 +822,19 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
     const size_t nvec = count / elems_per_vec(dtype);
     return dispatch(nranks, pick_unroll(o, nranks), dtype, [&](auto n_, auto u_, auto d_) -> int {
         NUNA_NUD(n_, u_, d_);
-        constexpr auto k = k_twoshot_put<N, U, DT>;
+        constexpr auto looping = k_twoshot_put<N, U, DT, false>;
         // host-memory sources (max_blocks > 0) are read through the link, not through L2: no prefetch, full tiles
-        TileShape t = max_blocks > 0 ? TileShape{(unsigned)kThreads, (unsigned)kThreads, 0u}
-                                     : tile_shape(c, o, nranks, nvec, 1, resident_blocks<k>(c), flags, mode == kLaunchPdl);
+        const TileShape t = max_blocks > 0 ? TileShape{(unsigned)kThreads, (unsigned)kThreads, 0u}
+                                           : tile_shape(c, o, nranks, nvec, 1, resident_blocks<looping>(c), flags, mode == kLaunchPdl);
         const size_t ntiles = ceil_div(nvec, (size_t)t.tv * U);
-        unsigned grid = pick_grid(c, o, std::max<size_t>(ntiles, 1), resident_blocks<k>(c), 0);
+        unsigned grid = pick_grid(c, o, std::max<size_t>(ntiles, 1), 0, 0);
         if (max_blocks > 0 && o.blocks <= 0) grid = std::min(grid, max_blocks);
+        const auto go = [&](auto kernel) {
+            return launch_padded(kernel, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
+        };
         t_block = t.threads;
-        return launch_padded(k, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
+        if constexpr (U == 1) { if (grid >= ntiles && runs_once(c, N, nvec, flags)) return go(k_twoshot_put<N, U, DT, true>); }
+        return go(looping);
     });
 }
 
@@ -1438,7 +1452,7 @@ int nuna_debug_access_latency(const void* const* src, void* const* dst, size_t c
     return st;
 }
 
-// See nuna_debug.h.  The same tile size, grid and mode bits as launch_regs<8, 8, bf16>.
+// See nuna_debug.h.  The same tile size, grid and form of the kernel as launch_regs<8, 8, bf16>.
 int nuna_debug_oneshot_regs_traced(const void* const* src, void* const* dst, size_t count, unsigned flags, unsigned slot,
                                    unsigned long long* trace, unsigned* grid_blocks, void* stream)
 {
@@ -1449,17 +1463,21 @@ int nuna_debug_oneshot_regs_traced(const void* const* src, void* const* dst, siz
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
     const Options o = snapshot(c);
-    constexpr auto k = k_oneshot_regs_timed<N, 8, kBf16>;
+    constexpr auto looping = k_oneshot_regs<N, 8, kBf16, false, false>;
+    const bool hot = (flags & NUNA_HINT_RESIDENT) != 0u;
     const size_t nvec = count / 8;
-    const unsigned mode = (flags & NUNA_LAUNCH_PDL) ? kLaunchPdl : kLaunchPlain;
-    const TileShape t = tile_shape(c, o, N, nvec, 1, resident_blocks<k>(c), flags, mode == kLaunchPdl);
+    const unsigned mode = launch_mode(flags);
+    const TileShape t = tile_shape(c, o, N, nvec, 1, resident_blocks<looping>(c), flags, mode == kLaunchPdl);
     const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
     const size_t nitems = std::max<size_t>(ntiles, (count % 8) ? (size_t)N : 0);
-    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), resident_blocks<k>(c), 0);
+    const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), 0, 0);
     if (grid_blocks) *grid_blocks = grid;
     t_block = t.threads;
-    return launch(k, grid, (cudaStream_t)stream, mode, make_ptrs(src, dst, N), count, ntiles, t.tv,
-                  (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks, trace, slot, (unsigned)NUNA_DEBUG_TRACE_BLOCKS);
+    const bool once = hot && grid >= nitems && runs_once(c, N, nvec, flags);
+    const auto k = once ? k_oneshot_regs_timed<N, 8, kBf16, true, true> : hot ? k_oneshot_regs_timed<N, 8, kBf16, false, true>
+                                                                             : k_oneshot_regs_timed<N, 8, kBf16, false, false>;
+    return launch(k, grid, (cudaStream_t)stream, mode, make_ptrs(src, dst, N), count, ntiles, t.tv, hot ? 0 : 1,
+                  t.prefetch_blocks, trace, slot, (unsigned)NUNA_DEBUG_TRACE_BLOCKS);
 }
 
 /* Test hook: a flag-synchronised two-shot whose consumers wait for a flag value that nobody publishes

@@ -490,11 +490,14 @@ __device__ __forceinline__ uint4 fold_vectors_own(const uint4 (&v)[N])
 // The block has 32 ... kThreads threads, at least tv.  stream_stores: destinations are not re-read soon.  The first
 // prefetch_blocks blocks ask L2 for their first tile's source slices before they wait for the predecessor kernel
 // (dependent launches with cold sources only: without a predecessor there is nothing to overlap with).
-// kHot: L2-resident sources, i.e. stream_stores = prefetch_blocks = 0 known at compile time.
+// kOnce: the grid has a block per item.  Without the loop there is less between the wait and the first load, and a node of
+// about 1 us shows it (us, L2-resident, looping | once: 2 ranks x 64 KiB 0.976 | 0.910, 4 ranks 1.018 | 0.949, 8 ranks 1.082 |
+// 1.011).  kHot: L2-resident sources, i.e. stream_stores = prefetch_blocks = 0 known at compile time.  (Neither the parameters' padding nor asking for them ahead of the wait changes anything, and carrying the
+// first addresses through the wait costs 0.02 ... 0.25 us: what a block does before its wait is not hidden.)
 // kTimed (a measurement aid): thread 0 of every block also records, in nanoseconds of the global timer, when the
 // block started, when its wait for the predecessor returned and when it had issued its last store, plus the SM
 // it ran on: trace[(slot * trace_blocks + blockIdx.x) * 4 + {0, 1, 2, 3}] for blockIdx.x < trace_blocks.
-template <int N, int C, int DT, bool kTimed, bool kHot>
+template <int N, int C, int DT, bool kTimed, bool kOnce, bool kHot>
 __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_t count, const size_t ntiles, const unsigned tv,
                                                   const int stream_stores, const unsigned prefetch_blocks,
                                                   unsigned long long* trace, const unsigned slot, const unsigned trace_blocks)
@@ -513,9 +516,7 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
     }
     pdl_wait();
     if (kTimed && threadIdx.x == 0) t_wait = globaltimer_ns();
-    for (size_t item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const size_t i = (item / kSplit) * tv + threadIdx.x;
-        const int d0 = (int)(item % kSplit) * C;
+    const auto tile = [&](size_t i, int d0) {                        // vector i of the sources, destinations d0 ... d0 + C - 1
         if (threadIdx.x < tv && i < nvec) {
             uint4 v[N];
 #pragma unroll
@@ -529,6 +530,11 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
                 }
             }
         }
+    };
+    if (kOnce) {
+        tile((size_t)(blockIdx.x / kSplit) * tv + threadIdx.x, (int)(blockIdx.x % kSplit) * C);   // blocks beyond the tiles are beyond nvec
+    } else {
+        for (size_t item = blockIdx.x; item < nitems; item += gridDim.x) tile((item / kSplit) * tv + threadIdx.x, (int)(item % kSplit) * C);
     }
     pdl_trigger();
     if (kTimed) {
@@ -549,20 +555,20 @@ __device__ __forceinline__ void oneshot_regs_body(const RankPtrs& p, const size_
     }
 }
 
-template <int N, int C, int DT, bool kHot>
+template <int N, int C, int DT, bool kOnce, bool kHot>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
 k_oneshot_regs(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int stream_stores,
                const unsigned prefetch_blocks, const ParamPad<4>)
 {
-    oneshot_regs_body<N, C, DT, false, kHot>(p, count, ntiles, tv, stream_stores, prefetch_blocks, nullptr, 0u, 0u);
+    oneshot_regs_body<N, C, DT, false, kOnce, kHot>(p, count, ntiles, tv, stream_stores, prefetch_blocks, nullptr, 0u, 0u);
 }
 
-template <int N, int C, int DT>
+template <int N, int C, int DT, bool kOnce, bool kHot>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
 k_oneshot_regs_timed(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int stream_stores,
                      const unsigned prefetch_blocks, unsigned long long* trace, const unsigned slot, const unsigned trace_blocks)
 {
-    oneshot_regs_body<N, C, DT, true, false>(p, count, ntiles, tv, stream_stores, prefetch_blocks, trace, slot, trace_blocks);
+    oneshot_regs_body<N, C, DT, true, kOnce, kHot>(p, count, ntiles, tv, stream_stores, prefetch_blocks, trace, slot, trace_blocks);
 }
 
 // ---- one-shot allreduce, co-located group staged through shared memory ---------------------------------
@@ -1526,8 +1532,8 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
 // Two-shot without the intermediate: the block that reduces a tile stores it into all N destinations.
 // (A form that moves the tile through shared memory with bulk copies in both directions was measured too:
 // slower up to 4 MiB per rank -- 512 KiB: 3.2 vs 2.85 us -- and within 1.5 % beyond, so it was not kept.)
-// A tile is U rows of tv vectors; block, tile and prefetch as in k_oneshot_regs.
-template <int N, int U, int DT>
+// A tile is U rows of tv vectors; block, tile and prefetch as in k_oneshot_regs, and so is kOnce (U = 1): a block per tile.
+template <int N, int U, int DT, bool kOnce>
 __global__ void __launch_bounds__(kThreads, min_blocks(N * U))
 k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const unsigned tv, const int stream_stores,
               const unsigned prefetch_blocks, const ParamPad<4>)
@@ -1541,9 +1547,7 @@ k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const u
         if (i0 < nvec) prefetch_l2_bulk(a + i0, (unsigned)(nvec - i0 < (size_t)(tv * U) ? nvec - i0 : (size_t)(tv * U)) * 16u);
     }
     pdl_wait();
-    for (size_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const size_t base = tile * (tv * U) + threadIdx.x;
-        const size_t end = threadIdx.x < tv ? nvec : 0;
+    const auto put = [&](size_t base, size_t end) {                  // vectors base, base + tv, ... below end
         uint4 v[U][N];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -1567,6 +1571,12 @@ k_twoshot_put(const RankPtrs p, const size_t count, const size_t ntiles, const u
                 }
             }
         }
+    };
+    if (kOnce) {
+        if (threadIdx.x < tv) put((size_t)blockIdx.x * tv + threadIdx.x, nvec);
+    } else {
+        for (size_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+            put(tile * (tv * U) + threadIdx.x, threadIdx.x < tv ? nvec : 0);
     }
     pdl_trigger();
     const size_t tail0 = nvec * Elem<DT>::kElems;
