@@ -430,7 +430,7 @@ def run_gpu(args):
             per.append((time.perf_counter() - t0) * 1e6)
         return max_over_ranks(statistics.median(per))
     e2e_variants = {"inplace_twoshot_put": time_host(flags=nb.NUNA_TWOSHOT_PUT, two_shot=True),
-                    "staged_copies_oneshot": time_host()}
+                    "staged_copies_oneshot": time_host(flags=nb.NUNA_PLACE_AWARE)}
     e2e_best = min(e2e_variants, key=e2e_variants.get)
     e2e = {"value": e2e_variants[e2e_best], "unit": "us", "h2d_bytes_per_step": N_RANKS * w.bytes_per_rank,
            "d2h_bytes_per_step": N_RANKS * w.bytes_per_rank, "path": "nuna_allreduce_host, pinned host buffers: " + e2e_best}
@@ -787,7 +787,7 @@ def run_gpu(args):
     if cpu is not None:
         line["cpu_baseline"] = cpu
     try:
-        out_dir = os.path.join(ROOT, os.environ.get("BENCH_OUT_DIR", "gpurun_out"))
+        out_dir = os.path.join(ROOT, os.environ.get("BENCH_OUT_DIR", "build"))
         os.makedirs(out_dir, exist_ok=True)
         with open(os.path.join(out_dir, "bench_detail.json"), "w") as f:
             json.dump({"result": line, "detail": detail}, f, indent=1)
