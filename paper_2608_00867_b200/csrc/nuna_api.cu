@@ -575,6 +575,42 @@ struct TileShape {
     unsigned tv, threads, prefetch_blocks;
 };
 
+// The same for L2-resident sources.  Measured at 2, 3, 4, 6, 8, 12 and 16 ranks, 8 KiB ... 8 MiB per rank, tiles of 8 ... 256
+// vectors in blocks of 32 ... 256 threads, dependent graph nodes, one-shot (the put form chooses the same within 1 %); us:
+// * Small messages want few, narrow blocks: up to u = 32 half the SMs up to 4 ranks (2 x 64 KiB 0.960 with 32 vectors, 0.934 with
+//   64) and all of them beyond, in 128 threads (8 x 16 KiB 1.05 -> 1.00).
+// * Up to u = 128 a block per SM.  Few ranks have that much less to do per vector that two blocks of 64 vectors per SM are ahead
+//   (2 x 96 KiB 0.960 -> 0.936, 6 x 128 KiB 1.103 -> 1.057 against 64 vectors in 64 threads).  Every SM gets a tile: 8 ranks x
+//   128 KiB take 147 tiles of 56 vectors, 1.11, where 128 tiles of 64 took 1.15.
+// * Between, four full-width blocks per SM as for cold sources; up to 4 ranks three blocks of 128 threads up to u = 256
+//   (2 x 512 KiB 1.17 -> 1.08).
+// * Larger messages are dealt evenly, in blocks as wide as their tiles: tiles of up to 128 vectors, whose number is a whole
+//   multiple of the SMs (8 x 1 MiB 2.54 -> 2.32, 8 x 1.5 MiB 3.18 -> 2.95 against 128 vectors throughout); of up to 256 for few
+//   ranks and the longest messages (2 x 4 MiB 3.06 with 128 vectors, 2.16 with 256; 6 x 4 MiB 6.67, 6.49).
+// * What sources and destinations of one call take of L2 leaves no room for a second set beyond half of it: the hint cannot be
+//   true of a chain then, and half-full blocks keep more DRAM requests in flight (8 x 4 MiB 10.3 -> 9.9).
+static TileShape hot_shape(const Context* c, int nranks, size_t units, size_t total, size_t per_sm)
+{
+    const size_t sms = (size_t)c->num_sms;
+    const bool few = nranks <= 4;
+    const auto deal = [&](size_t blocks, size_t least) {
+        return (unsigned)std::min<size_t>(kThreads, std::max(least, ceil_div(ceil_div(units, blocks), (size_t)8) * 8));
+    };
+    const auto tight = [](unsigned tv) { return TileShape{tv, (tv + 31u) / 32u * 32u, 0u}; };
+    const auto even = [&](size_t most) { return tight(deal(sms * ceil_div(units, sms * most), 8)); };
+    const TileShape four = {deal(sms * per_sm, 56), (unsigned)kThreads, 0u};
+    if (2 * total > c->l2_bytes / 2) return {128u, (unsigned)kThreads, 0u};
+    if (units <= sms * 32) return {deal(few ? sms / 2 : sms, 16), 128u, 0u};
+    if (units <= sms * 128) {
+        if (nranks <= 6) return {64u, 128u, 0u};
+        const TileShape t = tight(deal(sms, 8));
+        return {t.tv, nranks <= 8 ? std::max(t.threads, units <= sms * 64 ? 128u : 0u) : t.threads, 0u};
+    }
+    if (few) return units <= sms * 256 ? TileShape{deal(sms * 3, 8), 128u, 0u} : units <= sms * 384 ? four : even(256);
+    if (units <= sms * (nranks <= 8 ? 384 : 448)) return four;
+    return nranks <= 8 && units > sms * 1000 ? even(256) : even(128);
+}
+
 // One tile per block.  Measured at 2, 4, 8 and 16 ranks, 16 KiB ... 64 MiB per rank, tiles of 16 ... 256 vectors in blocks
 // of 32 ... 256 threads, as dependent graph nodes (us at 8 ranks; u = vectors per source and SM; `ksplit` blocks share a
 // tile, each with a part of the destinations):
@@ -588,10 +624,7 @@ struct TileShape {
 //   prefetches: later blocks would ask L2 for what they load at once (4 MiB 11.4 -> 11.0, 6 MiB 16.9 -> 16.1, 8 MiB
 //   21.5 -> 21.1; 4 ranks x 8 MiB 11.5 -> 10.9).
 // * beyond, cold: no prefetch, half the destinations per block; half-full blocks from 5 to 8 ranks (64 MiB 159.3 -> 157.6).
-// * L2-resident sources: narrower blocks, cheaper to start: 128 threads up to u = 32 (16 KiB 1.05 -> 1.02), beyond 4 ranks
-//   one block per SM of just as many threads as the tile up to u = 128 (128 KiB 1.22 -> 1.13, 256 KiB 1.37 -> 1.32), blocks
-//   of 128 vectors and threads from u = 448 (2 MiB 4.2 -> 3.5, 4 ranks x 2 MiB 3.2 -> 2.2); otherwise the full-width blocks
-//   above are ahead.  (Cold, narrow blocks are slower up to 8 MiB of sources: more of them start
+// * L2-resident sources: hot_shape, below.  (Cold, narrow blocks are slower up to 8 MiB of sources: more of them start
 //   on an SM while the predecessor still drains, unevenly -- 512 KiB 2.07 with 256 threads, 2.6 with 64.)
 // `resident` = full-width blocks of the kernel an SM holds.
 static TileShape tile_shape(const Context* c, const Options& o, int nranks, size_t nvec, int ksplit, int resident, unsigned flags,
@@ -606,15 +639,10 @@ static TileShape tile_shape(const Context* c, const Options& o, int nranks, size
     if (o.regs_vecs > 0) return {(unsigned)std::min(kThreads, std::max(8, o.regs_vecs / 8 * 8)), (unsigned)kThreads, everyone};
     if (o.blocks > 0 && (size_t)o.blocks < sms * per_sm)             // a capped grid: as few tiles as blocks, then full tiles
         return {clamp(tile_for((size_t)o.blocks), 8), (unsigned)kThreads, everyone};
-    if (hot && units <= sms * 32) return {clamp(tile_for(sms), 16), 128u, 0u};
-    if (hot && nranks > 4 && units <= sms * 128) {
-        const unsigned tv = clamp(tile_for(sms), 64);
-        return {tv, (tv + 31u) / 32u * 32u, 0u};
-    }
-    if (hot && units > sms * 448) return {128u, 128u, 0u};
+    if (hot) return hot_shape(c, nranks, units, total, per_sm);
     if (units <= sms * 56) return {clamp(tile_for(sms), 8), (unsigned)kThreads, everyone};
     const unsigned four = clamp(tile_for(sms * per_sm), 56);
-    if (hot || total < ((size_t)6 << 20)) return {four, (unsigned)kThreads, everyone};
+    if (total < ((size_t)6 << 20)) return {four, (unsigned)kThreads, everyone};
     if (total <= ((size_t)16 << 20))
         return {std::min(four, clamp(tile_for(sms * 2 * per_sm), 112)), (unsigned)kThreads, total <= ((size_t)8 << 20) ? everyone : first_wave};
     if (total <= ((size_t)64 << 20)) {
@@ -627,13 +655,13 @@ static TileShape tile_shape(const Context* c, const Options& o, int nranks, size
 // Whether a kernel runs its form without the tile loop, which wants a block per item (us per node, looping | once):
 // * cold, up to 4 ranks, at every size (2 x 64 KiB 0.999 | 0.947, 4 x 512 KiB 1.845 | 1.787, 3 x 4 MiB 4.39 | 4.32); beyond, the
 //   loop is ahead (8 x 64 KiB 1.358 | 1.398, 16 x 256 KiB 2.38 | 3.61: every block pays for the longer text of more ranks).
-// * L2-resident, where the text is shorter, with one block per SM or fewer (u <= 128) at every rank count, and up to 8 ranks with
-//   blocks as wide as their tiles (u > 448) again; between the two the loop is 1 ... 2 % ahead (8 x 384 KiB 1.505 | 1.55).
-static bool runs_once(const Context* c, int nranks, size_t units, unsigned flags)
+// * L2-resident, where the text is shorter, but for the four full-width blocks per SM of hot_shape, where the loop is 1 ... 2 % ahead
+//   (8 x 384 KiB 1.505 | 1.55), and beyond 8 ranks from u = 448 (12 x 2 MiB 6.59 | 6.82).
+static bool runs_once(const Context* c, int nranks, size_t units, const TileShape& t, unsigned flags)
 {
-    const size_t sms = (size_t)c->num_sms;
     if (!(flags & NUNA_HINT_RESIDENT)) return nranks <= 4;
-    return units <= sms * 128 || (units > sms * 448 && nranks <= 8);
+    const bool large = units > (size_t)c->num_sms * 448;
+    return large ? nranks <= 8 : t.threads < (unsigned)kThreads;
 }
 
 template <int N, int C, int DT>
@@ -647,7 +675,7 @@ static int launch_regs(Context* c, const Options& o, const RankPtrs& p, size_t c
     const size_t ntiles = ceil_div(nvec, (size_t)t.tv);
     const size_t nitems = std::max<size_t>(ntiles * kSplit, (count % Elem<DT>::kElems) ? (size_t)N : 0);
     const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), 0, 0);
-    const bool once = grid >= nitems && runs_once(c, N, nvec * kSplit, flags);
+    const bool once = grid >= nitems && runs_once(c, N, nvec * kSplit, t, flags);
     const auto go = [&](auto kernel) { return launch_padded(kernel, grid, stream, mode, p, count, ntiles, t.tv, hot ? 0 : 1, t.prefetch_blocks); };
     t_block = t.threads;
     if constexpr (kSplit == 1) { if (hot && once) return go(k_oneshot_regs<N, C, DT, true, true>); }
@@ -833,7 +861,7 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
             return launch_padded(kernel, grid, stream, mode, p, count, ntiles, t.tv, (flags & NUNA_HINT_RESIDENT) ? 0 : 1, t.prefetch_blocks);
         };
         t_block = t.threads;
-        if constexpr (U == 1) { if (grid >= ntiles && runs_once(c, N, nvec, flags)) return go(k_twoshot_put<N, U, DT, true>); }
+        if constexpr (U == 1) { if (grid >= ntiles && runs_once(c, N, nvec, t, flags)) return go(k_twoshot_put<N, U, DT, true>); }
         return go(looping);
     });
 }
@@ -1473,7 +1501,7 @@ int nuna_debug_oneshot_regs_traced(const void* const* src, void* const* dst, siz
     const unsigned grid = pick_grid(c, o, std::max<size_t>(nitems, 1), 0, 0);
     if (grid_blocks) *grid_blocks = grid;
     t_block = t.threads;
-    const bool once = hot && grid >= nitems && runs_once(c, N, nvec, flags);
+    const bool once = hot && grid >= nitems && runs_once(c, N, nvec, t, flags);
     const auto k = once ? k_oneshot_regs_timed<N, 8, kBf16, true, true> : hot ? k_oneshot_regs_timed<N, 8, kBf16, false, true>
                                                                              : k_oneshot_regs_timed<N, 8, kBf16, false, false>;
     return launch(k, grid, (cudaStream_t)stream, mode, make_ptrs(src, dst, N), count, ntiles, t.tv, hot ? 0 : 1,

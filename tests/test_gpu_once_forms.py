@@ -42,3 +42,32 @@ def test_block_per_tile_and_capped_grid(n, dtype, blocks):
     finally:
         nb.nuna_set_option(nb.NUNA_OPT_BLOCKS, 0)
     assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+L2 = torch.cuda.get_device_properties(0).L2_cache_size if torch.cuda.is_available() else 126 << 20
+
+
+@pytest.mark.parametrize("n", [2, 5, 7, 9, 16])
+def test_resident_shapes_on_both_sides_of_every_line(n):
+    """Vectors per SM (32, 64, 128, 256, 384, 448, 1000) and a quarter of L2 in sources, one vector below, at and above."""
+    lines = [SMS * u for u in (32, 64, 128, 256, 384, 448, 1000)] + [L2 // 4 // 16 // n]
+    top = 8 * (max(lines) + 2)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    src = [torch.randn(top, generator=gen, device="cuda").bfloat16() for _ in range(n)]
+    acc = src[0].float()
+    for s in src[1:]:
+        acc += s.float()
+    want = acc.bfloat16()
+    dst = [torch.empty(top + GUARD, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    for vectors in sorted({v + d for v in lines for d in (-1, 0, 1)}):
+        count = 8 * vectors + vectors % 8
+        for call, flags in FORMS:
+            for d in dst:
+                d[:count + GUARD].fill_(7.0)
+            call(src, dst, count, flags=flags | nb.NUNA_HINT_RESIDENT)
+            for d in dst:
+                assert torch.equal(d[:count], want[:count]), (count, flags)
+                assert bool((d[count:count + GUARD] == 7.0).all()), (count, flags)
+    assert nb.nuna_device_status() == nb.NUNA_OK
