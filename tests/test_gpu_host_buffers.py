@@ -5,7 +5,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2608_00867_b200 import binding as nb
+from paper_2608_00867_b200 import workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -40,3 +42,34 @@ def test_a_buffer_is_mapped_only_if_all_of_it_is_page_locked():
     t = torch.zeros(3 << 20, dtype=torch.uint8).pin_memory()
     assert mapped(t.data_ptr(), 3 << 20) == 1 and mapped(t.data_ptr() + 16, (3 << 20) - 16) == 1
     assert mapped(torch.zeros(64, device="cuda").data_ptr(), 16) == 0
+
+
+WORD = {"bf16": np.uint16, "f16": np.uint16, "f32": np.uint32}
+GUARD = 64
+
+
+@pytest.mark.parametrize("flags", [0, nb.NUNA_PLACE_AUTO, nb.NUNA_HINT_RESIDENT, nb.NUNA_PLACE_AWARE, nb.NUNA_PLACE_AUTO | nb.NUNA_LAUNCH_PDL])
+@pytest.mark.parametrize("dtype", ["bf16", "f16", "f32"])
+def test_one_shot_on_page_locked_buffers(dtype, flags):
+    """In place (but for NUNA_PLACE_AWARE, which stages): ragged counts, several passes of the few blocks, buffers that are
+    page-locked but not aligned to a vector, guard zones around the destinations."""
+    word = WORD[dtype]
+    size = np.dtype(word).itemsize
+    for n, count in ((2, 5), (8, 1001), (3, 40 * 2048 + 3), (16, 4096)):
+        src = workloads.rank_buffers_typed(n, count, "normal", 11 + count, dtype)
+        want = oracle.allreduce(src, dtype=dtype)[0]
+        for shift in (0, size):
+            psrc, pdst = [], []
+            for a in src:
+                t = torch.zeros(shift + a.nbytes, dtype=torch.uint8)
+                t[shift:] = torch.from_numpy(a.view(np.uint8).copy())
+                psrc.append(t.pin_memory())
+                pdst.append(torch.full((a.nbytes + 2 * GUARD + shift,), 0x5A, dtype=torch.uint8).pin_memory())
+            nb.nuna_allreduce_host([t.data_ptr() + shift for t in psrc], [t.data_ptr() + GUARD + shift for t in pdst], count,
+                                   dtype=nb.DTYPE_BY_NAME[dtype], flags=flags)
+            for t in pdst:
+                h = t.numpy()
+                at = GUARD + shift
+                assert (h[:at] == 0x5A).all() and (h[at + want.nbytes:] == 0x5A).all(), (n, count, shift)
+                assert np.array_equal(h[at:at + want.nbytes].view(word), want), (n, count, shift)
+    assert nb.nuna_device_status() == nb.NUNA_OK
