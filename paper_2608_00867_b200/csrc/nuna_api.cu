@@ -1277,11 +1277,17 @@ int nuna_allreduce_host(const void* const* src, void* const* dst, int nranks, si
             mapped = msrc[r] && mdst[r] && (((uintptr_t)msrc[r] | (uintptr_t)mdst[r]) & 15u) == 0;
         }
         if (mapped) {
-            // Few blocks: reads of host memory issued by many SMs at once get less out of the link than the same reads
-            // from a few, and twelve suffice to fill it (8 x 512 KiB: 166 us with one block per tile, 124.9 with 24 blocks,
-            // 122.8 with 12, 123.0 with 8; 8 x 64 KiB 31.6 with 24, 30.4 with 12; 2 x 2 MB 117.5 with 12, 130 with 8).
-            // What is left: either direction of the link alone takes 89 us of device time for 4 MiB.
-            st = launch_twoshot_put(c, make_ptrs(msrc, mdst, nranks), nranks, dtype, count, flags & ~NUNA_LAUNCH_PDL, c->stream, 12u);
+            // Few blocks: reads of host memory issued by many SMs at once get less out of the link than the same reads from
+            // a few (8 x 512 KiB: 166 us with one block per tile).  The fewer, though, the longer the first call on buffers
+            // that were just page-locked, when every translation of theirs is still missing.  us on the first call | later, 12,
+            // 20 and 24 blocks: 8 x 512 KiB 167 153 148 | 124.2 123.7 124.9, 4 x 1 MiB 172 157 160 | 124.6 124.4 124.4, 2 x 512 KiB
+            // 64 59 58 | 42.7 41.7 41.7, 2 x 2 MiB 191 187 187 | 126.7 122.0 122.3.  Twelve suffice for the first call, and are
+            // ahead later, beyond 8 ranks (16 x 256 KiB 154 149 153 | 127 134 138) and for little data of many ranks (8 x 128 KiB
+            // 64 64 62 | 44.0 45.5 47.0, 8 x 64 KiB 47 46 46 | 31.7 33.1 33.1; 2 x 64 KiB 25 24 24 | 19.5 18.8 18.7).
+            // What is left: either direction of the link alone takes 86 us of device time for 4 MiB.
+            const bool twelve = nranks > 8 || (nranks > 4 && bytes * (size_t)nranks <= ((size_t)1 << 20));
+            st = launch_twoshot_put(c, make_ptrs(msrc, mdst, nranks), nranks, dtype, count, flags & ~NUNA_LAUNCH_PDL, c->stream,
+                                    twelve ? 12u : 20u);
             if (st != NUNA_OK) return st;
             return cudaStreamSynchronize(c->stream) == cudaSuccess ? NUNA_OK : NUNA_ERR_CUDA;
         }
