@@ -4,8 +4,8 @@
 // 1.7 (dependent launch) to 2.1 us (plain), and marshalling 2 * nranks tensors in Python around a ctypes call cost
 // 7-12 us more (a data_ptr() method call and a ctypes item store per tensor, 3.2 us for torch.cuda.current_stream()).
 // Here a tensor's address is read from the tensor object itself and the current stream from c10.  Measured back to
-// back, before -> now: 2 ranks x 8 KiB one-shot 10.2 -> 3.2 us, 8 ranks x 512 KiB allreduce 12.2 -> 2.6, 16 ranks x
-// 64 KiB allgather 15.5 -> 3.4; a call that only validates (count 0) costs 0.25 us at 2 ranks, 0.38 us at 16.
+// back, before -> now: 2 ranks x 8 KiB one-shot 10.1 -> 2.3 us, 8 ranks x 512 KiB allreduce 11.9 -> 2.5, 16 ranks x
+// 64 KiB allgather 15.1 -> 3.35; a call that only validates (count 0) costs 0.25 us at 2 ranks, 0.38 us at 16.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
