@@ -831,17 +831,19 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
     });
 }
 
-// The put form: one tile per block by default; `max_blocks` > 0 makes it a grid-stride loop over that many blocks.
-// Whether a two-shot kernel asks L2 for its blocks' first tiles ahead of the dependent-launch wait: cold
-// device-memory sources, and a message small enough that the predecessor's drain is a visible share of it.
-// Measured with the put form (us, with | without): 8 ranks 2 MiB 6.16 | 6.44, 8 MiB 21.4 | 21.8, 16 MiB 42.1 | 42.1,
-// 64 MiB 162.5 | 160.8; 16 ranks 256 KiB 3.25 | 3.46, 1 MiB 6.74 | 6.59, 8 MiB 43.1 | 42.6; 4 ranks 32 MiB 41.3 | 41.7.
+// Whether the flag two-shot, the allgather and the alltoall ask L2 for their blocks' first tiles ahead of the
+// dependent-launch wait: cold device-memory sources, and a message small enough that the predecessor's drain is a visible
+// share of it.  us with | without, by MiB of sources: flag two-shot, 8 ranks, 2 4.8 | 5.2, 8 10.1 | 11.7, 32 14.5 | 15.9, 128
+// 44.0 | 45.4; 2 ranks 32 15.2 | 16.5, but 128 53.6 | 52.3; allgather, 16 ranks, 4 10.9 | 12.5, 4 ranks 32 26.8 | 28.0, 128
+// 103.3 | 104.3; alltoall, 8 ranks, 4 2.2 | 2.8, 32 10.3 | 11.5, 128 40.9 | 41.8.  Beyond 8 ranks 8 MiB (16 ranks, flag two-shot, 7.3 | 8.2)
+// is as far as it has been measured to pay.
 static bool prefetch_pays(const Options& o, unsigned flags, int nranks, size_t bytes)
 {
     if (!(flags & NUNA_LAUNCH_PDL) || (flags & NUNA_HINT_RESIDENT) || o.prefetch == 1) return false;
     return bytes * (size_t)nranks <= (nranks <= 8 ? (size_t)128 << 20 : (size_t)8 << 20);
 }
 
+// The put form: one tile per block by default; `max_blocks` > 0 makes it a grid-stride loop over that many blocks.
 int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, size_t count, unsigned flags, cudaStream_t stream,
                        unsigned max_blocks)
 {
@@ -930,11 +932,14 @@ int launch_allgather(Context* c, const RankPtrs& p, int nranks, size_t shard_byt
         const size_t tiles = ceil_div(shard_vec + (shard_vec % 8 ? 7 : 0), (size_t)small_tv);   // the first tile of a shard may be short
         const unsigned grid = (unsigned)(tiles * nranks);
         if (o.blocks <= 0 || (size_t)o.blocks >= grid) {           // one tile per block: a capped grid takes the looping form below
-            // from 4 ranks and 112 vectors, blocks of no more threads than the tile: more of them fit beside each other
-            // (8 x 256 KiB 3.87 -> 3.26 us, 4 x 512 KiB 2.48 -> 2.23, 16 x 64 KiB 3.29 -> 3.26; smaller tiles are up to 15 %
-            // faster in full-width blocks)
-            if (nranks >= 4 && small_tv >= 112) t_block = (small_tv + 31u) / 32u * 32u;
-            return launch_padded(k_allgather_small, grid, stream, mode, p, nranks, shard_vec, small_tv, prefetch ? 1 : 0);
+            // Blocks of no more threads than the tile once tiles are large: more of them fit beside each other.  Full-width |
+            // narrow, cold, us: 8 ranks, tiles of 104 vectors 2.15 | 2.18, 112 2.25 | 2.16, 192 3.28 | 2.99; 16 ranks 96 3.01 | 2.93,
+            // 144 4.37 | 3.90; 12 ranks 112 2.78 | 2.80, 144 3.49 | 3.25.  With fewer ranks to store to, the line lies further up:
+            // 4 ranks 112 1.91 | 1.93, 128 1.96 | 2.08, 160 2.08 | 2.09, 192 2.28 | 2.25; 6 ranks 128 2.20 | 2.34, 160 2.61 | 2.66, 192 3.18 | 2.69.  Two
+            // and three ranks and smaller tiles are up to 30 % faster in full-width blocks.
+            if (nranks >= 4 && small_tv >= (nranks >= 8 ? 112u : 176u)) t_block = (small_tv + 31u) / 32u * 32u;
+            return launch_padded(shard_vec % 8 ? k_allgather_small<true> : k_allgather_small<false>, grid, stream, mode, p, nranks, shard_vec,
+                                 small_tv, prefetch ? 1 : 0);
         }
     }
     if (o.ag_bulk_vecs != 1) {

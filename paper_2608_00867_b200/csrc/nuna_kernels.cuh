@@ -1056,14 +1056,16 @@ k_allgather(const RankPtrs p, const int nranks, const size_t shard_vec, const si
 // stores it to the N destinations.  With the tile sized so that every SM gets about four blocks this is faster than
 // the bulk-copy form below up to 128 MiB of output (16 x 8 KiB 1.28 against 1.68 us, 16 x 64 KiB 3.46 against 3.81,
 // 8 x 64 KiB 1.60 against 1.92, 16 x 512 KiB 22.9 against 24.1; 8 x 8 MiB 96.5 against 93.9).
+template <bool kLines>
 __global__ void __launch_bounds__(kThreads)
 k_allgather_small(const RankPtrs p, const int nranks, const size_t shard_vec, const unsigned tv, const int prefetch,
                   const ParamPad<8>)
 {
     const int r = (int)(blockIdx.x % (unsigned)nranks);
-    // tiles end on 128-byte lines of the destinations: the first one is short by what the shard starts into a line (shards of
-    // 65 552 bytes 3.66 -> 3.51 us; it changes nothing for the bulk copies of k_alltoall_bulk)
-    const size_t tile = blockIdx.x / (unsigned)nranks, skip = (size_t)r * shard_vec & 7u;
+    // kLines: tiles end on 128-byte lines of the destinations although shards do not: the first one is short by what the shard
+    // starts into a line (shards of 65 552 bytes 3.66 -> 3.51 us; it changes nothing for the bulk copies of k_alltoall_bulk).
+    // Shards of whole lines do without the arithmetic, which stands between the wait and the load (4 x 336 256 bytes 2.07 -> 2.04 us).
+    const size_t tile = blockIdx.x / (unsigned)nranks, skip = kLines ? (size_t)r * shard_vec & 7u : 0;
     if (prefetch && threadIdx.x == 0) {
         const size_t i0 = tile ? tile * tv - skip : 0, i1 = tile * tv + tv - skip;
         if (i0 < shard_vec) prefetch_l2_bulk(p.src[r] + i0, (unsigned)((i1 < shard_vec ? i1 : shard_vec) - i0) * 16u);

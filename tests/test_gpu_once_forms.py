@@ -71,3 +71,17 @@ def test_resident_shapes_on_both_sides_of_every_line(n):
                 assert torch.equal(d[:count], want[:count]), (count, flags)
                 assert bool((d[count:count + GUARD] == 7.0).all()), (count, flags)
     assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+@pytest.mark.parametrize("n", [3, 4, 7, 8, 16])
+def test_allgather_on_both_sides_of_the_block_width_lines(n):
+    """Tiles of 104 ... 184 vectors: blocks become as wide as their tiles at 112 (from 8 ranks) and 176 (from 4)."""
+    for tile in (104, 112, 168, 176, 184):
+        for vectors in (tile * 4 * SMS // n, tile * 4 * SMS // n // 8 * 8, tile * 4 * SMS // n - 3):
+            src = [torch.randint(0, 1 << 15, (8 * vectors,), device="cuda", dtype=torch.int16) for _ in range(n)]
+            dst = [torch.full((8 * vectors * n + GUARD,), -7, device="cuda", dtype=torch.int16) for _ in range(n)]
+            nb.nuna_allgather(src, dst, 8 * vectors)
+            want = torch.cat(src)
+            for d in dst:
+                assert torch.equal(d[:want.numel()], want) and bool((d[want.numel():] == -7).all()), (n, tile, vectors)
+    assert nb.nuna_device_status() == nb.NUNA_OK
