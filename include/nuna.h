@@ -304,9 +304,13 @@ int nuna_allreduce_oneshot(const void* const* src, void* const* dst, int nranks,
  * after acquire-polling that tile's flag (bounded wait: on expiry NUNA_ERR_TIMEOUT is latched and the block
  * returns).  A wait is only ever for an item with a smaller ticket, held by a block that already runs, so
  * the kernel needs no co-residency guarantee and no cooperative launch.  Consumed shard lines are dropped
- * from L2 (discard) instead of being written back.  Same bits as the one-shot.  Any `count`; chunk =
+ * from L2 (discard) instead of being written back.  Small and mid-sized messages (up to 8 MiB per rank, 6 MiB up to 4 ranks) take a
+ * form without a flag per tile: every 32-bit word of the reduced tile is stored together with the launch's
+ * epoch in one 64-bit access, and the gathering block polls the words themselves, under the same bound.  It is
+ * not used with NUNA_TWOSHOT_SYS_SCOPE, NUNA_OPT_TWOSHOT_VECS or NUNA_OPT_BLOCKS.  Same bits as the one-shot.  Any `count`; chunk =
  * ceil(count/N) rounded up to a whole 16-byte vector, trailing chunks may be short or empty.  Uses the
- * context's shard scratch (count*elemsize bytes plus one flag word per 256 bytes, grown on demand; an
+ * context's shard scratch (count*elemsize bytes plus one flag word per 256 bytes, plus twice as much for up to
+ * 8 MiB of it, where the words stand with their epochs; grown on demand; an
  * outgrown scratch stays allocated until nuna_shutdown because captured graphs may still name it) unless
  * NUNA_TWOSHOT_PUT is set.  Calls that share the context must be stream-ordered with respect to each other. */
 int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,

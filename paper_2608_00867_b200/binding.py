@@ -440,11 +440,12 @@ def debug_oneshot_regs_traced(src, dst, count, flags: int, slot: int, trace, str
     return grid.value
 
 
-def debug_twoshot(src, dst, count, dtype=NUNA_BF16, timeout_ms: int = 1000, unset_flags: bool = False) -> int:
-    """Test hook: the flag-synchronised two-shot with an explicit timeout; with unset_flags its consumers
-    wait for flags nobody publishes, so every (bounded) wait runs out."""
+def debug_twoshot(src, dst, count, dtype=NUNA_BF16, timeout_ms: int = 1000, unset_flags: bool = False,
+                  tagged: bool = False) -> int:
+    """Test hook: the flag-synchronised two-shot (`tagged`: the form whose words carry their flags) with an explicit timeout;
+    with unset_flags its consumers wait for flags nobody publishes, so every (bounded) wait runs out."""
     return lib().nuna_debug_twoshot(ptr_table(src), ptr_table(dst), len(src), count, dtype, timeout_ms,
-                                    1 if unset_flags else 0)
+                                    (1 if unset_flags else 0) | (32 if tagged else 0))
 
 
 def debug_barrier_selftest(grid: int, expected: int, timeout_ms: int):

@@ -24,6 +24,7 @@ static std::atomic<Context*> g_ctx[kMaxDevices];              // written under g
 
 static int static_status_read_and_clear(unsigned* out);     // the allocation-free entry point's status word (end of file)
 constexpr unsigned kMinFlagTileVec = 16;                    // smallest two-shot tile (vectors): 256 bytes of shard per flag
+constexpr size_t kTaggedMaxShard = (size_t)8 << 20;         // largest message, in bytes per rank, that the tagged two-shot takes
 constexpr unsigned kStaticTileVec = 128;                    // tile of the allocation-free entry point: 2 KiB of shard per flag
 
 static int env_int(const char* name, int fallback)
@@ -82,24 +83,27 @@ int get_context(Context** out)
     return NUNA_OK;
 }
 
-// Grows the two-shot scratch (shard intermediate + one ready flag per smallest tile of it).  The caller holds
-// c->mutex.  An outgrown allocation is never freed before nuna_shutdown: a CUDA graph captured earlier
+// Grows the two-shot scratch: shard intermediate, one ready flag per smallest tile of it, and the slots of the tagged form
+// for as large a shard as that form takes.  The caller holds c->mutex.  An outgrown allocation is never freed before nuna_shutdown: a CUDA graph captured earlier
 // (a chain, or a user's capture of a two-shot call) still carries its address as a kernel argument.
 int ensure_scratch(Context* c, size_t bytes)
 {
     if (bytes <= c->scratch_bytes && c->scratch) return NUNA_OK;
     const size_t want = (std::max<size_t>(bytes, 4096) + 4095) & ~(size_t)4095;
     const size_t nflags = want / (kMinFlagTileVec * 16) + 1;         // one ready flag per smallest tile
+    const size_t slots_at = (want + nflags * sizeof(unsigned) + 255) & ~(size_t)255;
+    const size_t total = slots_at + tagged_bytes(std::min(want, kTaggedMaxShard));
     void* p = nullptr;
-    if (cudaMalloc(&p, want + nflags * sizeof(unsigned)) != cudaSuccess) return NUNA_ERR_CUDA;
-    // flags start at zero; epochs start at one, so a fresh flag never reads as "ready"
-    if (cudaMemset(static_cast<char*>(p) + want, 0, nflags * sizeof(unsigned)) != cudaSuccess) {
+    if (cudaMalloc(&p, total) != cudaSuccess) return NUNA_ERR_CUDA;
+    // flags and tags start at zero; epochs start at one, so a fresh one never reads as "ready"
+    if (cudaMemset(static_cast<char*>(p) + want, 0, total - want) != cudaSuccess) {
         cudaFree(p);
         return NUNA_ERR_CUDA;
     }
     if (c->scratch) c->retired_scratch.push_back(c->scratch);
     c->scratch = p;
     c->flags = reinterpret_cast<unsigned*>(static_cast<char*>(p) + want);
+    c->slots = static_cast<char*>(p) + slots_at;
     c->scratch_bytes = want;
     return NUNA_OK;
 }
@@ -831,6 +835,40 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
     });
 }
 
+// How the tagged two-shot is launched, always in full-width blocks: narrow ones start on an SM while the predecessor still
+// drains, unevenly (8 x 64 KiB 1.8 us in 256 threads, 2.5 in 64).  Measured at 2, 4, 8 and 16 ranks, 16 KiB ... 16 MiB per rank, cold, tiles
+// of 16 ... 256 vectors, leads of 1 ... 1184 tiles, dependent graph nodes (us):
+// * As long as all blocks are resident together, each gathers the tile before its own (lead 1: 8 x 512 KiB 2.9, 3.6 with a lead of
+//   three tiles per SM): four tiles per SM of 56 ... 128 vectors, from 96 up to 8 ranks (8 x 512 KiB 2.95 with 56, 2.89; 16 x
+//   256 KiB 2.88 with 56, 3.00), fewer and larger ones up to 4 ranks (2 x 1 MiB 2.75 with 96 vectors, 2.53 with 192).
+// * Beyond, a lead of three tiles per SM, so that what a block gathers was reduced a wave earlier (8 x 4 MiB 11.5; five 11.6,
+//   one 11.7, eight 11.9), and tiles of 128 vectors (192 12.1), 192 up to 4 ranks (2 x 8 MiB 8.84; 128 9.2, 256 8.97).
+struct TaggedShape {
+    unsigned tv, lead;
+};
+
+static TaggedShape tagged_shape(const Context* c, int nranks, size_t nvec)
+{
+    const size_t sms = (size_t)c->num_sms;
+    const auto deal = [&](size_t blocks, size_t least, size_t most) {
+        return (unsigned)std::min(most, std::max(least, ceil_div(ceil_div(nvec, blocks), (size_t)8) * 8));
+    };
+    if (nvec <= sms * 32) return {nranks <= 4 ? 96u : 32u, 1u};
+    if (nranks <= 4) return nvec <= sms * 4 * 192 ? TaggedShape{deal(sms * 2, 96, 192), 1u} : TaggedShape{192u, (unsigned)sms * 3};
+    const size_t least = nranks <= 8 && nvec > sms * 96 ? 96 : 56;
+    return nvec <= sms * 4 * 128 ? TaggedShape{deal(sms * 4, least, 128), 1u} : TaggedShape{128u, (unsigned)sms * 3};
+}
+
+// Whether a two-shot call runs the tagged form.  us per node, flags | tagged: 2 ranks x 64 KiB 3.19 | 1.96, 4 MiB 9.9 | 6.1,
+// 8 MiB 9.4 | 9.8; 4 x 512 KiB 6.4 | 2.6, 4 MiB 8.8 | 7.9; 8 x 8 KiB 3.3 | 2.0, 512 KiB 5.0 | 2.9, 4 MiB 14.2 | 12.2, 8 MiB 24.7 | 22.7,
+// 16 MiB 44.6 | 45.9; 16 x 64 KiB 5.6 | 2.6, 1 MiB 10.1 | 7.5, 4 MiB 25.6 | 22.7.  The fewer the ranks, the more the shard's doubled
+// bytes are beside theirs.  What asks about the flags (their scope, their tile, the shard's lines) gets the form that has them.
+static bool takes_tags(const Options& o, int nranks, size_t bytes, unsigned flags)
+{
+    return bytes <= (nranks <= 4 ? kTaggedMaxShard / 4 * 3 : kTaggedMaxShard) && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard &&
+           o.twoshot_vecs <= 0 && o.blocks <= 0;
+}
+
 // Whether the flag two-shot, the allgather and the alltoall ask L2 for their blocks' first tiles ahead of the
 // dependent-launch wait: cold device-memory sources, and a message small enough that the predecessor's drain is a visible
 // share of it.  us with | without, by MiB of sources: flag two-shot, 8 ranks, 2 4.8 | 5.2, 8 10.1 | 11.7, 32 14.5 | 15.9, 128
@@ -868,17 +906,37 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
     });
 }
 
+// The form whose shard words carry their own flags: a block per tile and `lead` more that only gather.
+static int launch_twoshot_tagged(const Context* c, const Options& o, const RankPtrs& p, int nranks, int dtype, size_t count, uint4* slots,
+                                 unsigned long long timeout_ns, unsigned flags, unsigned debug_bits, cudaStream_t stream)
+{
+    const unsigned mode = launch_mode(flags);
+    const size_t nvec = count / elems_per_vec(dtype), bytes = count * elem_size(dtype);
+    const TaggedShape t = tagged_shape(c, nranks, nvec);
+    const size_t ntiles = std::max<size_t>(1, ceil_div(nvec, (size_t)t.tv));
+    const unsigned grid = (unsigned)(ntiles + std::min<size_t>(ntiles, t.lead));
+    const unsigned bits = debug_bits | (prefetch_pays(o, flags, nranks, bytes) ? 16u : 0u);
+    return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
+        constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
+        return launch_padded(k_twoshot_tagged<N, DT>, grid, stream, mode, p, slots, count, t.tv, t.lead, c->bw, timeout_ns, bits);
+    });
+}
+
 int launch_twoshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t count, unsigned flags, cudaStream_t stream)
 {
     if (flags & NUNA_TWOSHOT_PUT) return launch_twoshot_put(c, p, nranks, dtype, count, flags, stream, 0u);
-    const Options o = snapshot(c);
-    uint4* scratch;
+    uint4 *scratch, *slots;
     unsigned* tile_flags;
+    Options o;
     {
         std::lock_guard<std::mutex> lock(c->mutex);
+        o = c->opt;
         scratch = reinterpret_cast<uint4*>(c->scratch);
+        slots = reinterpret_cast<uint4*>(c->slots);
         tile_flags = c->flags;
     }
+    if (takes_tags(o, nranks, count * elem_size(dtype), flags))
+        return launch_twoshot_tagged(c, o, p, nranks, dtype, count, slots, o.timeout_ns, flags, 0u, stream);
     return launch_twoshot_flags(c->num_sms, o.blocks, p, nranks, dtype, count, (unsigned)std::max(0, o.twoshot_vecs), kMinFlagTileVec,
                                 scratch, tile_flags, c->bw, o.timeout_ns, (flags & NUNA_LAUNCH_PDL) != 0,
                                 (o.keep_shard ? 4u : 0u) | ((flags & NUNA_TWOSHOT_SYS_SCOPE) ? 8u : 0u) |
@@ -1528,17 +1586,22 @@ int nuna_debug_twoshot(const void* const* src, void* const* dst, int nranks, siz
 {
     int st = check_args(src, dst, nranks, count, count, dtype, 0u, true);
     if (st != NUNA_OK || count == 0) return st;
-    if ((debug_bits & ~5u) != 0u) return NUNA_ERR_INVALID_ARG;
+    const bool tagged = (debug_bits & 32u) != 0u;
+    if ((debug_bits & ~37u) != 0u || (tagged && count * elem_size(dtype) > kTaggedMaxShard)) return NUNA_ERR_INVALID_ARG;
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
-    uint4* scratch;
+    uint4 *scratch, *slots;
     unsigned* tile_flags;
     {
         std::lock_guard<std::mutex> lock(c->mutex);
         if ((st = ensure_scratch(c, (count * elem_size(dtype) + 15) & ~(size_t)15)) != NUNA_OK) return st;
         scratch = reinterpret_cast<uint4*>(c->scratch);
+        slots = reinterpret_cast<uint4*>(c->slots);
         tile_flags = c->flags;
     }
+    if (tagged)
+        return launch_twoshot_tagged(c, snapshot(c), make_ptrs(src, dst, nranks), nranks, dtype, count, slots,
+                                     (unsigned long long)timeout_ms * 1000000ull, 0u, debug_bits & 1u, (cudaStream_t)0);
     return launch_twoshot_flags(c->num_sms, 0, make_ptrs(src, dst, nranks), nranks, dtype, count, 0u, kMinFlagTileVec, scratch,
                                 tile_flags, c->bw, (unsigned long long)timeout_ms * 1000000ull, false, debug_bits,
                                 (cudaStream_t)0);

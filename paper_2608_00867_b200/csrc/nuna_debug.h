@@ -26,7 +26,7 @@ int nuna_debug_barrier_selftest(unsigned grid, unsigned expected, unsigned timeo
 
 /* The flag-synchronised two-shot allreduce with an explicit timeout.  debug_bits = 1: consumers wait for a
  * flag value nobody publishes, so every wait runs out after timeout_ms, the kernel returns and the status
- * word latches NUNA_ERR_TIMEOUT.                                                                        */
+ * word latches NUNA_ERR_TIMEOUT.  + 32: the tagged form, whose consumers wait for tags nobody writes.      */
 int nuna_debug_twoshot(const void* const* src, void* const* dst, int nranks, size_t count, int dtype,
                        unsigned timeout_ms, unsigned debug_bits);
 

@@ -51,6 +51,7 @@ struct Context {
     BarrierWords* bw = nullptr;          // flag-barrier words, work cursor, epoch + latched status, device memory
     void* scratch = nullptr;             // two-shot shard intermediate, followed by its per-tile ready flags
     unsigned* flags = nullptr;           // one word per smallest tile of the scratch (inside the same allocation)
+    void* slots = nullptr;               // slots of the tagged two-shot (inside the same allocation)
     size_t scratch_bytes = 0;
     std::vector<void*> retired_scratch;  // outgrown scratch allocations: captured graphs may still name them
     void* staging = nullptr;             // device copies of host buffers (nuna_allreduce_host)

@@ -1411,6 +1411,17 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* flag, unsigned int
     return true;
 }
 
+// Draws the block's ticket and the launch's epoch (low and high half) in one round trip.  The block that draws the last
+// ticket sets the word up for the next launch, and has its exchange answered, i.e. performed at L2, before it goes on: a
+// dependent launch's blocks start as soon as every block of its predecessor has triggered (its first warp to do so counts),
+// and one that draws ahead of its wait must find the word set up.
+__device__ __forceinline__ unsigned long long draw_ticket(BarrierWords* bw)
+{
+    const unsigned long long t = atomicAdd(&bw->ticket, 1ull);
+    if ((unsigned)t != gridDim.x - 1u) return t;
+    return atomicExch(&bw->ticket, ((t >> 32) + 1ull) << 32) - 1ull;   // answers with what the add left: t + 1
+}
+
 // Barrier among the 128 threads of one half of the block (ids 1 and 2; 0 is __syncthreads).
 __device__ __forceinline__ void half_sync(int id) { asm volatile("bar.sync %0, 128;" :: "r"(id) : "memory"); }
 
@@ -1454,12 +1465,7 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
         if (i0 < nvec) prefetch_l2_bulk(a + i0, (unsigned)(nvec - i0 < (size_t)tv ? nvec - i0 : (size_t)tv) * 16u);
     }
     pdl_wait();                                                     // before the first global load or store
-    if (threadIdx.x == 0) {
-        const unsigned long long t = atomicAdd(&bw->ticket, 1ull);  // epoch and ticket in one round trip
-        if ((unsigned)t == gridDim.x - 1u)                          // the last ticket: set up the next launch
-            *reinterpret_cast<volatile unsigned long long*>(&bw->ticket) = ((t >> 32) + 1ull) << 32;
-        sh_ticket = t;
-    }
+    if (threadIdx.x == 0) sh_ticket = draw_ticket(bw);             // (ahead of the wait: 8 x 128 KiB 4.0 -> 6.2 us)
     __syncthreads();
     const size_t item = (unsigned)sh_ticket;
     const unsigned epoch1 = (unsigned)(sh_ticket >> 32) + 1u;
@@ -1527,6 +1533,129 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
                 }
             }
         }
+    }
+    pdl_trigger();
+}
+
+// ---- two-shot allreduce whose shard words carry their own ready flags ----------------------------------------
+//
+// The same two phases for small and mid-sized messages, where the flag kernel's dependent steps are what counts: a bulk copy
+// into shared memory, a release fence, a poll, and only then the shard's load.  Here every 32-bit word of the reduced tile
+// is stored in one 64-bit store together with this launch's epoch (its tag), and the gathering thread polls the data
+// itself: a word whose tag is this launch's has arrived, with no fence and no second round trip.  A 64-bit access is
+// performed as a whole, so no word is seen with a tag that is not its own, and words need no order among each other.  It
+// costs the shard twice its bytes in L2, whose writes are what bounds it beside HBM.  The block with ticket i reduces tile i
+// (thread j: vector j of all N sources, in registers) and gathers tile i - lead; a wait is only ever for a smaller ticket, as
+// above, and is bounded.  Tags of earlier launches never match, so nothing is reset.  The ticket is drawn ahead of the
+// dependent-launch wait: its round trip runs beside the predecessor's drain.  8 ranks, cold, flags | this (us): 16 KiB 3.4 | 2.06,
+// 512 KiB 5.0 | 2.9, 4 MiB 13.9 | 11.5.  (Data without tags, an impossible bit pattern for "not there", cleared behind the
+// gather: 1 ... 2 % faster at 8 ranks, 3 ... 7 % up to 4, but what a timed-out launch leaves behind would be read as data.)
+//
+// slots: 128 bytes for the tail (a 64-bit {word, tag} per element), then 1 KiB per 32 vectors: the first two words of every
+// vector, then the other two, so that a warp's accesses are whole lines.
+constexpr size_t kTailSlots = 8;
+__host__ __device__ constexpr size_t tagged_slot(size_t vec) { return kTailSlots + (vec / 32) * 64 + (vec & 31u); }
+constexpr size_t tagged_bytes(size_t shard_bytes) { return (kTailSlots + (shard_bytes / 16 + 32) / 32 * 64) * 16; }
+
+__device__ __forceinline__ void st_tagged(uint4* p, uint32_t a, uint32_t b, uint32_t tag)
+{
+    asm volatile("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%1, %3};\n\tmov.b64 y, {%2, %3};\n\tst.relaxed.gpu.global.v2.b64 [%0], {x, y};\n\t}"
+                 :: "l"(p), "r"(a), "r"(b), "r"(tag) : "memory");
+}
+
+__device__ __forceinline__ uint4 ld_tagged(const uint4* p)            // {word, its tag, word, its tag}
+{
+    uint4 v;
+    asm volatile("{\n\t.reg .b64 x, y;\n\tld.relaxed.gpu.global.v2.b64 {x, y}, [%4];\n\tmov.b64 {%0, %1}, x;\n\tmov.b64 {%2, %3}, y;\n\t}"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_tagged1(uint2* p, uint32_t a, uint32_t tag)
+{
+    asm volatile("{\n\t.reg .b64 x;\n\tmov.b64 x, {%1, %2};\n\tst.relaxed.gpu.global.b64 [%0], x;\n\t}" :: "l"(p), "r"(a), "r"(tag) : "memory");
+}
+
+__device__ __forceinline__ uint2 ld_tagged1(const uint2* p)
+{
+    uint2 v;
+    asm volatile("{\n\t.reg .b64 x;\n\tld.relaxed.gpu.global.b64 x, [%2];\n\tmov.b64 {%0, %1}, x;\n\t}" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
+// Repeats `arrived`, which loads and looks, until it says yes.  Bounded like wait_flag.
+template <typename Arrived>
+__device__ __forceinline__ bool poll_tagged(Arrived&& arrived, unsigned long long timeout_ns, unsigned int* status)
+{
+    if (arrived()) return true;
+    const unsigned long long t0 = globaltimer_ns();
+    unsigned int polls = 0;
+    while (!arrived()) {
+        if ((++polls & 63u) == 0u && globaltimer_ns() - t0 > timeout_ns) {
+            atomicMax(status, 6u);                     // NUNA_ERR_TIMEOUT
+            return false;
+        }
+    }
+    return true;
+}
+
+// tv: vectors per tile, at most the block's width.  debug bits as in k_twoshot_flags: 0 and 4.
+// Up to 4 ranks the first look at the words to gather goes out together with the loads of the sources, which are few
+// (4 x 512 KiB 2.63 -> 2.35 us, 2 x 1 MiB 2.9 -> 2.55); beyond it only delays them (16 x 1 MiB 6.74 -> 7.54).
+constexpr int kTaggedEarly = 4;
+
+template <int N, int DT>
+__global__ void __launch_bounds__(kThreads, min_blocks(N <= kTaggedEarly ? N + 3 : N))
+k_twoshot_tagged(const RankPtrs p, uint4* slots, const size_t count, const unsigned tv, const unsigned lead_max, BarrierWords* bw,
+                 const unsigned long long timeout_ns, const unsigned int debug, const ParamPad<52>)
+{
+    __shared__ unsigned long long sh_ticket;
+    const size_t nvec = count / Elem<DT>::kElems;
+    const size_t ntiles = nvec ? (nvec + tv - 1) / tv : 1;         // a ragged tail rides on the last tile
+    const size_t lead = ntiles < lead_max ? ntiles : lead_max;
+    if ((debug & 16u) && blockIdx.x < ntiles && threadIdx.x < N) { // tickets come out nearly in block order
+        const size_t i0 = (size_t)blockIdx.x * tv;
+        const uint4* a = p.src[0];
+#pragma unroll
+        for (int r = 1; r < N; ++r) if ((int)threadIdx.x == r) a = p.src[r];
+        if (i0 < nvec) prefetch_l2_bulk(a + i0, (unsigned)(nvec - i0 < (size_t)tv ? nvec - i0 : (size_t)tv) * 16u);
+    }
+    if (threadIdx.x == 0) sh_ticket = draw_ticket(bw);
+    __syncthreads();
+    pdl_wait();                                                     // before the first access to the buffers or the slots
+    const size_t item = (unsigned)sh_ticket, ct = item - lead;      // tiles reduced and gathered; ct wraps where there is none
+    const unsigned tag = (unsigned)(sh_ticket >> 32) + 1u, want = tag + (debug & 1u);
+    const size_t i = item * tv + threadIdx.x, ci = ct * tv + threadIdx.x;
+    const bool produce = threadIdx.x < tv && i < nvec, consume = threadIdx.x < tv && item >= lead && ci < nvec;
+    uint4 v[N];
+    if (produce) {
+#pragma unroll
+        for (int r = 0; r < N; ++r) v[r] = ld_src(p.src[r] + i);
+    }
+    const uint4* in = slots + tagged_slot(consume ? ci : 0);
+    uint4 a, b;
+    const auto look = [&] { a = ld_tagged(in); b = ld_tagged(in + 32); };
+    const auto arrived = [&] { return a.y == want && a.w == want && b.y == want && b.w == want; };
+    if (N <= kTaggedEarly && consume) look();
+    if (produce) {
+        const uint4 o = fold_vectors<N, DT>(v);
+        uint4* out = slots + tagged_slot(i);
+        st_tagged(out, o.x, o.y, tag);
+        st_tagged(out + 32, o.z, o.w, tag);
+    }
+    const size_t e = nvec * Elem<DT>::kElems + threadIdx.x;         // element of the ragged tail
+    uint2* tail = reinterpret_cast<uint2*>(slots) + threadIdx.x;
+    if (item == ntiles - 1 && e < count) st_tagged1(tail, fold_scalar<N, DT>(p, e), tag);
+    if (consume && ((N <= kTaggedEarly && arrived()) ||
+                    poll_tagged([&] { look(); return arrived(); }, timeout_ns, &bw->status))) {
+        const uint4 o = make_uint4(a.x, a.z, b.x, b.z);
+#pragma unroll
+        for (int d = 0; d < N; ++d) st_stream(p.dst[d] + ci, o);
+    }
+    if (ct == ntiles - 1 && e < count) {
+        uint2 w;
+        if (poll_tagged([&] { w = ld_tagged1(tail); return w.y == want; }, timeout_ns, &bw->status))
+            for (int d = 0; d < N; ++d) store_elem<DT>(p.dst[d], e, w.x);
     }
     pdl_trigger();
 }

@@ -1,0 +1,120 @@
+"""The two-shot whose shard words carry their own flags: no vector at all, a ragged end only, one vector around a tile, the
+message sizes at which its shape and its range change, mixed with the other two-shot forms that draw from the same ticket
+word, replayed, and with a wait that runs out.  Bit for bit against the oracle or a rank-ordered binary32 fold in torch."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_00867_b200 import binding as nb
+from paper_2608_00867_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+
+GUARD = 64
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16", "f32"])
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 9, 16])
+def test_small_and_ragged(n, dtype):
+    code, word = nb.DTYPE_BY_NAME[dtype], np.uint16 if dtype != "f32" else np.uint32
+    size = np.dtype(word).itemsize
+    for vectors in (0, 1, 7, 8, 31, 32, 33, 64, 65, 500):
+        for ragged in (0, 1, 16 // size - 1):
+            count = vectors * (16 // size) + ragged
+            if count == 0:
+                continue
+            src = workloads.rank_buffers_typed(n, count, "normal", 5 + count, dtype)
+            src[0][: min(count, 3)] = np.array([0x7FFF, 0xFFFF, 0x7F80][: min(count, 3)] if size == 2 else
+                                               [0x7FFFFFFF, 0xFFFFFFFF, 0x7F800000][: min(count, 3)], dtype=word)
+            want = oracle.allreduce(src, dtype=dtype)[0]
+            mag = {"bf16": (0x7FFF, 0x7F80), "f16": (0x7FFF, 0x7C00), "f32": (0x7FFFFFFF, 0x7F800000)}[dtype]
+            nan = (want & word(mag[0])) > mag[1]
+            dsrc = [torch.from_numpy(a.view(np.uint8).copy()).cuda() for a in src]
+            full = [torch.full((count * size + 2 * GUARD,), 0x5A, dtype=torch.uint8, device="cuda") for _ in range(n)]
+            nb.nuna_allreduce_twoshot(dsrc, [t.data_ptr() + GUARD for t in full], count, dtype=code)
+            for t in full:
+                h = t.cpu().numpy()
+                assert (h[:GUARD] == 0x5A).all() and (h[GUARD + count * size:] == 0x5A).all(), count
+                got = h[GUARD:GUARD + count * size].view(word)
+                assert np.array_equal((got & word(mag[0])) > mag[1], nan) and np.array_equal(got[~nan], want[~nan]), count
+    assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+@pytest.mark.parametrize("n", [2, 4, 8, 16])
+def test_both_sides_of_every_line_and_every_neighbour(n):
+    """Vectors per rank around the lines of the shape and the end of the range; tagged, flagged and put calls in turn on one
+    stream, so that each draws its tickets, and writes its tags, behind the others."""
+    lines = [SMS * u for u in (8, 32, 96, 192, 224, 384, 512, 768)] + [((6 if n <= 4 else 8) << 20) // 16]   # the last: end of the range
+    top = 8 * (max(lines) + 2)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    src = [torch.randn(top, generator=gen, device="cuda").bfloat16() for _ in range(n)]
+    acc = src[0].float()
+    for s in src[1:]:
+        acc = acc + s.float()
+    want = acc.bfloat16()
+    dst = [torch.zeros(top, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    for line in lines:
+        for vectors in (line - 1, line, line + 1):
+            count = 8 * vectors + 5
+            for flags in (0, nb.NUNA_TWOSHOT_SYS_SCOPE, 0, nb.NUNA_TWOSHOT_PUT, nb.NUNA_LAUNCH_PDL | nb.NUNA_HINT_RESIDENT):
+                for d in dst:
+                    d.fill_(7.0)
+                nb.nuna_allreduce_twoshot(src, dst, count, flags=flags)
+                for d in dst:
+                    assert torch.equal(d[:count], want[:count]) and bool((d[count:count + GUARD] == 7.0).all()), (count, flags)
+    assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+@pytest.mark.parametrize("pdl", [0, nb.NUNA_LAUNCH_PDL])
+def test_back_to_back_replays_of_mixed_sizes(pdl):
+    """A captured run in which every call reads what the one before wrote, sizes alternating, replayed and mixed with eager
+    calls: a ticket drawn ahead of the wait must find the word set up by the launch before."""
+    n, sizes = 4, (64, 70001, 8, 300000, 2049, 262144)
+    top = max(sizes)
+    nb.nuna_init(4 * top + 16)
+    bufs = [[torch.zeros(top, dtype=torch.float32, device="cuda") for _ in range(n)] for _ in range(2)]
+
+    def run():
+        for k, c in enumerate(sizes):
+            nb.nuna_allreduce_twoshot(bufs[k % 2], bufs[1 - k % 2], c, dtype=nb.NUNA_F32, flags=pdl)
+
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        run()
+    for it in range(20):
+        for r in range(n):
+            bufs[0][r].fill_(r + 1)
+            bufs[1][r].zero_()
+        for _ in range(1 + it % 3):
+            g.replay() if it % 2 else run()
+            last = [b.clone() for b in bufs[0]]
+            for r in range(n):
+                bufs[0][r].fill_(r + 1)
+        smallest = min(sizes)
+        want = 10.0 * 4.0 ** (len(sizes) - 1)                       # 1 + 2 + 3 + 4, then four times itself in every further call
+        assert all(bool((b[:smallest] == want).all()) for b in last), it
+    assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+def test_wait_for_a_tag_times_out_cleanly():
+    """Consumers that wait for tags nobody writes: every wait runs out after 50 ms, the status word latches the timeout, and
+    the next ordinary calls work."""
+    w = workloads.config_decode_activation()
+    src = workloads.make(w)
+    want = oracle.allreduce(src, nthreads=4)[0]
+    dsrc = [torch.from_numpy(a.view(np.int16).copy()).cuda() for a in src]
+    dst = [torch.zeros(w.count, dtype=torch.int16, device="cuda") for _ in range(w.nranks)]
+    assert nb.debug_twoshot(dsrc, dst, w.count, timeout_ms=50, unset_flags=True, tagged=True) == nb.NUNA_OK
+    torch.cuda.synchronize()
+    assert all(not bool(d.any()) for d in dst)
+    assert nb.nuna_device_status() == nb.NUNA_ERR_TIMEOUT
+    assert nb.nuna_device_status() == nb.NUNA_OK
+    for _ in range(2):
+        nb.nuna_allreduce_twoshot(dsrc, dst, w.count)
+        for d in dst:
+            assert np.array_equal(d.cpu().numpy().view(np.uint16), want)
+    assert nb.nuna_device_status() == nb.NUNA_OK
