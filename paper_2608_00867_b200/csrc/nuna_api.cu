@@ -957,8 +957,26 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
             return launch_padded(k, pick_grid(c, o, (tiles + 1) * N, resident_blocks<k>(c), 0), stream, mode, p, shard, tiles);
         });
     }
-    const size_t shard_vec = shard / epv;
-    return dispatch(nranks, pick_unroll(o, nranks), dtype, [&](auto n_, auto u_, auto d_) -> int {
+    const size_t shard_vec = shard / epv, total = shard * elem_size(dtype) * (size_t)nranks * (size_t)nranks;
+    const int unroll = pick_unroll(o, nranks);
+    // Dependent launches without the hint, a block per tile: from 32 full tiles (64 up to 4 ranks), below which the early successor's
+    // blocks get in the way, to 128 MiB of sources, 256 beyond 8 ranks.  us, ordinary | ahead, cold, by bytes per source: 8 ranks 64 KiB
+    // 1.16 | 1.32, 128 KiB 1.63 | 1.38, 512 KiB 2.10 | 1.90, 4 MiB 6.51 | 5.66, 16 MiB 22.4 | 20.6, 32 MiB 43.2 | 43.7; 2 x 128 KiB 1.09 | 1.09, 512 KiB
+    // 1.63 | 1.30; 4 x 4 MiB 4.59 | 3.78; 16 x 4 MiB 11.4 | 9.45, 16 MiB 41.2 | 38.9.  On sources that are in L2 without the hint saying so 8 x
+    // 512 KiB 1.36 | 1.43, 1 MiB 1.69 | 1.93, 4 MiB 5.9 | 4.7.  Beyond 4 ranks blocks of 192 threads, 128 from 9 ranks, once full-width ones do
+    // not fit beside each other: they leave, and make room for the successor's, more evenly (8 x 4 MiB 5.49 | 5.31, 16 x 4 MiB 10.5 | 9.35).
+    const size_t full = ceil_div(shard_vec, (size_t)kThreads) * (size_t)nranks, sms = (size_t)c->num_sms;
+    if (mode == kLaunchPdl && !(flags & NUNA_HINT_RESIDENT) && o.prefetch != 1 && o.blocks <= 0 && unroll == 1 && full >= (nranks <= 4 ? 64 : 32) &&
+        total <= (nranks <= 8 ? (size_t)128 << 20 : (size_t)256 << 20)) {
+        const unsigned threads = nranks <= 4 || full <= sms * 4 ? (unsigned)kThreads : nranks <= 8 ? 192u : 128u;
+        const unsigned tiles = (unsigned)ceil_div(shard_vec, (size_t)threads);
+        return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
+            constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
+            t_block = threads;
+            return launch_padded(k_reduce_scatter_ahead<N, DT>, tiles * N, stream, mode, p, shard_vec, tiles, (unsigned)sms * 4u);
+        });
+    }
+    return dispatch(nranks, unroll, dtype, [&](auto n_, auto u_, auto d_) -> int {
         NUNA_NUD(n_, u_, d_);
         constexpr auto k = k_reduce_scatter<N, U, DT>;
         const size_t tiles = ceil_div(shard_vec, (size_t)kThreads * U);

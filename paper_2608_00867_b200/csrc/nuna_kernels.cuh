@@ -921,9 +921,6 @@ __device__ __forceinline__ void reduce_tile(const RankPtrs& p, uint4* out, size_
     }
 }
 
-// (No L2 prefetch ahead of the dependent-launch wait here: this kernel reads N bytes for every byte it writes and is
-// bound by the reads at every size, so the extra requests only cost -- 8 x 512 KiB 2.43 against 2.16 us, 8 x 4 MiB 7.27
-// against 6.40.)
 template <int N, int U, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N * U))
 k_reduce_scatter(const RankPtrs p, const size_t shard_vec, const size_t tiles_per_shard, const ParamPad<16>)
@@ -936,6 +933,35 @@ k_reduce_scatter(const RankPtrs p, const size_t shard_vec, const size_t tiles_pe
         reduce_tile<N, U, DT, true>(p, p.dst[r], (size_t)r * shard_vec, shard_vec, tile);
     }
     pdl_trigger();
+}
+
+// The same for a run of dependent launches on cold sources.  Bound by the reads (N bytes for every byte written): a block
+// releases the next launch as soon as its own wait returns, and the first wave's blocks ask L2 for their sources ahead of
+// that wait, so the successor's first wave comes in while this kernel's last one drains and the reads never stop.  Each alone
+// does nothing or costs (us, 8 ranks x 4 MiB of sources: neither 6.6, release only 6.7, prefetch only 6.9, both 5.3 ... 5.7; 4 x
+// 4 MiB 4.6 -> 3.7, 16 x 4 MiB 11.3 -> 9.6).  A prefetch by every block asks L2 for what the block loads at once (5.9).  Tile:
+// blockDim.x vectors.
+template <int N, int DT>
+__global__ void __launch_bounds__(kThreads, min_blocks(N))
+k_reduce_scatter_ahead(const RankPtrs p, const size_t shard_vec, const unsigned tiles_per_shard, const unsigned prefetch_blocks, const ParamPad<16>)
+{
+    const unsigned r = blockIdx.x / tiles_per_shard;
+    const size_t i0 = (size_t)(blockIdx.x - r * tiles_per_shard) * blockDim.x, off = (size_t)r * shard_vec;
+    if (blockIdx.x < prefetch_blocks && threadIdx.x < N && i0 < shard_vec) {                // thread k: source k's slice
+        const uint4* a = p.src[0];
+#pragma unroll
+        for (int k = 1; k < N; ++k) if ((int)threadIdx.x == k) a = p.src[k];
+        prefetch_l2_bulk(a + off + i0, (unsigned)(shard_vec - i0 < (size_t)blockDim.x ? shard_vec - i0 : (size_t)blockDim.x) * 16u);
+    }
+    pdl_wait();
+    pdl_trigger();
+    const size_t i = i0 + threadIdx.x;
+    if (i < shard_vec) {
+        uint4 v[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = ld_src(p.src[k] + off + i);
+        st_stream(p.dst[r] + i, fold_vectors<N, DT>(v));
+    }
 }
 
 // Any shard length.  Shard r starts `sh` bytes into a 16-byte vector of every source (the same sh in all of them), so the
