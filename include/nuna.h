@@ -93,7 +93,8 @@ typedef enum { NUNA_BF16 = 0, NUNA_F16 = 1, NUNA_F32 = 2 } nuna_dtype_t;   /* el
  * where it was measured not to pay.  Unless NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot
  * and of the put form (up to 64 MiB of sources; beyond 8 MiB the first wave only), of the flag-synchronised
  * two-shot and of the allgather and alltoall (up to 128 MiB of sources; 8 MiB beyond 8 ranks), and a block of the
- * reduce-scatter's first wave (up to 128 MiB; 256 beyond 8 ranks; whole vectors only), also asks L2, before that wait, to fetch its first tile of the sources (a prefetch returns nothing to the kernel; L2 is the
+ * reduce-scatter's first wave (whole vectors, up to 128 MiB of sources; 256 beyond 8 ranks), also asks L2, before
+ * that wait, to fetch its first tile of the sources (a prefetch returns nothing to the kernel; L2 is the
  * point of coherence, so what the predecessor still writes is what the loads after the wait see).          */
 #define NUNA_LAUNCH_PDL       64u
 /* `flags`, bit 7, with NUNA_PLACE_AWARE on nuna_allreduce_oneshot: dispatch the co-located groups through
@@ -304,10 +305,12 @@ int nuna_allreduce_oneshot(const void* const* src, void* const* dst, int nranks,
  * after acquire-polling that tile's flag (bounded wait: on expiry NUNA_ERR_TIMEOUT is latched and the block
  * returns).  A wait is only ever for an item with a smaller ticket, held by a block that already runs, so
  * the kernel needs no co-residency guarantee and no cooperative launch.  Consumed shard lines are dropped
- * from L2 (discard) instead of being written back.  Small and mid-sized messages (up to 8 MiB per rank, 6 MiB up to 4 ranks) take a
+ * from L2 (discard) instead of being written back.  Up to 4 ranks, and up to 128 MiB of sources up to 8, there is no
+ * scratch: a tile is reduced into its place in its owner's destination (owners' chunks are whole tiles) and gathered from
+ * there into the others (plain launches: at 3 and 4 ranks only).  Small and mid-sized messages (up to 8 MiB per rank, 6 MiB at 3 and 4 ranks, 5 MiB below) take a
  * form without a flag per tile: every 32-bit word of the reduced tile is stored together with the launch's
- * epoch in one 64-bit access, and the gathering block polls the words themselves, under the same bound.  It is
- * not used with NUNA_TWOSHOT_SYS_SCOPE, NUNA_OPT_TWOSHOT_VECS or NUNA_OPT_BLOCKS.  Same bits as the one-shot.  Any `count`; chunk =
+ * epoch in one 64-bit access, and the gathering block polls the words themselves, under the same bound.  Neither
+ * form is used with NUNA_TWOSHOT_SYS_SCOPE, NUNA_OPT_TWOSHOT_VECS or NUNA_OPT_BLOCKS.  Same bits as the one-shot.  Any `count`; chunk =
  * ceil(count/N) rounded up to a whole 16-byte vector, trailing chunks may be short or empty.  Uses the
  * context's shard scratch (count*elemsize bytes plus one flag word per 256 bytes, plus twice as much for up to
  * 8 MiB of it, where the words stand with their epochs; grown on demand; an

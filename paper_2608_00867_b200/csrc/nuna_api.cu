@@ -794,6 +794,13 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
 {
     const size_t bytes = count * elem_size(dtype);
     const size_t nvec = count / elems_per_vec(dtype);
+    const bool in_place = (debug_bits & 64u) != 0u;
+    // The register-thrifty instantiation, six blocks per SM instead of four: once a message is bandwidth-bound.  In place it is
+    // ahead later, with a lead of eight blocks per SM instead of six, and in tiles of 32 KiB instead of 24, 16 of 2 ranks in both (us, four |
+    // six: 2 x 16 MiB 13.6 | 14.0, 32 MiB 24.5 | 23.4, 64 MiB 44.0 | 42.9; 3 x 23 MiB 24.6 | 25.7; 4 x 16 MiB 23.5 | 24.2, 64 MiB 88.1 | 84.5;
+    // 8 x 16 MiB 42.7 | 44.5).
+    const size_t all_src = bytes * (size_t)nranks;
+    const bool many_resident = !in_place ? all_src >= ((size_t)64 << 20) : all_src > (nranks <= 2 ? (size_t)32 << 20 : (size_t)160 << 20);
     bool mid_sized = false;
     if (tv == 0) {
         // Tile bytes across all N sources, from a sweep at 8 ranks (16 ... 256 vectors per tile at every size):
@@ -813,13 +820,14 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
                                 : src_bytes <= ((size_t)8 << 20) ? (many ? 24576u : 12288u)
                                 : src_bytes <= ((size_t)14 << 20) ? (many ? 32768u : 16384u)
                                 : src_bytes <= ((size_t)16 << 20) ? 16384u : mid_sized ? 24576u : 32768u;
-        tv = tile_src / 16u / (unsigned)nranks;
+        tv = (!in_place ? tile_src : nranks <= 2 ? 16384u : many_resident ? 32768u : 24576u) / 16u / (unsigned)nranks;
     }
     tv = std::max(min_tv, std::min(tv, 2048u / (unsigned)nranks));
     tv = std::max(1u, tv / 8u * 8u);
     if (tv < min_tv) tv = min_tv;
     const size_t ntiles = std::max<size_t>(1, ceil_div(nvec, (size_t)tv));
     unsigned lead_max = (unsigned)num_sms * (mid_sized ? 5u : 8u);
+    if (in_place) lead_max = (unsigned)num_sms * (many_resident ? 8u : 6u);
     if (blocks_override > 0) lead_max = (unsigned)std::max(1, blocks_override);
     const size_t lead = std::min<size_t>(ntiles, lead_max);
     const unsigned grid = (unsigned)(ntiles + lead);
@@ -827,7 +835,7 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
         constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
         t_dyn_smem = (unsigned)N * tv * 16u;
         const unsigned mode = pdl ? kLaunchPdl : kLaunchPlain;
-        if (bytes * (size_t)nranks >= ((size_t)64 << 20))           // bandwidth-bound: trade registers for resident blocks
+        if (many_resident)
             return launch_padded(k_twoshot_flags<N, DT, 6>, grid, stream, mode, p, scratch, tile_flags, count,
                           tv, lead_max, bw, timeout_ns, debug_bits);
         return launch_padded(k_twoshot_flags<N, DT, 4>, grid, stream, mode, p, scratch, tile_flags, count, tv,
@@ -865,7 +873,7 @@ static TaggedShape tagged_shape(const Context* c, int nranks, size_t nvec)
 // bytes are beside theirs.  What asks about the flags (their scope, their tile, the shard's lines) gets the form that has them.
 static bool takes_tags(const Options& o, int nranks, size_t bytes, unsigned flags)
 {
-    return bytes <= (nranks <= 4 ? kTaggedMaxShard / 4 * 3 : kTaggedMaxShard) && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard &&
+    return bytes <= (nranks <= 2 ? kTaggedMaxShard / 8 * 5 : nranks <= 4 ? kTaggedMaxShard / 4 * 3 : kTaggedMaxShard) && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard &&
            o.twoshot_vecs <= 0 && o.blocks <= 0;
 }
 
@@ -906,6 +914,17 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
     });
 }
 
+// Whether the flag two-shot uses the owners' destinations as its shard.  us, scratch | in place, dependent launches: 2 ranks x 8 MiB
+// 9.4 | 8.4, 64 MiB 53.2 | 42.7; 3 x 23 MiB 27.8 | 25.3; 4 x 16 MiB 26.5 | 23.5, 64 MiB 92 | 84.5; 6 x 12 MB 26.5 | 25.1; 8 x 9 MiB 27.7 |
+// 26.1, 16 MiB 44.0 | 42.7, but 22 MiB 61.5 | 63.7, 6 x 24 MB 49.9 | 50.9; 12 x 10 MB 43.0 | 44.3; 16 x 12 MB 63.4 | 63.8.  Launched
+// plainly, without a prefetch: 2 x 16 MiB 17.5 | 19.5, 3 x 64 MiB 71.8 | 67.4, 4 x 16 MiB 28.0 | 26.9, 8 x 16 MiB 46.8 | 48.2.
+static bool shard_in_place(const Options& o, int nranks, size_t bytes, unsigned flags)
+{
+    const bool pays = (flags & NUNA_LAUNCH_PDL) ? nranks <= 4 || (nranks <= 8 && bytes * (size_t)nranks <= ((size_t)128 << 20))
+                                                : nranks == 3 || nranks == 4;
+    return pays && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard && o.twoshot_vecs <= 0 && o.blocks <= 0;
+}
+
 // The form whose shard words carry their own flags: a block per tile and `lead` more that only gather.
 static int launch_twoshot_tagged(const Context* c, const Options& o, const RankPtrs& p, int nranks, int dtype, size_t count, uint4* slots,
                                  unsigned long long timeout_ns, unsigned flags, unsigned debug_bits, cudaStream_t stream)
@@ -940,7 +959,8 @@ int launch_twoshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t 
     return launch_twoshot_flags(c->num_sms, o.blocks, p, nranks, dtype, count, (unsigned)std::max(0, o.twoshot_vecs), kMinFlagTileVec,
                                 scratch, tile_flags, c->bw, o.timeout_ns, (flags & NUNA_LAUNCH_PDL) != 0,
                                 (o.keep_shard ? 4u : 0u) | ((flags & NUNA_TWOSHOT_SYS_SCOPE) ? 8u : 0u) |
-                                    (prefetch_pays(o, flags, nranks, count * elem_size(dtype)) ? 16u : 0u), stream);
+                                    (prefetch_pays(o, flags, nranks, count * elem_size(dtype)) ? 16u : 0u) |
+                                    (shard_in_place(o, nranks, count * elem_size(dtype), flags) ? 64u : 0u), stream);
 }
 
 int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, size_t shard, unsigned flags,

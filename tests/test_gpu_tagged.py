@@ -1,4 +1,4 @@
-"""The two-shot whose shard words carry their own flags: no vector at all, a ragged end only, one vector around a tile, the
+"""The two-shot whose shard words carry their own flags, and the one whose shard is the owners' destinations: no vector at all, a ragged end only, one vector around a tile, the
 message sizes at which its shape and its range change, mixed with the other two-shot forms that draw from the same ticket
 word, replayed, and with a wait that runs out.  Bit for bit against the oracle or a rank-ordered binary32 fold in torch."""
 import numpy as np
@@ -46,7 +46,7 @@ def test_small_and_ragged(n, dtype):
 def test_both_sides_of_every_line_and_every_neighbour(n):
     """Vectors per rank around the lines of the shape and the end of the range; tagged, flagged and put calls in turn on one
     stream, so that each draws its tickets, and writes its tags, behind the others."""
-    lines = [SMS * u for u in (8, 32, 96, 192, 224, 384, 512, 768)] + [((6 if n <= 4 else 8) << 20) // 16]   # the last: end of the range
+    lines = [SMS * u for u in (8, 32, 96, 192, 224, 384, 512, 768)] + [((5 if n <= 2 else 6 if n <= 4 else 8) << 20) // 16]   # the last: end of the range
     top = 8 * (max(lines) + 2)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(n)
@@ -65,6 +65,35 @@ def test_both_sides_of_every_line_and_every_neighbour(n):
                 nb.nuna_allreduce_twoshot(src, dst, count, flags=flags)
                 for d in dst:
                     assert torch.equal(d[:count], want[:count]) and bool((d[count:count + GUARD] == 7.0).all()), (count, flags)
+    assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+@pytest.mark.parametrize("n,mib", [(1, 9), (2, 6), (2, 17), (3, 7), (3, 60), (4, 41), (5, 9), (7, 19), (8, 9), (8, 17)])
+def test_shard_in_the_owners_destinations(n, mib):
+    """Beyond the tagged form, on both sides of the lines where the shard moves into the destinations and its tile changes:
+    counts that end in a whole tile, in the middle of one and in the middle of a vector; eager and captured plainly."""
+    top = (mib << 20) // 2
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(mib)
+    src = [torch.randn(top, generator=gen, device="cuda").bfloat16() for _ in range(n)]
+    acc = src[0].float()
+    for s in src[1:]:
+        acc = acc + s.float()
+    want = acc.bfloat16()
+    nb.nuna_init(2 * top)
+    dst = [torch.zeros(top, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    for count in (top, top - 8 * 4096, top - 8 * 1001, top - 8 * 333 - 3):
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g):
+            nb.nuna_allreduce_twoshot(src, dst, count)
+        for call in (lambda: nb.nuna_allreduce_twoshot(src, dst, count), g.replay):
+            for d in dst:
+                d.fill_(7.0)
+            call()
+            call()
+            for d in dst:
+                assert torch.equal(d[:count], want[:count]) and bool((d[count:] == 7.0).all()), count
     assert nb.nuna_device_status() == nb.NUNA_OK
 
 
