@@ -87,7 +87,7 @@ typedef enum { NUNA_BF16 = 0, NUNA_F16 = 1, NUNA_F32 = 2 } nuna_dtype_t;   /* el
 #define NUNA_HINT_RESIDENT    32u
 /* `flags`, bit 6: launch with programmatic stream serialization and tune for it.  The kernel may be scheduled
  * while its predecessor in the stream drains; it waits for that grid's completion and memory visibility before
- * its first global access, so results are those of an ordinary stream-ordered launch.  Collectives called outside
+ * its first access to the callers' buffers, so results are those of an ordinary stream-ordered launch.  Collectives called outside
  * stream capture behave as if the flag were given; in a captured graph the edge is an ordinary one and the
  * kernel is chosen for it unless the flag is given.  The round-robin one-shot ignores it above 16 MiB of sources,
  * where it was measured not to pay.  Unless NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot

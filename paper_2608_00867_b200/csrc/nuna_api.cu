@@ -226,7 +226,7 @@ static unsigned launch_mode(unsigned flags, size_t total_src_bytes = 0)
     return ((flags & NUNA_LAUNCH_PDL) && total_src_bytes <= ((size_t)16 << 20)) ? kLaunchPdl : kLaunchPlain;
 }
 
-// The flags a collective runs with.  Every collective kernel waits for its predecessor before its first global access
+// The flags a collective runs with.  Every collective kernel waits for its predecessor before it touches the buffers
 // (pdl_wait), so it may be launched with or without the programmatic attribute with the same result, and a call that
 // goes into a stream directly gets it without asking.  A run of plain launches that the host issues faster than the
 // device drains costs a fixed 2.05 us step per kernel on B200: short kernels came out at 4.10 us each whatever their

@@ -38,12 +38,14 @@ constexpr int min_blocks(int vectors)
 // Every collective kernel opens with pdl_wait() and calls pdl_trigger() when its block has issued
 // its main work.  When a kernel is launched with programmatic stream serialization
 // (NUNA_LAUNCH_PDL) its blocks may be scheduled while the predecessor in the stream drains:
-// griddepcontrol.wait holds them, before their first global access, until the predecessor grid has
+// griddepcontrol.wait holds them, before their first access to the callers' buffers, until the predecessor grid has
 // completed and its memory operations are visible; griddepcontrol.launch_dependents, issued once a
 // block is past its main loop, lets the successor's blocks take the freed SM slots so that their
-// launch latency overlaps this kernel's tail.  (Triggering at kernel entry, or as soon as a block has
-// issued its loads, was measured slower -- 8 x 512 KiB one-shot: 3.07 against 2.81 us -- the successor's
-// waiting blocks then compete with this kernel's own blocks for slots.)
+// launch latency overlaps this kernel's tail.  The first warp of a block that issues it does so for the block: in blocks
+// wider than their tile an idle warp releases the successor right after the wait, which on cold sources is what its
+// prefetch needs (put form, 8 x 512 KiB, tiles of 56: 2.09 us in 256 threads, 2.58 in 64), and full blocks can ask for
+// (k_reduce_scatter_ahead).  (Triggering at kernel entry was measured slower -- 8 x 512 KiB one-shot: 3.07 against 2.81 us -- the
+// successor's waiting blocks then compete with this kernel's own blocks for slots.)
 // Launched normally, both instructions do nothing.
 __device__ __forceinline__ void pdl_wait()
 {
