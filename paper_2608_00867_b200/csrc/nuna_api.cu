@@ -33,9 +33,20 @@ static int env_int(const char* name, int fallback)
     return (s && *s) ? atoi(s) : fallback;
 }
 
+// Zeroes device memory that a kernel on any stream may use next: cudaMemset returns before it is done, and only the legacy
+// stream and those that wait for it come after it.  On a stream of its own it waits for nobody else's work.
+static bool zero_now(void* p, size_t bytes)
+{
+    cudaStream_t s = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
+    const bool ok = cudaMemsetAsync(p, 0, bytes, s) == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
+    cudaStreamDestroy(s);
+    return ok;
+}
+
 int init_barrier_words(Context* c)
 {
-    return cudaMemset(c->bw, 0, sizeof(BarrierWords)) == cudaSuccess ? NUNA_OK : NUNA_ERR_CUDA;
+    return zero_now(c->bw, sizeof(BarrierWords)) ? NUNA_OK : NUNA_ERR_CUDA;
 }
 
 // After a latched timeout the barrier's arrival counter is in an undefined state: zero it and clear the
@@ -96,7 +107,7 @@ int ensure_scratch(Context* c, size_t bytes)
     void* p = nullptr;
     if (cudaMalloc(&p, total) != cudaSuccess) return NUNA_ERR_CUDA;
     // flags and tags start at zero; epochs start at one, so a fresh one never reads as "ready"
-    if (cudaMemset(static_cast<char*>(p) + want, 0, total - want) != cudaSuccess) {
+    if (!zero_now(static_cast<char*>(p) + want, total - want)) {
         cudaFree(p);
         return NUNA_ERR_CUDA;
     }

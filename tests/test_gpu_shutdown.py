@@ -30,3 +30,22 @@ def test_a_call_during_shutdown_waits_and_gets_a_new_context():
     dst = [torch.zeros(64, device="cuda") for _ in range(2)]
     nb.nuna_allreduce(src, dst, 64, dtype=nb.NUNA_F32)
     assert all(bool((d == 1.0).all()) for d in dst) and nb.nuna_device_status() == nb.NUNA_OK
+
+
+def test_the_first_calls_after_shutdown_on_a_stream_of_their_own():
+    """A new context's control words, flags and tags are zeroed before a stream that waits for no other may use them: the
+    memory may be what an earlier context's last launches wrote, and its epochs start over."""
+    n, count = 4, 1 << 20
+    src = [torch.full((count,), float(r + 1), device="cuda") for r in range(n)]
+    dst = [torch.zeros(count, device="cuda") for _ in range(n)]
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(8):
+        assert nb.lib().nuna_shutdown() == nb.NUNA_OK
+        with torch.cuda.stream(stream):
+            for d in dst:
+                d.zero_()
+            nb.nuna_allreduce_twoshot(src, dst, count, dtype=nb.NUNA_F32)
+            nb.nuna_allreduce_twoshot(src, dst, count, dtype=nb.NUNA_F32, flags=nb.NUNA_TWOSHOT_SYS_SCOPE)
+        assert nb.nuna_device_status() == nb.NUNA_OK
+        assert all(bool((d == 10.0).all()) for d in dst)
