@@ -846,11 +846,11 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
         constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;
         t_dyn_smem = (unsigned)N * tv * 16u;
         const unsigned mode = pdl ? kLaunchPdl : kLaunchPlain;
-        if (many_resident)
-            return launch_padded(k_twoshot_flags<N, DT, 6>, grid, stream, mode, p, scratch, tile_flags, count,
-                          tv, lead_max, bw, timeout_ns, debug_bits);
-        return launch_padded(k_twoshot_flags<N, DT, 4>, grid, stream, mode, p, scratch, tile_flags, count, tv,
-                      lead_max, bw, timeout_ns, debug_bits);
+        const auto go = [&](auto kernel) {
+            return launch_padded(kernel, grid, stream, mode, p, scratch, tile_flags, count, tv, lead_max, bw, timeout_ns, debug_bits);
+        };
+        if constexpr (N <= 8) { if (in_place) return go(many_resident ? k_twoshot_flags<N, DT, 6, true> : k_twoshot_flags<N, DT, 4, true>); }
+        return go(many_resident ? k_twoshot_flags<N, DT, 6, false> : k_twoshot_flags<N, DT, 4, false>);
     });
 }
 

@@ -1460,23 +1460,25 @@ __device__ __forceinline__ void half_sync(int id) { asm volatile("bar.sync %0, 1
 // tv: vectors per tile; shared memory = N * tv * 16 bytes.  lead_max: upper bound of `lead`.
 // mode bits: 0 in normal use; bit 0: consumers wait for a flag value nobody publishes (test of the bounded
 // wait); bit 2: keep consumed shard lines in L2 (for measuring what the discard saves); bit 3: flags are
-// released and acquired at system scope (NUNA_TWOSHOT_SYS_SCOPE); bit 6: in place -- the shard of a tile is its place in its
-// owner's destination (the owners' chunks are whole tiles), scratch is not used and the gathering block stores to the N - 1 others.
+// released and acquired at system scope (NUNA_TWOSHOT_SYS_SCOPE).
+// kInPlace: the shard of a tile is its place in its owner's destination (the owners' chunks are whole tiles), scratch is not
+// used and the gathering block stores to the N - 1 others.  A template argument: read at run time it costs the scratch form its
+// registers (8 x 36 MiB 98.3 -> 102 us).
 // That saves the shard's writes to L2, which count the more the fewer the ranks (2 x 64 MiB 53.2 -> 42.9 us, 3 x 23 MiB 28.4 -> 24.6,
 // 8 x 16 MiB 44.4 -> 42.7; but 8 x 64 MiB 167 -> 170).
 // kMinBlocks: resident blocks per SM the register allocation is held to.  4 (64 registers) gives the shortest
 // path per block, best while the message is small enough for latency to dominate (8 KiB per rank: 3.4 us
 // against 3.7 us).  6 holds it to 40 registers: more tiles in flight per SM, which is what counts once the
 // message is bandwidth-bound (measured at 8 ranks: 16 MiB per rank 48.7 -> 45.6 us).
-template <int N, int DT, int kMinBlocks>
+template <int N, int DT, int kMinBlocks, bool kInPlace>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
 k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const size_t count, const unsigned tv,
                 const unsigned lead_max, BarrierWords* bw, const unsigned long long timeout_ns, const unsigned int debug, const ParamPad<44>)
 {
     constexpr unsigned kHalf = kThreads / 2;
     const unsigned wait_bias = debug & 1u;
-    const bool discard_shard = (debug & 68u) == 0u;
-    const bool sys_scope = (debug & 8u) != 0u, in_place = (debug & 64u) != 0u;
+    const bool discard_shard = !kInPlace && (debug & 4u) == 0u;
+    const bool sys_scope = (debug & 8u) != 0u;
     extern __shared__ __align__(128) unsigned char stage_raw[];
     uint4* stage = reinterpret_cast<uint4*>(stage_raw);            // [N][tv]
     __shared__ __align__(8) uint64_t bar;
@@ -1500,14 +1502,14 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
     __syncthreads();
     const size_t item = (unsigned)sh_ticket;
     const unsigned epoch1 = (unsigned)(sh_ticket >> 32) + 1u;
-    const size_t chunk = (ntiles + N - 1) / N;                      // tiles of one owner, in place
+    const size_t chunk = kInPlace ? (ntiles + N - 1) / N : 1;       // tiles of one owner
     const bool produce = item < ntiles, consume = item >= lead && item < ntiles + lead;
 
     if (threadIdx.x < kHalf) {
         // ---- produce half ----
         if (produce) {
             const size_t pbase = item * tv;
-            uint4* shard = in_place ? p.dst[item / chunk] : scratch;
+            uint4* shard = kInPlace ? p.dst[item / chunk] : scratch;
             const unsigned pnv = pbase < nvec ? (unsigned)((nvec - pbase < tv) ? nvec - pbase : tv) : 0u;
             bool landed = true;
             if (pnv != 0u) {
@@ -1540,8 +1542,8 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
         // ---- consume half ----
         if (consume) {
             const size_t ct = item - lead, cbase = ct * tv;
-            const int own = in_place ? (int)(ct / chunk) : -1;       // the destination that has the tile already
-            const uint4* shard = in_place ? p.dst[own] : scratch;
+            const int own = kInPlace ? (int)(ct / chunk) : -1;       // the destination that has the tile already
+            const uint4* shard = kInPlace ? p.dst[own] : scratch;
             if (threadIdx.x == kHalf)
                 sh_ok = wait_flag(flags + ct, epoch1 + wait_bias, timeout_ns, &bw->status, sys_scope) ? 1 : 0;
             half_sync(2);                              // flag acquired by one thread -> every thread may read the tile
@@ -1550,7 +1552,7 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
                 for (unsigned j = threadIdx.x - kHalf; j < cnv; j += kHalf) {
                     const uint4 c = ld_cg(shard + cbase + j);
 #pragma unroll
-                    for (int d = 0; d < N; ++d) if (d != own) st_stream(p.dst[d] + cbase + j, c);
+                    for (int d = 0; d < N; ++d) if (!kInPlace || d != own) st_stream(p.dst[d] + cbase + j, c);
                 }
                 // The tile has exactly one consumer, so its shard lines are dead now: drop them from L2
                 // instead of letting them be written back to DRAM (whole, 128-byte aligned lines only).
@@ -1563,7 +1565,7 @@ k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const siz
                     const size_t e = tail0 + (threadIdx.x - kHalf);
                     if (e < count) {
                         const uint32_t w = load_elem_cg<DT>(shard, e);
-                        for (int d = 0; d < N; ++d) if (d != own) store_elem<DT>(p.dst[d], e, w);
+                        for (int d = 0; d < N; ++d) if (!kInPlace || d != own) store_elem<DT>(p.dst[d], e, w);
                     }
                 }
             }
