@@ -361,8 +361,8 @@ int nuna_alltoall(const void* const* src, void* const* dst, int nranks,
  *  - Limit: 4 MiB per rank, i.e. count <= NUNA_STATIC_MAX_COUNT elements of a 16-bit type (half that
  *    many of binary32); larger messages return NUNA_ERR_TOO_LARGE and print the limit.  The array
  *    costs 4 MiB of device memory on every GPU that loads the library, for the life of the process.
- *  - The first call on a device looks up the arrays' device addresses and zeroes the flags and control
- *    words (two small synchronous cudaMemset calls); make that first call before starting any stream capture.
+ *  - The first call on a device looks up the arrays' device addresses (flags and control words are zero from
+ *    the load of the library on); make that first call before starting any stream capture.
  *  - All calls on a device share the one array, which keeps the previous call's shard; the kernel
  *    overwrites every element it later reads, so stale contents never reach a result.  Two calls that
  *    overlap on the GPU (different streams, no ordering) race on it: keep calls stream-ordered.

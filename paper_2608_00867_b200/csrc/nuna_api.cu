@@ -1682,7 +1682,10 @@ struct StaticSetup {
 static StaticSetup g_static_setup[kMaxDevices];
 static std::mutex g_static_mutex;
 
-// Once per device: resolve the symbols and zero the control words and ready flags.  No allocation.
+// Once per device: resolve the symbols.  No allocation, and nothing is written: epoch, ticket and ready flags are zero from the
+// moment the module is loaded (device variables without an initialiser), before any stream can use them.  A memset here would
+// return before it is done, and would come after nobody but the legacy stream: on another one it could take back tickets that
+// the call's blocks have drawn.  The shard needs no clearing (every element is written before it is read).
 static int static_setup(StaticSetup** out)
 {
     int dev = -1;
@@ -1698,10 +1701,6 @@ static int static_setup(StaticSetup** out)
         if (cudaGetSymbolAddress(&barrier, g_static_barrier) != cudaSuccess || !barrier) return NUNA_ERR_CUDA;
         if (cudaDeviceGetAttribute(&s.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || s.num_sms < 1)
             return NUNA_ERR_CUDA;
-        // epoch, cursor and departure counter start from zero, and no tile may read as ready; the shard
-        // needs no clearing (every element is written before it is read)
-        if (cudaMemset(barrier, 0, sizeof(BarrierWords)) != cudaSuccess) return NUNA_ERR_CUDA;
-        if (cudaMemset(flags, 0, sizeof(g_static_flags)) != cudaSuccess) return NUNA_ERR_CUDA;
         s.shard = static_cast<uint4*>(shard);
         s.flags = static_cast<unsigned*>(flags);
         s.barrier = static_cast<BarrierWords*>(barrier);

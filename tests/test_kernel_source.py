@@ -18,3 +18,17 @@ def test_no_non_coherent_loads():
     for the kernel's lifetime, which ld.global.nc (and __ldg, and loads the compiler derives from const __restrict__) ask."""
     found = [at for at, code in device_code() if re.search(r"\bld\.global(\.\w+)*\.nc\b|__ldg\b|__restrict__", code)]
     assert not found, found
+
+
+def host_functions():
+    """(where, text) of every function of the host code, cut at the lines that start in the first column."""
+    with open(os.path.join(CSRC, "nuna_api.cu")) as f:
+        for text in re.split(r"\n(?=[a-z])", re.sub(r"//.*", "", f.read())):
+            yield text.split("\n", 1)[0], text
+
+
+def test_control_words_are_not_set_behind_the_streams_back():
+    """cudaMemset returns before it is done, and only the legacy stream and those that wait for it come after it: what a kernel
+    on any other stream may use next cannot be cleared that way.  The measuring hooks launch on the legacy stream itself."""
+    found = [at for at, text in host_functions() if re.search(r"\bcudaMemset\(", text) and "nuna_debug_" not in at]
+    assert not found, found
