@@ -33,16 +33,20 @@ static int env_int(const char* name, int fallback)
     return (s && *s) ? atoi(s) : fallback;
 }
 
-// Zeroes device memory that a kernel on any stream may use next: cudaMemset returns before it is done, and only the legacy
-// stream and those that wait for it come after it.  On a stream of its own it waits for nobody else's work.
-static bool zero_now(void* p, size_t bytes)
+// Sets device memory that a kernel on any stream may use next, to zero or to what `host` holds: cudaMemset, and cudaMemcpy from
+// pageable memory, return before they are done, and only the legacy stream and those that wait for it come after them.  On a
+// stream of its own it waits for nobody else's work.
+static bool set_now(void* p, const void* host, size_t bytes)
 {
     cudaStream_t s = nullptr;
     if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
-    const bool ok = cudaMemsetAsync(p, 0, bytes, s) == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
+    const cudaError_t e = host ? cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, s) : cudaMemsetAsync(p, 0, bytes, s);
+    const bool ok = cudaStreamSynchronize(s) == cudaSuccess && e == cudaSuccess;
     cudaStreamDestroy(s);
     return ok;
 }
+
+static bool zero_now(void* p, size_t bytes) { return set_now(p, nullptr, bytes); }
 
 int init_barrier_words(Context* c)
 {
@@ -57,7 +61,7 @@ static int rewind_barrier_words(BarrierWords* dev, const BarrierWords& seen)
     BarrierWords h = {};
     h.epoch = seen.epoch + 1u;
     h.ticket = ((seen.ticket >> 32) + 1ull) << 32;
-    return cudaMemcpy(dev, &h, sizeof h, cudaMemcpyHostToDevice) == cudaSuccess ? NUNA_OK : NUNA_ERR_CUDA;
+    return set_now(dev, &h, sizeof h) ? NUNA_OK : NUNA_ERR_CUDA;
 }
 
 // Returns the current device's context, creating it on first use (allocates: not capturable).

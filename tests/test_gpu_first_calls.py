@@ -4,6 +4,9 @@ import subprocess
 import sys
 
 import pytest
+import torch
+
+from paper_2608_00867_b200 import binding as nb
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +31,23 @@ assert nb.nuna_device_status() == nb.NUNA_OK
 """
     done = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert done.returncode == 0, done.stderr[-2000:]
+
+
+def test_calls_behind_a_rewind_on_a_stream_of_their_own():
+    """A wait that runs out leaves the ticket word rewound by nuna_device_status; the next calls draw from it at once."""
+    n, count = 4, 1 << 18
+    src = [torch.full((count,), float(r + 1), device="cuda") for r in range(n)]
+    dst = [torch.zeros(count, device="cuda") for _ in range(n)]
+    stream = torch.cuda.Stream()
+    for tagged in (False, True):
+        for _ in range(4):
+            assert nb.debug_twoshot(src, dst, count, dtype=nb.NUNA_F32, timeout_ms=20, unset_flags=True, tagged=tagged) == nb.NUNA_OK
+            assert nb.nuna_device_status() == nb.NUNA_ERR_TIMEOUT
+            with torch.cuda.stream(stream):
+                for d in dst:
+                    d.zero_()
+                nb.nuna_allreduce_twoshot(src, dst, count, dtype=nb.NUNA_F32)
+                nb.nuna_allreduce_twoshot(src, dst, count, dtype=nb.NUNA_F32, flags=nb.NUNA_TWOSHOT_SYS_SCOPE)
+            torch.cuda.synchronize()
+            assert all(bool((d == 10.0).all()) for d in dst)
+            assert nb.nuna_device_status() == nb.NUNA_OK
