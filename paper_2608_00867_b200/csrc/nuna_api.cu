@@ -515,7 +515,7 @@ static int get_sm_plan(Context* c, int nranks, size_t nvec, int coloc, int domai
         const size_t cur0 = off.size() + std::max<size_t>(tiles.size(), 1);
         pl.nonempty = 0;
         for (int s = 0; s < c->num_sms; ++s) pl.nonempty += !lists[s].empty();
-        if (cudaMemcpy(d, host.data(), words * sizeof(unsigned), cudaMemcpyHostToDevice) != cudaSuccess) {
+        if (!set_now(d, host.data(), words * sizeof(unsigned))) {
             cudaFree(d);
             return NUNA_ERR_CUDA;
         }

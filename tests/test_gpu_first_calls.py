@@ -51,3 +51,18 @@ def test_calls_behind_a_rewind_on_a_stream_of_their_own():
             torch.cuda.synchronize()
             assert all(bool((d == 10.0).all()) for d in dst)
             assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+def test_the_first_call_with_work_lists_on_a_stream_of_its_own():
+    """The lists of a new shape are built and sent during the call that then reads them."""
+    flags = nb.NUNA_PLACE_AWARE | nb.NUNA_PLACE_SM_LISTS
+    stream = torch.cuda.Stream()
+    for n, count in ((4, 8 * 70001), (8, 8 * 30011), (2, 8 * 150007)):
+        src = [torch.full((count,), float(r + 1), device="cuda") for r in range(n)]
+        dst = [torch.zeros(count, device="cuda") for _ in range(n)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            nb.nuna_allreduce_oneshot(src, dst, count, dtype=nb.NUNA_F32, flags=flags)
+        torch.cuda.synchronize()
+        assert all(bool((d == n * (n + 1) / 2).all()) for d in dst)
+    assert nb.nuna_device_status() == nb.NUNA_OK

@@ -27,11 +27,10 @@ def host_functions():
             yield text.split("\n", 1)[0], text
 
 
-def test_control_words_are_not_set_behind_the_streams_back():
-    """cudaMemset returns before it is done, and only the legacy stream and those that wait for it come after it: what a kernel
-    on any other stream may use next cannot be cleared that way, nor rewound by cudaMemcpy out of pageable memory.  The
-    measuring hooks launch on the legacy stream itself."""
-    behind = {"rewind_barrier_words": r"\bcudaMem(set|cpy)\("}
+def test_device_tables_are_not_set_behind_the_streams_back():
+    """cudaMemset, and cudaMemcpy out of pageable memory, return before they are done, and only the legacy stream and those that
+    wait for it come after them: control words, flags and work lists, which a kernel on any other stream may use next, cannot
+    be set that way.  The measuring hooks launch on the legacy stream itself."""
     found = [at for at, text in host_functions() if "nuna_debug_" not in at and
-             re.search(next((p for name, p in behind.items() if name in at), r"\bcudaMemset\("), text)]
+             re.search(r"\bcudaMemset\(|\bcudaMemcpy\([^;]*HostToDevice", text)]
     assert not found, found
