@@ -312,9 +312,9 @@ int nuna_allreduce_oneshot(const void* const* src, void* const* dst, int nranks,
  * epoch in one 64-bit access, and the gathering block polls the words themselves, under the same bound.  Neither
  * form is used with NUNA_TWOSHOT_SYS_SCOPE, NUNA_OPT_TWOSHOT_VECS or NUNA_OPT_BLOCKS.  Same bits as the one-shot.  Any `count`; chunk =
  * ceil(count/N) rounded up to a whole 16-byte vector, trailing chunks may be short or empty.  Uses the
- * context's shard scratch (count*elemsize bytes plus one flag word per 256 bytes, plus twice as much for up to
- * 8 MiB of it, where the words stand with their epochs; grown on demand; an
- * outgrown scratch stays allocated until nuna_shutdown because captured graphs may still name it) unless
+ * context's shard scratch (count*elemsize bytes plus one flag word per 256 bytes, and the slots where words stand
+ * with their epochs: twice the next power of two, at most 16 MiB; grown on demand; what is outgrown stays
+ * allocated until nuna_shutdown because captured graphs may still name it) unless
  * NUNA_TWOSHOT_PUT is set.  Calls that share the context must be stream-ordered with respect to each other. */
 int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,
                            size_t count, int dtype, unsigned flags, void* stream);

@@ -98,27 +98,32 @@ int get_context(Context** out)
     return NUNA_OK;
 }
 
-// Grows the two-shot scratch: shard intermediate, one ready flag per smallest tile of it, and the slots of the tagged form
+// Grows the two-shot scratch: shard intermediate with one ready flag per smallest tile of it, and the slots of the tagged form
 // for as large a shard as that form takes.  The caller holds c->mutex.  An outgrown allocation is never freed before nuna_shutdown: a CUDA graph captured earlier
-// (a chain, or a user's capture of a two-shot call) still carries its address as a kernel argument.
+// (a chain, or a user's capture of a two-shot call) still carries its address as a kernel argument.  The slots, twice their
+// shard's bytes, are therefore an allocation of their own that doubles: what has been outgrown is never more than the last.
 int ensure_scratch(Context* c, size_t bytes)
 {
     if (bytes <= c->scratch_bytes && c->scratch) return NUNA_OK;
-    const size_t want = (std::max<size_t>(bytes, 4096) + 4095) & ~(size_t)4095;
-    const size_t nflags = want / (kMinFlagTileVec * 16) + 1;         // one ready flag per smallest tile
-    const size_t slots_at = (want + nflags * sizeof(unsigned) + 255) & ~(size_t)255;
-    const size_t total = slots_at + tagged_bytes(std::min(want, kTaggedMaxShard));
-    void* p = nullptr;
-    if (cudaMalloc(&p, total) != cudaSuccess) return NUNA_ERR_CUDA;
     // flags and tags start at zero; epochs start at one, so a fresh one never reads as "ready"
-    if (!zero_now(static_cast<char*>(p) + want, total - want)) {
-        cudaFree(p);
-        return NUNA_ERR_CUDA;
+    const auto grow = [c](void** at, size_t data, size_t zeroed) {
+        void* p = nullptr;
+        if (cudaMalloc(&p, data + zeroed) != cudaSuccess) return false;
+        if (!zero_now(static_cast<char*>(p) + data, zeroed)) { cudaFree(p); return false; }
+        if (*at) c->retired_scratch.push_back(*at);
+        *at = p;
+        return true;
+    };
+    const size_t want = (std::max<size_t>(bytes, 4096) + 4095) & ~(size_t)4095;
+    size_t slots_shard = 64 << 10;
+    while (slots_shard < std::min(want, kTaggedMaxShard)) slots_shard *= 2;
+    if (slots_shard > c->slots_shard) {
+        if (!grow(&c->slots, 0, tagged_bytes(slots_shard))) return NUNA_ERR_CUDA;
+        c->slots_shard = slots_shard;
     }
-    if (c->scratch) c->retired_scratch.push_back(c->scratch);
-    c->scratch = p;
-    c->flags = reinterpret_cast<unsigned*>(static_cast<char*>(p) + want);
-    c->slots = static_cast<char*>(p) + slots_at;
+    const size_t nflags = want / (kMinFlagTileVec * 16) + 1;         // one ready flag per smallest tile
+    if (!grow(&c->scratch, want, nflags * sizeof(unsigned))) return NUNA_ERR_CUDA;
+    c->flags = reinterpret_cast<unsigned*>(static_cast<char*>(c->scratch) + want);
     c->scratch_bytes = want;
     return NUNA_OK;
 }
@@ -1503,6 +1508,7 @@ int nuna_shutdown(void)
     cudaDeviceSynchronize();
     if (c->bw) cudaFree(c->bw);
     if (c->scratch) cudaFree(c->scratch);
+    if (c->slots) cudaFree(c->slots);
     for (void* d : c->retired_scratch) cudaFree(d);
     if (c->staging) cudaFree(c->staging);
     if (c->stream) cudaStreamDestroy(c->stream);

@@ -51,9 +51,10 @@ struct Context {
     BarrierWords* bw = nullptr;          // flag-barrier words, work cursor, epoch + latched status, device memory
     void* scratch = nullptr;             // two-shot shard intermediate, followed by its per-tile ready flags
     unsigned* flags = nullptr;           // one word per smallest tile of the scratch (inside the same allocation)
-    void* slots = nullptr;               // slots of the tagged two-shot (inside the same allocation)
     size_t scratch_bytes = 0;
-    std::vector<void*> retired_scratch;  // outgrown scratch allocations: captured graphs may still name them
+    void* slots = nullptr;               // slots of the tagged two-shot, device memory
+    size_t slots_shard = 0;              // bytes of the largest shard they hold
+    std::vector<void*> retired_scratch;  // outgrown scratch and slots: captured graphs may still name them
     void* staging = nullptr;             // device copies of host buffers (nuna_allreduce_host)
     size_t staging_bytes = 0;
     cudaStream_t stream = nullptr;       // private stream of the host-buffer entry point
