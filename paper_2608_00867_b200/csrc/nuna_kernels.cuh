@@ -68,6 +68,10 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* g, unsigned bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(g), "r"(bytes) : "memory");
 }
 
+// The same for the one line that holds `g`.  Requests of their own for every line are in nobody's way for long: behind a kernel
+// that is not the library's, whose end the wait finds already there, a block's loads queue behind what it has just asked for.
+__device__ __forceinline__ void prefetch_l2_line(const void* g) { asm volatile("prefetch.global.L2 [%0];" :: "l"(g) : "memory"); }
+
 // Nanoseconds of the device-wide timer (bounds every in-kernel wait; timestamps of the measurement aids).
 __device__ __forceinline__ unsigned long long globaltimer_ns()
 {
@@ -938,26 +942,26 @@ k_reduce_scatter(const RankPtrs p, const size_t shard_vec, const size_t tiles_pe
 }
 
 // The same for a run of dependent launches on cold sources.  Bound by the reads (N bytes for every byte written): a block
-// releases the next launch as soon as its own wait returns, and the first wave's blocks ask L2 for their sources ahead of
-// that wait, so the successor's first wave comes in while this kernel's last one drains and the reads never stop.  Each alone
-// does nothing or costs (us, 8 ranks x 4 MiB of sources: neither 6.6, release only 6.7, prefetch only 6.9, both 5.3 ... 5.7; 4 x
-// 4 MiB 4.6 -> 3.7, 16 x 4 MiB 11.3 -> 9.6).  A prefetch by every block asks L2 for what the block loads at once (5.9).  Tile:
-// blockDim.x vectors.
+// releases the next launch as soon as its own wait returns, and the first 4 blocks per SM ask L2 for their sources ahead of
+// that wait, so the successor's first blocks' data comes in while this kernel's last ones drain and the reads never stop.  Each
+// alone does nothing or costs (us, 8 ranks x 4 MiB of sources: neither 6.30, release only 6.38, prefetch only 7.05, both 5.5 ... 5.7;
+// 4 x 4 MiB 4.44, 4.43, 4.66, 3.66; 16 x 4 MiB 10.9 -> 9.3).  A prefetch by every block asks L2 for what the block loads at once (5.9).
+// Line by line, every eighth thread for the line where it will load (bulk requests | lines: 8 x 1 MiB 2.54 | 2.42, 16 x 2 MiB 6.55 |
+// 5.67; behind a kernel that has nothing to do with these sources 8 x 128 KiB 9.52 | 8.88, without a prefetch 8.86, 8 x 4 MiB
+// 15.10 | 14.70, 14.38; behind one that has just written them, 16 x 2 MiB 18.6 | 16.9, 16.2; all with that kernel's time).
+// Tile: blockDim.x vectors.
 template <int N, int DT>
 __global__ void __launch_bounds__(kThreads, min_blocks(N))
 k_reduce_scatter_ahead(const RankPtrs p, const size_t shard_vec, const unsigned tiles_per_shard, const unsigned prefetch_blocks, const ParamPad<16>)
 {
     const unsigned r = blockIdx.x / tiles_per_shard;
-    const size_t i0 = (size_t)(blockIdx.x - r * tiles_per_shard) * blockDim.x, off = (size_t)r * shard_vec;
-    if (blockIdx.x < prefetch_blocks && threadIdx.x < N && i0 < shard_vec) {                // thread k: source k's slice
-        const uint4* a = p.src[0];
+    const size_t i = (size_t)(blockIdx.x - r * tiles_per_shard) * blockDim.x + threadIdx.x, off = (size_t)r * shard_vec;
+    if (blockIdx.x < prefetch_blocks && (threadIdx.x & 7u) == 0u && i < shard_vec) {
 #pragma unroll
-        for (int k = 1; k < N; ++k) if ((int)threadIdx.x == k) a = p.src[k];
-        prefetch_l2_bulk(a + off + i0, (unsigned)(shard_vec - i0 < (size_t)blockDim.x ? shard_vec - i0 : (size_t)blockDim.x) * 16u);
+        for (int k = 0; k < N; ++k) prefetch_l2_line(p.src[k] + off + i);
     }
     pdl_wait();
     pdl_trigger();
-    const size_t i = i0 + threadIdx.x;
     if (i < shard_vec) {
         uint4 v[N];
 #pragma unroll
