@@ -92,10 +92,12 @@ typedef enum { NUNA_BF16 = 0, NUNA_F16 = 1, NUNA_F32 = 2 } nuna_dtype_t;   /* el
  * kernel is chosen for it unless the flag is given.  The round-robin one-shot ignores it above 16 MiB of sources,
  * where it was measured not to pay.  Unless NUNA_HINT_RESIDENT is set, a block of the register-sharing one-shot
  * and of the put form (up to 64 MiB of sources; beyond 8 MiB the first wave only), of the flag-synchronised
- * two-shot and of the allgather and alltoall (up to 128 MiB of sources; 8 MiB beyond 8 ranks), and a block of the
- * reduce-scatter's first wave (whole vectors, up to 128 MiB of sources; 256 beyond 8 ranks), also asks L2, before
- * that wait, to fetch its first tile of the sources (a prefetch returns nothing to the kernel; L2 is the
- * point of coherence, so what the predecessor still writes is what the loads after the wait see).          */
+ * two-shot and of the allgather and alltoall (up to 128 MiB of sources; 8 MiB beyond 8 ranks), and each of the
+ * reduce-scatter's first blocks, four per SM (whole vectors, from 32 tiles of 4 KiB, 64 up to 4 ranks, to 128 MiB of
+ * sources; 256 beyond 8 ranks), also asks L2, before that wait, to fetch its first tile of the sources (a prefetch
+ * returns nothing to the kernel; L2 is the point of coherence, so what the predecessor still writes is what the
+ * loads after the wait see).  Reduce-scatters of less than 32 MiB of sources, 48 beyond 8 ranks, do so only if the flag
+ * is given: it pays in runs of the library's own launches on sources that are not in L2.                    */
 #define NUNA_LAUNCH_PDL       64u
 /* `flags`, bit 7, with NUNA_PLACE_AWARE on nuna_allreduce_oneshot: dispatch the co-located groups through
  * per-SM work lists.  The lists are planned by Algorithm 1 from the topology the last

@@ -983,7 +983,8 @@ int launch_twoshot(Context* c, const RankPtrs& p, int nranks, int dtype, size_t 
                                     (shard_in_place(o, nranks, count * elem_size(dtype), flags) ? 64u : 0u), stream);
 }
 
-int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, size_t shard, unsigned flags,
+// `asked`: the caller gave NUNA_LAUNCH_PDL itself.
+int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, size_t shard, unsigned flags, bool asked,
                           cudaStream_t stream)
 {
     const Options o = snapshot(c);
@@ -999,14 +1000,22 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
     }
     const size_t shard_vec = shard / epv, total = shard * elem_size(dtype) * (size_t)nranks * (size_t)nranks;
     const int unroll = pick_unroll(o, nranks);
-    // Dependent launches without the hint, a block per tile: from 32 full tiles (64 up to 4 ranks), below which the early successor's
-    // blocks get in the way, to 128 MiB of sources, 256 beyond 8 ranks.  us, ordinary | ahead, cold, by bytes per source: 8 ranks 64 KiB
-    // 1.16 | 1.32, 128 KiB 1.63 | 1.38, 512 KiB 2.10 | 1.90, 4 MiB 6.51 | 5.66, 16 MiB 22.4 | 20.6, 32 MiB 43.2 | 43.7; 2 x 128 KiB 1.09 | 1.09, 512 KiB
-    // 1.63 | 1.30; 4 x 4 MiB 4.59 | 3.78; 16 x 4 MiB 11.4 | 9.45, 16 MiB 41.2 | 38.9.  On sources that are in L2 without the hint saying so 8 x
-    // 512 KiB 1.36 | 1.43, 1 MiB 1.69 | 1.93, 4 MiB 5.9 | 4.7.  Beyond 4 ranks blocks of 192 threads, 128 from 9 ranks, once full-width ones do
+    // The form that works ahead.  A caller who asks for dependent launches, and does not say that the sources are in L2, gets it from
+    // 32 full tiles (64 up to 4 ranks), below which the early successor's blocks get in the way, to 128 MiB of sources, 256 beyond 8
+    // ranks.  us, ordinary | ahead, in a run of such calls on cold sources, by bytes per source: 8 ranks 64 KiB 1.16 | 1.32, 128 KiB
+    // 1.73 | 1.34, 512 KiB 2.20 | 1.86, 4 MiB 6.38 | 5.51, 16 MiB 21.7 | 20.5, 32 MiB 43.2 | 43.7; 2 x 128 KiB 1.21 | 1.16, 512 KiB 1.70 | 1.27;
+    // 4 x 4 MiB 4.49 | 3.66; 16 x 1 MiB 4.01 | 4.05, 4 MiB 10.9 | 9.3, 16 MiB 39.7 | 39.0.
+    // Nothing is known of what stands before any other call.  If its sources are in L2 all the same (8 x 512 KiB 1.37 | 1.40, 1 MiB
+    // 1.71 | 1.93, 2 MiB 2.38 | 2.54, but 4 MiB 5.44 | 4.50, 8 MiB 10.7 | 9.4), or a kernel that does not release early comes before it
+    // (with that kernel's time, one that writes the sources, and one that writes elsewhere: 8 x 1 MiB 6.98 | 7.29, 9.99 | 10.65, 4 MiB
+    // 16.41 | 16.74, 14.38 | 14.70, 8 MiB 28.24 | 28.57, 20.32 | 20.14; 4 x 4 MiB 10.54 | 10.74, 11.50 | 11.97, 8 MiB 17.06 | 17.22, 14.94 | 15.06;
+    // 16 x 2 MiB 16.24 | 16.93, 13.86 | 14.56, 3 MiB 22.13 | 22.39, 16.50 | 16.61), it costs up to 2 % from 32 MiB of sources, 48 beyond 8
+    // ranks, and up to 15 % below.
+    // Beyond 4 ranks blocks of 192 threads, 128 from 9 ranks, once full-width ones do
     // not fit beside each other: they leave, and make room for the successor's, more evenly (8 x 4 MiB 5.49 | 5.31, 16 x 4 MiB 10.5 | 9.35).
     const size_t full = ceil_div(shard_vec, (size_t)kThreads) * (size_t)nranks, sms = (size_t)c->num_sms;
-    if (mode == kLaunchPdl && !(flags & NUNA_HINT_RESIDENT) && o.prefetch != 1 && o.blocks <= 0 && unroll == 1 && full >= (nranks <= 4 ? 64 : 32) &&
+    const bool ahead = asked ? full >= (nranks <= 4 ? 64 : 32) : total >= (nranks <= 8 ? (size_t)32 << 20 : (size_t)48 << 20);
+    if (ahead && mode == kLaunchPdl && !(flags & NUNA_HINT_RESIDENT) && o.prefetch != 1 && o.blocks <= 0 && unroll == 1 &&
         total <= (nranks <= 8 ? (size_t)128 << 20 : (size_t)256 << 20)) {
         const unsigned threads = nranks <= 4 || full <= sms * 4 ? (unsigned)kThreads : nranks <= 8 ? 192u : 128u;
         const unsigned tiles = (unsigned)ceil_div(shard_vec, (size_t)threads);
@@ -1335,7 +1344,8 @@ int nuna_reduce_scatter(const void* const* src, void* const* dst, int nranks, si
     if (flags & NUNA_TWOSHOT_PUT) return NUNA_ERR_INVALID_ARG;
     Context* c = nullptr;
     if ((st = get_context(&c)) != NUNA_OK) return st;
-    return launch_reduce_scatter(c, make_ptrs(src, dst, nranks), nranks, dtype, shard_count, effective_flags(flags, stream), (cudaStream_t)stream);
+    return launch_reduce_scatter(c, make_ptrs(src, dst, nranks), nranks, dtype, shard_count, effective_flags(flags, stream),
+                                 (flags & NUNA_LAUNCH_PDL) != 0u, (cudaStream_t)stream);
 }
 
 int nuna_allgather(const void* const* src, void* const* dst, int nranks, size_t shard_count, int dtype,

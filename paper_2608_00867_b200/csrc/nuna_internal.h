@@ -89,7 +89,7 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
                          unsigned tv, unsigned min_tv, uint4* scratch, unsigned* tile_flags, BarrierWords* bw,
                          unsigned long long timeout_ns, bool pdl, unsigned debug_bits, cudaStream_t stream);
 bool chain_persistent_pays_off(int dtype, size_t count);
-int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, size_t shard, unsigned flags,
+int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, size_t shard, unsigned flags, bool asked,
                           cudaStream_t stream);
 int launch_allgather(Context* c, const RankPtrs& p, int nranks, size_t shard_bytes, unsigned flags, cudaStream_t stream);
 int launch_chain_persistent(Context* c, const ChainSets& sets, int nsets, int nnodes, int nranks, int dtype, size_t count,

@@ -1,0 +1,44 @@
+"""Which kernel a call runs, read from a trace, on both sides of the lines that a rule draws between two of them."""
+import warnings
+
+import pytest
+import torch
+
+from paper_2608_00867_b200 import binding as nb
+
+pytestmark = pytest.mark.gpu
+
+MIB = 1 << 20
+
+
+def kernels(call):
+    """Names of the kernels that the call launches, without their template arguments."""
+    call()
+    torch.cuda.synchronize()
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as trace:
+            call()
+            torch.cuda.synchronize()
+    names = [e.key for e in trace.key_averages() if "nuna::" in e.key]
+    if not names:
+        pytest.skip("nothing can be traced here")
+    return {name.split("nuna::")[1].split("<")[0].split("(")[0] for name in names}
+
+
+def reduce_scatter(n, nbytes, flags):
+    count = nbytes // 2 // n // 8 * 8
+    src = [torch.ones(n * count, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    dst = [torch.zeros(count, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    return kernels(lambda: nb.nuna_reduce_scatter(src, dst, count, flags=flags))
+
+
+@pytest.mark.parametrize("n,line_mib", [(2, 32), (8, 32), (16, 48)])
+def test_reduce_scatter_runs_ahead_unasked_only_where_no_predecessor_makes_it_slower(n, line_mib):
+    """`line_mib`: MiB of sources from which it does.  With NUNA_LAUNCH_PDL it also does below."""
+    ahead, ordinary = {"k_reduce_scatter_ahead"}, {"k_reduce_scatter"}
+    line = line_mib * MIB // n
+    assert reduce_scatter(n, line, 0) == ahead
+    assert reduce_scatter(n, line - 16 * n, 0) == ordinary
+    assert reduce_scatter(n, line - 16 * n, nb.NUNA_LAUNCH_PDL) == ahead
+    assert reduce_scatter(n, line, nb.NUNA_HINT_RESIDENT) == ordinary

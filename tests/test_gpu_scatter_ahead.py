@@ -25,7 +25,7 @@ def test_tiles_and_lines(n):
         for s in src[1:]:
             acc = acc + s[:n * shard].float()
         want = acc.bfloat16()
-        for flags in (0, nb.NUNA_HINT_RESIDENT):
+        for flags in (0, nb.NUNA_LAUNCH_PDL, nb.NUNA_HINT_RESIDENT):
             dst = [torch.full((shard + 64,), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
             nb.nuna_reduce_scatter(src, dst, shard, flags=flags)
             for r, d in enumerate(dst):
