@@ -1011,13 +1011,15 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
     // 16.41 | 16.74, 14.38 | 14.70, 8 MiB 28.24 | 28.57, 20.32 | 20.14; 4 x 4 MiB 10.54 | 10.74, 11.50 | 11.97, 8 MiB 17.06 | 17.22, 14.94 | 15.06;
     // 16 x 2 MiB 16.24 | 16.93, 13.86 | 14.56, 3 MiB 22.13 | 22.39, 16.50 | 16.61), it costs up to 2 % from 32 MiB of sources, 48 beyond 8
     // ranks, and up to 15 % below.
-    // Beyond 4 ranks blocks of 192 threads, 128 from 9 ranks, once full-width ones do
-    // not fit beside each other: they leave, and make room for the successor's, more evenly (8 x 4 MiB 5.49 | 5.31, 16 x 4 MiB 10.5 | 9.35).
+    // Beyond 4 ranks blocks of 192 threads, 128 from 9 ranks, once full-width ones do not fit beside each other: they leave, and make
+    // room for the successor's, more evenly (8 x 4 MiB 5.49 | 5.31, 16 x 2 MiB 5.67 | 5.04, 4 MiB 9.62 | 9.31); from 9 ranks full-width
+    // ones are ahead again beyond 64 MiB of sources (12 x 8 MiB 13.87 | 14.68, 16 x 8 MiB 18.65 | 19.02, 16 MiB 37.99 | 39.56).
     const size_t full = ceil_div(shard_vec, (size_t)kThreads) * (size_t)nranks, sms = (size_t)c->num_sms;
     const bool ahead = asked ? full >= (nranks <= 4 ? 64 : 32) : total >= (nranks <= 8 ? (size_t)32 << 20 : (size_t)48 << 20);
     if (ahead && mode == kLaunchPdl && !(flags & NUNA_HINT_RESIDENT) && o.prefetch != 1 && o.blocks <= 0 && unroll == 1 &&
         total <= (nranks <= 8 ? (size_t)128 << 20 : (size_t)256 << 20)) {
-        const unsigned threads = nranks <= 4 || full <= sms * 4 ? (unsigned)kThreads : nranks <= 8 ? 192u : 128u;
+        const bool wide = nranks <= 4 || full <= sms * 4 || (nranks > 8 && total > ((size_t)64 << 20));
+        const unsigned threads = wide ? (unsigned)kThreads : nranks <= 8 ? 192u : 128u;
         const unsigned tiles = (unsigned)ceil_div(shard_vec, (size_t)threads);
         return dispatch(nranks, 1, dtype, [&](auto n_, auto, auto d_) -> int {
             constexpr int N = decltype(n_)::value, DT = decltype(d_)::value;

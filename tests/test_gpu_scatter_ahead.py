@@ -16,6 +16,8 @@ def test_tiles_and_lines(n):
     first = ((64 if n <= 4 else 32) // n) * 256                     # vectors of a shard: below it the ordinary kernel runs
     wave = SMS * 4 * 256 // n // 256 * 256                          # the longest shard of one wave of full tiles
     vectors = [1, 127, 128, 129, 191, 192, 193, 255, 256, 257, first - 1, first, first + 1, wave, wave + 1, wave + 129]
+    if n > 8:
+        vectors += [(64 << 20) // 16 // n // n, (64 << 20) // 16 // n // n + 129]     # 64 MiB of sources: the tile is wide again beyond
     top = 8 * n * max(vectors)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(n)
