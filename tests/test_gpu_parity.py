@@ -156,7 +156,7 @@ def test_register_oneshot_tile_sizes_and_prefetch(vecs, n):
     assert nb.nuna_device_status() == nb.NUNA_OK
 
 
-@pytest.mark.parametrize("algo", ["oneshot_regs", "twoshot_put", "twoshot_flags"])
+@pytest.mark.parametrize("algo", ["oneshot_regs", "twoshot_put", "twoshot_tagged", "twoshot_flags"])
 def test_prefetch_ahead_of_the_wait_sees_the_predecessors_writes(algo):
     """A chain x -> allreduce -> allreduce -> ... in which every call's sources are the previous call's destinations,
     launched back to back with dependent launches: each kernel's prefetch is issued while its predecessor is still
@@ -166,7 +166,8 @@ def test_prefetch_ahead_of_the_wait_sees_the_predecessors_writes(algo):
     a, b = Dst(n, count), Dst(n, count)
     call, flags = {"oneshot_regs": (nb.nuna_allreduce_oneshot, nb.NUNA_PLACE_AWARE | nb.NUNA_PLACE_REGS),
                    "twoshot_put": (nb.nuna_allreduce_twoshot, nb.NUNA_TWOSHOT_PUT),
-                   "twoshot_flags": (nb.nuna_allreduce_twoshot, 0)}[algo]
+                   "twoshot_tagged": (nb.nuna_allreduce_twoshot, 0),
+                   "twoshot_flags": (nb.nuna_allreduce_twoshot, nb.NUNA_TWOSHOT_SYS_SCOPE)}[algo]   # no tagged form with it
     flags |= nb.NUNA_LAUNCH_PDL
     for _ in range(20):
         cur = upload(src)

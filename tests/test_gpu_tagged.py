@@ -68,64 +68,120 @@ def test_both_sides_of_every_line_and_every_neighbour(n):
     assert nb.nuna_device_status() == nb.NUNA_OK
 
 
-@pytest.mark.parametrize("n,mib", [(1, 9), (2, 6), (2, 17), (3, 7), (3, 60), (4, 41), (5, 9), (7, 19), (8, 9), (8, 17)])
-def test_shard_in_the_owners_destinations(n, mib):
+TORCH = {"bf16": torch.bfloat16, "f16": torch.float16, "f32": torch.float32}
+
+
+def same(got, want):
+    """Equal, NaN where there is to be one."""
+    return bool(((got == want) | (torch.isnan(got) & torch.isnan(want))).all())
+
+
+def fold(parts):
+    """The sum in rank order in binary32, rounded once."""
+    acc = parts[0].float()
+    for s in parts[1:]:
+        acc = acc + s.float()
+    return acc.to(parts[0].dtype)
+
+
+@pytest.mark.parametrize("dtype", TORCH)
+@pytest.mark.parametrize("n,mib", [(1, 9), (2, 6), (2, 17), (3, 7), (3, 60), (4, 41), (5, 9), (6, 9), (7, 19), (8, 9), (8, 17)])
+def test_shard_in_the_owners_destinations(n, mib, dtype):
     """Beyond the tagged form, on both sides of the lines where the shard moves into the destinations and its tile changes:
-    counts that end in a whole tile, in the middle of one and in the middle of a vector; eager and captured plainly."""
-    top = (mib << 20) // 2
+    counts that end in a whole tile, in the middle of one and in the middle of a vector; eager, captured plainly, with
+    dependent launches and with the resident hint; infinities and NaN among the values."""
+    size = nb.ELEM_SIZE[nb.DTYPE_BY_NAME[dtype]]
+    top, vec = (mib << 20) // size, 16 // size
     gen = torch.Generator(device="cuda")
     gen.manual_seed(mib)
-    src = [torch.randn(top, generator=gen, device="cuda").bfloat16() for _ in range(n)]
-    acc = src[0].float()
-    for s in src[1:]:
-        acc = acc + s.float()
-    want = acc.bfloat16()
-    nb.nuna_init(2 * top)
-    dst = [torch.zeros(top, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
-    for count in (top, top - 8 * 4096, top - 8 * 1001, top - 8 * 333 - 3):
-        g = torch.cuda.CUDAGraph()
-        torch.cuda.synchronize()
-        with torch.cuda.graph(g):
-            nb.nuna_allreduce_twoshot(src, dst, count)
-        for call in (lambda: nb.nuna_allreduce_twoshot(src, dst, count), g.replay):
-            for d in dst:
-                d.fill_(7.0)
-            call()
-            call()
-            for d in dst:
-                assert torch.equal(d[:count], want[:count]) and bool((d[count:] == 7.0).all()), count
+    src = [torch.randn(top, generator=gen, device="cuda").to(TORCH[dtype]) for _ in range(n)]
+    src[0][7], src[n - 1][11], src[0][top // 2], src[n - 1][top // 2] = float("inf"), float("nan"), float("inf"), float("-inf")
+    want = fold(src)
+    nb.nuna_init(size * top)
+    dst = [torch.zeros(top, dtype=TORCH[dtype], device="cuda") for _ in range(n)]
+    for count in (top, top - vec * 4096, top - vec * 1001, top - vec * 333 - 3):
+        for flags in (0, nb.NUNA_LAUNCH_PDL, nb.NUNA_LAUNCH_PDL | nb.NUNA_HINT_RESIDENT):
+            call = lambda: nb.nuna_allreduce_twoshot(src, dst, count, dtype=nb.DTYPE_BY_NAME[dtype], flags=flags)
+            g = torch.cuda.CUDAGraph()
+            torch.cuda.synchronize()
+            with torch.cuda.graph(g):
+                call()
+            for run in (call, g.replay):
+                for d in dst:
+                    d.fill_(7.0)
+                run()
+                run()
+                for d in dst:
+                    assert same(d[:count], want[:count]) and bool((d[count:] == 7.0).all()), (count, flags)
+    assert nb.nuna_device_status() == nb.NUNA_OK
+
+
+@pytest.mark.parametrize("form", ["tagged", "flags", "in place"])
+@pytest.mark.parametrize("n,dtype", [(2, "bf16"), (2, "f16"), (4, "f32"), (6, "f32"), (8, "bf16"), (8, "f16"), (8, "f32")])
+def test_every_call_reads_what_the_one_before_wrote(n, dtype, form):
+    """Four calls in a row, eager and captured with dependent launches, whose prefetch goes out while the call before still
+    writes what they read.  Whole numbers that differ from place to place and fit the type, infinities and NaN."""
+    code = nb.DTYPE_BY_NAME[dtype]
+    size = nb.ELEM_SIZE[code]
+    count = {"tagged": 300 << 10, "flags": 300 << 10, "in place": (9 << 20) + (64 << 10)}[form] // size - 3
+    flags = nb.NUNA_LAUNCH_PDL | (nb.NUNA_TWOSHOT_SYS_SCOPE if form == "flags" else 0)
+    nb.nuna_init(size * count + 16)
+    new = lambda: [torch.zeros(count, dtype=TORCH[dtype], device="cuda") for _ in range(n)]
+    x, a, b = new(), new(), new()
+
+    def run():
+        for s, d in ((x, a), (a, b), (b, a), (a, b)):
+            nb.nuna_allreduce_twoshot(s, d, count, dtype=code, flags=flags)
+
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        run()
+    place = torch.arange(count, device="cuda")
+    for it in range(8):
+        for r in range(n):
+            x[r].copy_((place * (3 + it) % 31) // 4 + r % 2)
+        x[0][5::4099], x[n - 1][7::4099], x[0][9::4099], x[n - 1][9::4099] = float("inf"), float("nan"), float("inf"), float("-inf")
+        want = x
+        for _ in range(4):
+            want = [fold(want)] * n
+        g.replay() if it % 2 else run()
+        for t in b:
+            assert same(t, want[0]), it
     assert nb.nuna_device_status() == nb.NUNA_OK
 
 
 @pytest.mark.parametrize("pdl", [0, nb.NUNA_LAUNCH_PDL])
 def test_back_to_back_replays_of_mixed_sizes(pdl):
     """A captured run in which every call reads what the one before wrote, sizes alternating, replayed and mixed with eager
-    calls: a ticket drawn ahead of the wait must find the word set up by the launch before."""
+    calls: a ticket drawn ahead of the wait must find the word set up by the launch before.  Every element of both buffers
+    after every run; whole numbers below 2^24 that differ from place to place."""
     n, sizes = 4, (64, 70001, 8, 300000, 2049, 262144)
     top = max(sizes)
     nb.nuna_init(4 * top + 16)
-    bufs = [[torch.zeros(top, dtype=torch.float32, device="cuda") for _ in range(n)] for _ in range(2)]
+    bufs = torch.zeros(2, n, top, device="cuda")
+    ranks = [list(b) for b in bufs]
 
     def run():
         for k, c in enumerate(sizes):
-            nb.nuna_allreduce_twoshot(bufs[k % 2], bufs[1 - k % 2], c, dtype=nb.NUNA_F32, flags=pdl)
+            nb.nuna_allreduce_twoshot(ranks[k % 2], ranks[1 - k % 2], c, dtype=nb.NUNA_F32, flags=pdl)
 
     g = torch.cuda.CUDAGraph()
     torch.cuda.synchronize()
     with torch.cuda.graph(g):
         run()
+    place = torch.arange(top, device="cuda")
     for it in range(20):
-        for r in range(n):
-            bufs[0][r].fill_(r + 1)
-            bufs[1][r].zero_()
+        bufs[0] = torch.stack([place * (2 + it) % 13 + r for r in range(n)])
+        bufs[1].zero_()
+        start = bufs.clone()
         for _ in range(1 + it % 3):
+            bufs.copy_(start)
             g.replay() if it % 2 else run()
-            last = [b.clone() for b in bufs[0]]
-            for r in range(n):
-                bufs[0][r].fill_(r + 1)
-        smallest = min(sizes)
-        want = 10.0 * 4.0 ** (len(sizes) - 1)                       # 1 + 2 + 3 + 4, then four times itself in every further call
-        assert all(bool((b[:smallest] == want).all()) for b in last), it
+        want = start
+        for k, c in enumerate(sizes):
+            want[1 - k % 2, :, :c] = want[k % 2, :, :c].sum(0)
+        assert torch.equal(bufs, want), it
     assert nb.nuna_device_status() == nb.NUNA_OK
 
 
