@@ -890,10 +890,14 @@ static TaggedShape tagged_shape(const Context* c, int nranks, size_t nvec)
 // Whether a two-shot call runs the tagged form.  us per node, flags | tagged: 2 ranks x 64 KiB 3.19 | 1.96, 4 MiB 9.9 | 6.1,
 // 8 MiB 9.4 | 9.8; 4 x 512 KiB 6.4 | 2.6, 4 MiB 8.8 | 7.9; 8 x 8 KiB 3.3 | 2.0, 512 KiB 5.0 | 2.9, 4 MiB 14.2 | 12.2, 8 MiB 24.7 | 22.7,
 // 16 MiB 44.6 | 45.9; 16 x 64 KiB 5.6 | 2.6, 1 MiB 10.1 | 7.5, 4 MiB 25.6 | 22.7.  The fewer the ranks, the more the shard's doubled
-// bytes are beside theirs.  What asks about the flags (their scope, their tile, the shard's lines) gets the form that has them.
+// bytes are beside theirs.  On sources that are in L2 there is less to hide them behind (flags, scratch or in place | tagged, with the
+// hint: 3 x 5 MiB 7.51 | 7.51, 6 MiB 8.50 | 8.79, 4 x 5 MiB 9.09 | 8.88, 6 MiB 10.22 | 10.56; 8 x 8 MiB 25.5 | 23.5).  Captured plainly the order is
+// that of cold sources (3 x 6 MiB 11.6 | 10.5, 4 x 6 MiB 13.3 | 12.0, 8 x 8 MiB 26.6 | 24.6, 16 x 8 MiB 46.5 | 45.1; 3 x 6 MiB from L2 9.2 | 9.7).
+// What asks about the flags (their scope, their tile, the shard's lines) gets the form that has them.
 static bool takes_tags(const Options& o, int nranks, size_t bytes, unsigned flags)
 {
-    return bytes <= (nranks <= 2 ? kTaggedMaxShard / 8 * 5 : nranks <= 4 ? kTaggedMaxShard / 4 * 3 : kTaggedMaxShard) && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard &&
+    const bool five = nranks <= 2 || (nranks <= 4 && (flags & NUNA_HINT_RESIDENT));
+    return bytes <= (five ? kTaggedMaxShard / 8 * 5 : nranks <= 4 ? kTaggedMaxShard / 4 * 3 : kTaggedMaxShard) && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard &&
            o.twoshot_vecs <= 0 && o.blocks <= 0;
 }
 

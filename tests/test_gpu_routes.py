@@ -12,7 +12,7 @@ MIB = 1 << 20
 
 
 def kernels(call):
-    """Names of the kernels that the call launches, without their template arguments."""
+    """Names of the kernels that the call launches, without their template arguments but for one that is a truth value."""
     call()
     torch.cuda.synchronize()
     with warnings.catch_warnings():
@@ -23,7 +23,7 @@ def kernels(call):
     names = [e.key for e in trace.key_averages() if "nuna::" in e.key]
     if not names:
         pytest.skip("nothing can be traced here")
-    return {name.split("nuna::")[1].split("<")[0].split("(")[0] for name in names}
+    return {name.split("nuna::")[1].split("<")[0].split("(")[0] + (" true" if "true>" in name else "") for name in names}
 
 
 def reduce_scatter(n, nbytes, flags):
@@ -42,3 +42,19 @@ def test_reduce_scatter_runs_ahead_unasked_only_where_no_predecessor_makes_it_sl
     assert reduce_scatter(n, line - 16 * n, 0) == ordinary
     assert reduce_scatter(n, line - 16 * n, nb.NUNA_LAUNCH_PDL) == ahead
     assert reduce_scatter(n, line, nb.NUNA_HINT_RESIDENT) == ordinary
+
+
+def twoshot(n, nbytes, flags):
+    count = nbytes // 2
+    src = [torch.ones(count, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    dst = [torch.zeros(count, dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    nb.nuna_init(nbytes)
+    return kernels(lambda: nb.nuna_allreduce_twoshot(src, dst, count, flags=flags))
+
+
+@pytest.mark.parametrize("n,cold,resident", [(2, 5, 5), (3, 6, 5), (4, 6, 5), (8, 8, 8)])
+def test_the_largest_message_of_the_tagged_twoshot(n, cold, resident):
+    """In MiB per rank, without and with the resident hint."""
+    for flags, most in ((0, cold * MIB), (nb.NUNA_HINT_RESIDENT, resident * MIB)):
+        assert twoshot(n, most, flags) == {"k_twoshot_tagged"}
+        assert "k_twoshot_tagged" not in twoshot(n, most + 16, flags)
