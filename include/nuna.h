@@ -307,17 +307,21 @@ int nuna_allreduce_oneshot(const void* const* src, void* const* dst, int nranks,
  * after acquire-polling that tile's flag (bounded wait: on expiry NUNA_ERR_TIMEOUT is latched and the block
  * returns).  A wait is only ever for an item with a smaller ticket, held by a block that already runs, so
  * the kernel needs no co-residency guarantee and no cooperative launch.  Consumed shard lines are dropped
- * from L2 (discard) instead of being written back.  Up to 4 ranks, and up to 128 MiB of sources up to 8, there is no
- * scratch: a tile is reduced into its place in its owner's destination (owners' chunks are whole tiles) and gathered from
- * there into the others (plain launches: at 3 and 4 ranks only).  Small and mid-sized messages (up to 8 MiB per rank, 6 MiB at 3 and 4 ranks, 5 MiB below) take a
- * form without a flag per tile: every 32-bit word of the reduced tile is stored together with the launch's
- * epoch in one 64-bit access, and the gathering block polls the words themselves, under the same bound.  Neither
- * form is used with NUNA_TWOSHOT_SYS_SCOPE, NUNA_OPT_TWOSHOT_VECS or NUNA_OPT_BLOCKS.  Same bits as the one-shot.  Any `count`; chunk =
- * ceil(count/N) rounded up to a whole 16-byte vector, trailing chunks may be short or empty.  Uses the
- * context's shard scratch (count*elemsize bytes plus one flag word per 256 bytes, and the slots where words stand
- * with their epochs: twice the next power of two, at most 16 MiB; grown on demand; what is outgrown stays
- * allocated until nuna_shutdown because captured graphs may still name it) unless
- * NUNA_TWOSHOT_PUT is set.  Calls that share the context must be stream-ordered with respect to each other. */
+ * from L2 (discard) instead of being written back.  Up to 4 ranks, and up to 128 MiB of sources up to 8, the
+ * reduced data does not pass through the scratch: a tile is reduced into its place in its owner's destination
+ * (owners' chunks are whole tiles) and gathered from there into the others (captured without NUNA_LAUNCH_PDL
+ * at 3 and 4 ranks only; with NUNA_HINT_RESIDENT up to 6 ranks, but at 2 not between 20 and 32 MiB of
+ * sources).  Small and mid-sized messages (up to 8 MiB per rank, 6 MiB at 3 and 4 ranks, 5 there with
+ * NUNA_HINT_RESIDENT and below 3 ranks) take a form without a flag per tile: every 32-bit word of the reduced
+ * tile is stored together with the launch's epoch in one 64-bit access, and the gathering block polls the
+ * words themselves, under the same bound.  Neither form is used with NUNA_TWOSHOT_SYS_SCOPE,
+ * NUNA_OPT_TWOSHOT_VECS, NUNA_OPT_BLOCKS or the environment's NUNA_KEEP_SHARD.  Same bits as the one-shot.
+ * Any `count`; chunk = ceil(count/N) rounded up to a whole 16-byte vector, trailing chunks may be short or
+ * empty.  Whatever the form, uses the context's shard scratch (count*elemsize bytes plus one flag word per 256
+ * bytes, and the slots where words stand with their epochs: twice the next power of two, at most 16 MiB; grown
+ * on demand; what is outgrown stays allocated until nuna_shutdown because captured graphs may still name it)
+ * unless NUNA_TWOSHOT_PUT is set.  Calls that share the context must be stream-ordered with respect to each
+ * other.                                                                                                */
 int nuna_allreduce_twoshot(const void* const* src, void* const* dst, int nranks,
                            size_t count, int dtype, unsigned flags, void* stream);
 

@@ -942,10 +942,16 @@ int launch_twoshot_put(Context* c, const RankPtrs& p, int nranks, int dtype, siz
 // 9.4 | 8.4, 64 MiB 53.2 | 42.7; 3 x 23 MiB 27.8 | 25.3; 4 x 16 MiB 26.5 | 23.5, 64 MiB 92 | 84.5; 6 x 12 MB 26.5 | 25.1; 8 x 9 MiB 27.7 |
 // 26.1, 16 MiB 44.0 | 42.7, but 22 MiB 61.5 | 63.7, 6 x 24 MB 49.9 | 50.9; 12 x 10 MB 43.0 | 44.3; 16 x 12 MB 63.4 | 63.8.  Launched
 // plainly, without a prefetch: 2 x 16 MiB 17.5 | 19.5, 3 x 64 MiB 71.8 | 67.4, 4 x 16 MiB 28.0 | 26.9, 8 x 16 MiB 46.8 | 48.2.
+// With the resident hint there is no prefetch either: 2 x 9 MiB 9.5 | 9.2, 10 MiB 10.5 | 10.5, 12 MiB 11.9 | 14.4, 16 MiB 16.5 | 18.5, but 18 MiB 18.2 | 16.8, 64 MiB 52.3 | 47.6; 3 x
+// 23 MiB 29.2 | 27.7; 5 x 9 MiB 20.7 | 19.7, 25 MiB 49.0 | 47.0; 6 x 9 MiB 23.7 | 22.4, 20 MiB 43.8 | 43.8; 7 x 12 MiB 32.7 | 33.7, 18 MiB 45.3 |
+// 47.8; 8 x 9 MiB 28.2 | 28.9, 16 MiB 45.5 | 47.6.
 static bool shard_in_place(const Options& o, int nranks, size_t bytes, unsigned flags)
 {
-    const bool pays = (flags & NUNA_LAUNCH_PDL) ? nranks <= 4 || (nranks <= 8 && bytes * (size_t)nranks <= ((size_t)128 << 20))
-                                                : nranks == 3 || nranks == 4;
+    const size_t total = bytes * (size_t)nranks;
+    const bool hint = (flags & NUNA_HINT_RESIDENT) != 0u;
+    const bool pays = !(flags & NUNA_LAUNCH_PDL) ? nranks == 3 || nranks == 4
+                    : nranks > 4                 ? nranks <= (hint ? 6 : 8) && total <= ((size_t)128 << 20)
+                                                 : !hint || nranks != 2 || total <= ((size_t)20 << 20) || total > ((size_t)32 << 20);
     return pays && !(flags & NUNA_TWOSHOT_SYS_SCOPE) && !o.keep_shard && o.twoshot_vecs <= 0 && o.blocks <= 0;
 }
 

@@ -58,3 +58,11 @@ def test_the_largest_message_of_the_tagged_twoshot(n, cold, resident):
     for flags, most in ((0, cold * MIB), (nb.NUNA_HINT_RESIDENT, resident * MIB)):
         assert twoshot(n, most, flags) == {"k_twoshot_tagged"}
         assert "k_twoshot_tagged" not in twoshot(n, most + 16, flags)
+
+
+@pytest.mark.parametrize("n,mib,cold,resident", [(1, 9, True, True), (2, 10, True, True), (2, 16, True, False), (2, 17, True, True), (4, 16, True, True), (6, 16, True, True),
+                                                 (7, 12, True, False), (8, 12, True, False), (8, 17, False, False)])
+def test_the_flag_twoshot_reduces_in_place_where_that_pays(n, mib, cold, resident):
+    """MiB per rank; the kernel's last template argument says whether the shard is the owners' destinations."""
+    for flags, in_place in ((0, cold), (nb.NUNA_HINT_RESIDENT, resident)):
+        assert twoshot(n, mib * MIB, flags) == {"k_twoshot_flags" + (" true" if in_place else "")}

@@ -85,7 +85,7 @@ def fold(parts):
 
 
 @pytest.mark.parametrize("dtype", TORCH)
-@pytest.mark.parametrize("n,mib", [(1, 9), (2, 6), (2, 17), (3, 7), (3, 60), (4, 41), (5, 9), (6, 9), (7, 19), (8, 9), (8, 17)])
+@pytest.mark.parametrize("n,mib", [(1, 9), (2, 6), (2, 12), (2, 17), (3, 7), (3, 60), (4, 41), (5, 9), (6, 9), (7, 19), (8, 9), (8, 17)])
 def test_shard_in_the_owners_destinations(n, mib, dtype):
     """Beyond the tagged form, on both sides of the lines where the shard moves into the destinations and its tile changes:
     counts that end in a whole tile, in the middle of one and in the middle of a vector; eager, captured plainly, with
