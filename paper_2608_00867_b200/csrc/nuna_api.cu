@@ -823,6 +823,7 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
     const bool many_resident = !in_place ? all_src >= ((size_t)64 << 20) : all_src > (nranks <= 2 ? (size_t)32 << 20 : (size_t)160 << 20);
     bool mid_sized = false;
     if (tv == 0) {
+        // (Below takes_tags' limit these are the tiles of calls that ask for the flags' scope or cap the blocks, and of the hooks.)
         // Tile bytes across all N sources, from a sweep at 8 ranks (16 ... 256 vectors per tile at every size):
         // small tiles while the message is small (more blocks, less latency per tile), 32 KiB once there are
         // plenty.  At 8 MiB of sources 16 KiB tiles make 1024 blocks for 592 resident ones and the second
@@ -866,9 +867,10 @@ int launch_twoshot_flags(int num_sms, int blocks_override, const RankPtrs& p, in
 // How the tagged two-shot is launched, always in full-width blocks: narrow ones start on an SM while the predecessor still
 // drains, unevenly (8 x 64 KiB 1.8 us in 256 threads, 2.5 in 64).  Measured at 2, 4, 8 and 16 ranks, 16 KiB ... 16 MiB per rank, cold, tiles
 // of 16 ... 256 vectors, leads of 1 ... 1184 tiles, dependent graph nodes (us):
-// * As long as all blocks are resident together, each gathers the tile before its own (lead 1: 8 x 512 KiB 2.9, 3.6 with a lead of
-//   three tiles per SM): four tiles per SM of 56 ... 128 vectors, from 96 up to 8 ranks (8 x 512 KiB 2.95 with 56, 2.89; 16 x
-//   256 KiB 2.88 with 56, 3.00), fewer and larger ones up to 4 ranks (2 x 1 MiB 2.75 with 96 vectors, 2.53 with 192).
+// * Up to four tiles per SM each block gathers the tile before its own (lead 1: 8 x 512 KiB 2.9, 3.6 with a lead of three tiles per
+//   SM): tiles of 56 ... 128 vectors, from 96 up to 8 ranks (8 x 512 KiB 2.95 with 56, 2.89; 16 x 256 KiB 2.88 with 56, 3.00), fewer
+//   and larger ones up to 4 ranks (2 x 1 MiB 2.75 with 96 vectors, 2.53 with 192).  Up to 11 ranks registers hold four blocks per SM
+//   and all of them are resident together; from 12 they hold three, and the last quarter starts as the first leave (16 x 1 MiB 7.4).
 // * Beyond, a lead of three tiles per SM, so that what a block gathers was reduced a wave earlier (8 x 4 MiB 11.5; five 11.6,
 //   one 11.7, eight 11.9), and tiles of 128 vectors (192 12.1), 192 up to 4 ranks (2 x 8 MiB 8.84; 128 9.2, 256 8.97).
 struct TaggedShape {

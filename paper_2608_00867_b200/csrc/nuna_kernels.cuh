@@ -1466,14 +1466,13 @@ __device__ __forceinline__ void half_sync(int id) { asm volatile("bar.sync %0, 1
 // wait); bit 2: keep consumed shard lines in L2 (for measuring what the discard saves); bit 3: flags are
 // released and acquired at system scope (NUNA_TWOSHOT_SYS_SCOPE).
 // kInPlace: the shard of a tile is its place in its owner's destination (the owners' chunks are whole tiles), scratch is not
-// used and the gathering block stores to the N - 1 others.  A template argument: read at run time it costs the scratch form its
-// registers (8 x 36 MiB 98.3 -> 102 us).
-// That saves the shard's writes to L2, which count the more the fewer the ranks (2 x 64 MiB 53.2 -> 42.9 us, 3 x 23 MiB 28.4 -> 24.6,
-// 8 x 16 MiB 44.4 -> 42.7; but 8 x 64 MiB 167 -> 170).
+// used and the gathering block stores to the N - 1 others.  That saves the shard's writes to L2, which count the more the fewer
+// the ranks (2 x 64 MiB 53.2 -> 42.9 us, 3 x 23 MiB 28.4 -> 24.6, 8 x 16 MiB 44.4 -> 42.7; but 8 x 64 MiB 167 -> 170).  A template
+// argument: read at run time it costs the scratch form its registers (8 x 36 MiB 98.3 -> 102 us).
 // kMinBlocks: resident blocks per SM the register allocation is held to.  4 (64 registers) gives the shortest
 // path per block, best while the message is small enough for latency to dominate (8 KiB per rank: 3.4 us
-// against 3.7 us).  6 holds it to 40 registers: more tiles in flight per SM, which is what counts once the
-// message is bandwidth-bound (measured at 8 ranks: 16 MiB per rank 48.7 -> 45.6 us).
+// against 3.7 us).  6 holds it to 40 registers (4 to 36 bytes spilled from 3 ranks on, most at 4 and 5 in place): more tiles in
+// flight per SM, which is what counts once the message is bandwidth-bound (measured at 8 ranks: 16 MiB per rank 48.7 -> 45.6 us).
 template <int N, int DT, int kMinBlocks, bool kInPlace>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
 k_twoshot_flags(const RankPtrs p, uint4* scratch, unsigned int* flags, const size_t count, const unsigned tv,
@@ -1642,7 +1641,7 @@ __device__ __forceinline__ bool poll_tagged(Arrived&& arrived, unsigned long lon
 
 // tv: vectors per tile, at most the block's width.  debug bits as in k_twoshot_flags: 0 and 4.
 // Up to 4 ranks the first look at the words to gather goes out together with the loads of the sources, which are few
-// (4 x 512 KiB 2.63 -> 2.35 us, 2 x 1 MiB 2.9 -> 2.55); beyond it only delays them (16 x 1 MiB 6.74 -> 7.54).
+// (4 x 512 KiB 2.63 -> 2.35 us, 2 x 1 MiB 2.9 -> 2.55); beyond it only delays them (16 x 1 MiB by 12 %).
 constexpr int kTaggedEarly = 4;
 
 template <int N, int DT>
