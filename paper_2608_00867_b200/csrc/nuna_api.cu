@@ -1021,7 +1021,7 @@ int launch_reduce_scatter(Context* c, const RankPtrs& p, int nranks, int dtype, 
     // 1.71 | 1.93, 2 MiB 2.38 | 2.54, but 4 MiB 5.44 | 4.50, 8 MiB 10.7 | 9.4), or a kernel that does not release early comes before it
     // (with that kernel's time, one that writes the sources, and one that writes elsewhere: 8 x 1 MiB 6.98 | 7.29, 9.99 | 10.65, 4 MiB
     // 16.41 | 16.74, 14.38 | 14.70, 8 MiB 28.24 | 28.57, 20.32 | 20.14; 4 x 4 MiB 10.54 | 10.74, 11.50 | 11.97, 8 MiB 17.06 | 17.22, 14.94 | 15.06;
-    // 16 x 2 MiB 16.24 | 16.93, 13.86 | 14.56, 3 MiB 22.13 | 22.39, 16.50 | 16.61), it costs up to 2 % from 32 MiB of sources, 48 beyond 8
+    // 16 x 2 MiB 16.24 | 16.93, 13.86 | 14.56, 3 MiB 22.13 | 22.39, 16.50 | 16.61), it costs at most 2.3 % from 32 MiB of sources, 48 beyond 8
     // ranks, and up to 15 % below.
     // Beyond 4 ranks blocks of 192 threads, 128 from 9 ranks, once full-width ones do not fit beside each other: they leave, and make
     // room for the successor's, more evenly (8 x 4 MiB 5.49 | 5.31, 16 x 2 MiB 5.67 | 5.04, 4 MiB 9.62 | 9.31); from 9 ranks full-width
