@@ -22,7 +22,7 @@ std::atomic<unsigned long long> g_launches{0};
 static std::mutex g_ctx_mutex;
 static std::atomic<Context*> g_ctx[kMaxDevices];              // written under g_ctx_mutex
 
-static int static_status_read_and_clear(unsigned* out);     // the allocation-free entry point's status word (end of file)
+static int static_status_read_and_clear(const Context* c, unsigned* out);     // the allocation-free entry point's status word (end of file)
 constexpr unsigned kMinFlagTileVec = 16;                    // smallest two-shot tile (vectors): 256 bytes of shard per flag
 constexpr size_t kTaggedMaxShard = (size_t)8 << 20;         // largest message, in bytes per rank, that the tagged two-shot takes
 constexpr unsigned kStaticTileVec = 128;                    // tile of the allocation-free entry point: 2 KiB of shard per flag
@@ -33,35 +33,31 @@ static int env_int(const char* name, int fallback)
     return (s && *s) ? atoi(s) : fallback;
 }
 
+constexpr size_t align_up(size_t n, size_t to) { return (n + to - 1) / to * to; }
+
 // Sets device memory that a kernel on any stream may use next, to zero or to what `host` holds: cudaMemset, and cudaMemcpy from
 // pageable memory, return before they are done, and only the legacy stream and those that wait for it come after them.  On a
-// stream of its own it waits for nobody else's work.
-static bool set_now(void* p, const void* host, size_t bytes)
+// stream of the context's own it waits for nobody else's work.
+static bool set_now(const Context* c, void* p, const void* host, size_t bytes)
 {
-    cudaStream_t s = nullptr;
-    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
-    const cudaError_t e = host ? cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, s) : cudaMemsetAsync(p, 0, bytes, s);
-    const bool ok = cudaStreamSynchronize(s) == cudaSuccess && e == cudaSuccess;
-    cudaStreamDestroy(s);
-    return ok;
+    const cudaError_t e = host ? cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, c->setup) : cudaMemsetAsync(p, 0, bytes, c->setup);
+    return cudaStreamSynchronize(c->setup) == cudaSuccess && e == cudaSuccess;
 }
-
-static bool zero_now(void* p, size_t bytes) { return set_now(p, nullptr, bytes); }
 
 int init_barrier_words(Context* c)
 {
-    return zero_now(c->bw, sizeof(BarrierWords)) ? NUNA_OK : NUNA_ERR_CUDA;
+    return set_now(c, c->bw, nullptr, sizeof(BarrierWords)) ? NUNA_OK : NUNA_ERR_CUDA;
 }
 
 // After a latched timeout the barrier's arrival counter is in an undefined state: zero it and clear the
 // status, but keep both epochs moving forward -- the ready flags of earlier launches must never match a
 // later launch's epoch.  The device is idle (the caller synchronised).
-static int rewind_barrier_words(BarrierWords* dev, const BarrierWords& seen)
+static int rewind_barrier_words(const Context* c, BarrierWords* dev, const BarrierWords& seen)
 {
     BarrierWords h = {};
     h.epoch = seen.epoch + 1u;
     h.ticket = ((seen.ticket >> 32) + 1ull) << 32;
-    return set_now(dev, &h, sizeof h) ? NUNA_OK : NUNA_ERR_CUDA;
+    return set_now(c, dev, &h, sizeof h) ? NUNA_OK : NUNA_ERR_CUDA;
 }
 
 // Returns the current device's context, creating it on first use (allocates: not capturable).
@@ -78,8 +74,13 @@ int get_context(Context** out)
         if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { delete c; return NUNA_ERR_CUDA; }
         c->num_sms = prop.multiProcessorCount;
         c->l2_bytes = (size_t)prop.l2CacheSize;
-        if (cudaMalloc(&c->bw, sizeof(BarrierWords)) != cudaSuccess) { delete c; return NUNA_ERR_CUDA; }
-        if (init_barrier_words(c) != NUNA_OK) { cudaFree(c->bw); delete c; return NUNA_ERR_CUDA; }
+        if (cudaStreamCreateWithFlags(&c->setup, cudaStreamNonBlocking) != cudaSuccess) { delete c; return NUNA_ERR_CUDA; }
+        if (cudaMalloc(&c->bw, sizeof(BarrierWords)) != cudaSuccess || init_barrier_words(c) != NUNA_OK) {
+            if (c->bw) cudaFree(c->bw);
+            cudaStreamDestroy(c->setup);
+            delete c;
+            return NUNA_ERR_CUDA;
+        }
         c->opt.timeout_ns = (unsigned long long)env_int("NUNA_TIMEOUT_MS", 1000) * 1000000ull;
         c->opt.blocks = env_int("NUNA_BLOCKS", 0);
         c->opt.unroll = env_int("NUNA_UNROLL", 0);
@@ -98,33 +99,36 @@ int get_context(Context** out)
     return NUNA_OK;
 }
 
-// Grows the two-shot scratch: shard intermediate with one ready flag per smallest tile of it, and the slots of the tagged form
-// for as large a shard as that form takes.  The caller holds c->mutex.  An outgrown allocation is never freed before nuna_shutdown: a CUDA graph captured earlier
-// (a chain, or a user's capture of a two-shot call) still carries its address as a kernel argument.  The slots, twice their
-// shard's bytes, are therefore an allocation of their own that doubles: what has been outgrown is never more than the last.
+// Grows the two-shot scratch: shard intermediate, one ready flag per smallest tile of it, and behind them, where larger ones are
+// needed, the slots of the tagged form.  The caller holds c->mutex.  An outgrown allocation is never freed before nuna_shutdown: a
+// CUDA graph captured earlier (a chain, or a user's capture of a two-shot call) still carries its address as a kernel argument.
+// The slots take twice their shard's bytes, so they double, whatever the shard grows by: what has been outgrown of them is never
+// more than what is in use, and most growths leave them where they are.
 int ensure_scratch(Context* c, size_t bytes)
 {
     if (bytes <= c->scratch_bytes && c->scratch) return NUNA_OK;
-    // flags and tags start at zero; epochs start at one, so a fresh one never reads as "ready"
-    const auto grow = [c](void** at, size_t data, size_t zeroed) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, data + zeroed) != cudaSuccess) return false;
-        if (!zero_now(static_cast<char*>(p) + data, zeroed)) { cudaFree(p); return false; }
-        if (*at) c->retired_scratch.push_back(*at);
-        *at = p;
-        return true;
-    };
     const size_t want = (std::max<size_t>(bytes, 4096) + 4095) & ~(size_t)4095;
+    const size_t nflags = want / (kMinFlagTileVec * 16) + 1;         // one ready flag per smallest tile
+    const size_t slots_at = align_up(want + nflags * sizeof(unsigned), 256);
     size_t slots_shard = 64 << 10;
     while (slots_shard < std::min(want, kTaggedMaxShard)) slots_shard *= 2;
-    if (slots_shard > c->slots_shard) {
-        if (!grow(&c->slots, 0, tagged_bytes(slots_shard))) return NUNA_ERR_CUDA;
+    const bool more_slots = slots_shard > c->slots_shard;
+    const size_t total = slots_at + (more_slots ? tagged_bytes(slots_shard) : 0);
+    void* p = nullptr;
+    if (cudaMalloc(&p, total) != cudaSuccess) return NUNA_ERR_CUDA;
+    // flags and tags start at zero; epochs start at one, so a fresh one never reads as "ready"
+    if (!set_now(c, static_cast<char*>(p) + want, nullptr, total - want)) {
+        cudaFree(p);
+        return NUNA_ERR_CUDA;
+    }
+    if (c->scratch) c->retired_scratch.push_back(c->scratch);
+    c->scratch = p;
+    c->flags = reinterpret_cast<unsigned*>(static_cast<char*>(p) + want);
+    c->scratch_bytes = want;
+    if (more_slots) {
+        c->slots = static_cast<char*>(p) + slots_at;
         c->slots_shard = slots_shard;
     }
-    const size_t nflags = want / (kMinFlagTileVec * 16) + 1;         // one ready flag per smallest tile
-    if (!grow(&c->scratch, want, nflags * sizeof(unsigned))) return NUNA_ERR_CUDA;
-    c->flags = reinterpret_cast<unsigned*>(static_cast<char*>(c->scratch) + want);
-    c->scratch_bytes = want;
     return NUNA_OK;
 }
 
@@ -308,8 +312,6 @@ static int launch(void (*kernel)(Args...), unsigned grid, cudaStream_t stream, u
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return NUNA_OK;
 }
-
-constexpr size_t align_up(size_t n, size_t to) { return (n + to - 1) / to * to; }
 
 template <typename... Args>
 constexpr size_t param_bytes()
@@ -520,7 +522,7 @@ static int get_sm_plan(Context* c, int nranks, size_t nvec, int coloc, int domai
         const size_t cur0 = off.size() + std::max<size_t>(tiles.size(), 1);
         pl.nonempty = 0;
         for (int s = 0; s < c->num_sms; ++s) pl.nonempty += !lists[s].empty();
-        if (!set_now(d, host.data(), words * sizeof(unsigned))) {
+        if (!set_now(c, d, host.data(), words * sizeof(unsigned))) {
             cudaFree(d);
             return NUNA_ERR_CUDA;
         }
@@ -1480,10 +1482,10 @@ int nuna_device_status(int* out)
     BarrierWords h;
     if (cudaMemcpy(&h, c->bw, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return NUNA_ERR_CUDA;
     unsigned worst = h.status;
-    if (h.status != 0 && (st = rewind_barrier_words(c->bw, h)) != NUNA_OK) return st;
+    if (h.status != 0 && (st = rewind_barrier_words(c, c->bw, h)) != NUNA_OK) return st;
     // the allocation-free entry point keeps its own words in the library's fixed arrays
     unsigned static_status = 0;
-    if ((st = static_status_read_and_clear(&static_status)) != NUNA_OK) return st;
+    if ((st = static_status_read_and_clear(c, &static_status)) != NUNA_OK) return st;
     *out = (int)std::max(worst, static_status);
     return NUNA_OK;
 }
@@ -1532,10 +1534,10 @@ int nuna_shutdown(void)
     cudaDeviceSynchronize();
     if (c->bw) cudaFree(c->bw);
     if (c->scratch) cudaFree(c->scratch);
-    if (c->slots) cudaFree(c->slots);
     for (void* d : c->retired_scratch) cudaFree(d);
     if (c->staging) cudaFree(c->staging);
     if (c->stream) cudaStreamDestroy(c->stream);
+    cudaStreamDestroy(c->setup);
     for (auto& kv : c->sm_plans) cudaFree(kv.second.base);
     for (unsigned* d : c->retired_plans) cudaFree(d);
     delete c;
@@ -1747,7 +1749,7 @@ static int static_setup(StaticSetup** out)
 // For nuna_device_status: the status latched by the allocation-free entry point on the current device
 // (0 if that entry point was never used here).  A latched timeout leaves cursor and departure counter in
 // an undefined state, so the control words are zeroed again; the device is idle (the caller synchronised).
-static int static_status_read_and_clear(unsigned* out)
+static int static_status_read_and_clear(const Context* c, unsigned* out)
 {
     *out = 0;
     int dev = -1;
@@ -1758,7 +1760,7 @@ static int static_status_read_and_clear(unsigned* out)
     BarrierWords h;
     if (cudaMemcpy(&h, s.barrier, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return NUNA_ERR_CUDA;
     *out = h.status;
-    return h.status != 0 ? rewind_barrier_words(s.barrier, h) : NUNA_OK;
+    return h.status != 0 ? rewind_barrier_words(c, s.barrier, h) : NUNA_OK;
 }
 
 }  // namespace nuna

@@ -52,12 +52,13 @@ struct Context {
     void* scratch = nullptr;             // two-shot shard intermediate, followed by its per-tile ready flags
     unsigned* flags = nullptr;           // one word per smallest tile of the scratch (inside the same allocation)
     size_t scratch_bytes = 0;
-    void* slots = nullptr;               // slots of the tagged two-shot, device memory
+    void* slots = nullptr;               // slots of the tagged two-shot (inside this or a retired scratch allocation)
     size_t slots_shard = 0;              // bytes of the largest shard they hold
-    std::vector<void*> retired_scratch;  // outgrown scratch and slots: captured graphs may still name them
+    std::vector<void*> retired_scratch;  // outgrown scratch allocations: captured graphs may still name them
     void* staging = nullptr;             // device copies of host buffers (nuna_allreduce_host)
     size_t staging_bytes = 0;
     cudaStream_t stream = nullptr;       // private stream of the host-buffer entry point
+    cudaStream_t setup = nullptr;        // what sets control words, flags and work lists (set_now)
     Options opt;
     nuna_topology_t topology = {};       // last probe result (have_topology says whether it is valid)
     bool have_topology = false;
